@@ -314,8 +314,9 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     std::vector<Tile> cands;
     if (packed) cands.assign(std::begin(kPackedTiles), std::end(kPackedTiles));
     else cands.assign(std::begin(kTuneTiles), std::end(kTuneTiles));
-    for (const Tile &t : cands) {
-        if (t.packed && !packed_tile_ok(t, job.sc)) continue;
+    for (const Tile &cand : cands) {
+        if (cand.packed && !packed_tile_ok(cand, job.sc)) continue;
+        const Tile t = in_frame(cand, job.sc);
         const int bps = persistent_blocks_per_sm(t);
         if (bps <= 0) continue;
         float tmin = 1e30f;

@@ -15,8 +15,12 @@ struct Tile {
     int lanes;            // lanes per extension (4, 8, 16 or 32)
     int c;                // cells per lane per diagonal
     bool packed = false;  // 16-bit cells, two per register (xd_lockstep16.cuh)
+    bool absolute = false;  // packed: cells in the absolute frame (in_frame)
     int width() const { return lanes * c; }
-    bool same(const Tile &o) const { return lanes == o.lanes && c == o.c && packed == o.packed; }
+    bool same(const Tile &o) const
+    {
+        return lanes == o.lanes && c == o.c && packed == o.packed && absolute == o.absolute;
+    }
 };
 
 // Band tiles the library is built with, narrowest first.
@@ -46,6 +50,9 @@ bool packed_tile_ok(Tile t, const Scoring &sc);
 // The tile to run for this scoring: t itself if it holds it, else the
 // packed 16-slot tile of the same width, else a 32-bit tile of its width.
 Tile usable_tile(Tile t, const Scoring &sc);
+
+// The tile with the frame its cells need for this scoring (packed tiles).
+Tile in_frame(Tile t, const Scoring &sc);
 
 cudaError_t launch_wide(bool count, int grid, const Job *jp, Spill in, int32_t *scratch,
                         int64_t scratch_per_cta, cudaStream_t s);

@@ -7,7 +7,54 @@
 //   x + match <= 1536,
 // and, for lanes of 32 slots, packed32_ok(): also x + match <= 1022.
 //
-// Biased, normalised scores.  A live cell on anti-diagonal d holds
+// What bounds it: integer issue.  Byte permutes, logic, minima, maxima and
+// DPX instructions issue on the ALU pipe and multiply-adds on the FMA pipe,
+// two cycles each per warp, so the count of instructions per register and
+// their split over the two pipes decide the time.
+//
+// Relative frame (REL).  A live cell of anti-diagonal d is kept as its
+// height above the diagonal's X-drop threshold,
+//   v = KS * (H - (T_{d-1} - x)) >= 0        (KS = 16 or 32, see Key),
+// and a pruned one as a negative half, kDead = -2^14 or below.  In the
+// normalised score H + d*|gap| the threshold grows by step(d) = |gap| + the
+// rise of T on diagonal d, gap predecessors enter unchanged and diagonal
+// ones with s' = s + 2|gap| >= 0.  So, in the frame of d-2,
+//   r = max3(V + s', U_t + step(d-2), U_t+-1 + step(d-2)),
+// V the slot's value two diagonals ago and U diagonal d-1, and
+//   v = min_unsigned(r - step(d-2) - step(d-1), kDead)
+// moves r into the frame of d and prunes it in one DPX instruction: a live
+// result is >= 0 and stays, a result below the threshold wraps above kDead
+// as an unsigned half and becomes kDead.  No threshold, mask or rebase per
+// cell.  Per register: a LOP3, a three-way maximum, the add-minimum and half
+// a key maximum on the ALU pipe; the substitution, the step and the key on
+// the FMA pipe: 6.5 instructions, 3.5 of them ALU.  The absolute frame below
+// takes 8.5 and 4.5.  Measured on 304,178 pairs of 29x reads, first tier,
+// 2x32 tile, x = 50: 64.3 ms in the absolute frame, 50.2 ms in this one (x =
+// 100, 4x32: 122.8 and 94.8 ms; x = 15, 2x16: 35.3 and 31.3 ms).
+//   Ranges.  Every half formed from a live one is at most KS * (x + 2 match +
+// 2|gap|) + KS - 1 < 2^15 (relative_ok).  A pruned half sinks by at most one
+// step per diagonal; every lift_period pairs the pruned halves are lifted
+// back to kDead, before one can wrap.  s' and steps are at most 256 and 128
+// units, so a pruned half never reaches 0 by them either, and the plain
+// 32-bit adds never carry from the low half (it stays below 0xE000 when
+// pruned and below 2^15 when live).
+//   Substitution.  One XOR of the 2-bit base windows gives a flag per slot
+// (bit 2s+1).  A shift shared by two or three registers brings register
+// t's two flags to bits p and p+16, p = 1, 3 or 5; one LOP3 keeps them and
+// adds a constant c, and w * k + V adds the match bonus and, through c, the
+// mismatch score s'(mismatch) = k c / KS (subst_folds; other scorings take
+// one more add).
+//   Rectangle ends.  Cells with i > m or j > n are not masked; their match
+// flags are cleared instead.  Without matches no such cell exceeds T, and none
+// leads back inside, so scores, positions and the two-dead-diagonal end
+// are those of the cells inside.  They can only keep a finished extension
+// running, so every 16 pairs they are pruned explicitly.  Per-register
+// masks took 5 more instructions per register on a quarter of the
+// diagonals: 58.1 -> 52 ms of the first tier.
+//   Key.  v + (S-1-slot) per half, compared signed; then as below.
+//
+// Absolute frame (!REL; only lanes of 32 slots with x + 2 match + 2|gap| >=
+// 1023).  A live cell on anti-diagonal d holds
 //   r = H + x + d*|gap| - B + beta     (B: the rebase steps taken off,
 //                                       beta = match + |gap| + 1)
 // stored as 16*r in an unsigned half; a pruned cell holds 0.  The two gap
@@ -35,7 +82,7 @@
 // values, the lowest window slot: the first cell in order of increasing i
 // on the diagonal.
 //
-// Substitution.  The match bits of each 16 slots of a lane come from one
+// Substitution, absolute frame.  The match bits of each 16 slots of a lane come from one
 // XOR of two 2-bit base-window words (a lane of 32 slots keeps two words
 // per read, and byte permutes merge its two match words for each half of
 // its 16 registers).  For register t the two bits (slots t and t+C2) are
@@ -50,7 +97,7 @@
 // register t sits in register t+1 (t-1) at the same half; only the end
 // registers need a byte permute and one shuffle per diagonal.
 //
-// Ranges, in units of r, with kR = (0x8000 / KS - 8) - 3 match - 3|gap|
+// Ranges, absolute frame, in units of r, with kR = (0x8000 / KS - 8) - 3 match - 3|gap|
 // the rebase step (rebase_step16: at least 1656 for KS = 16 and 632 for
 // KS = 32 inside the ranges above, and at least match + 2|gap|, the most
 // one pair of diagonals can raise a threshold); the figures below are for
@@ -65,13 +112,12 @@
 // range stays non-negative) and every live value is at most
 // thr + x + match <= 3576 (16 times that < 2^16).
 //
-// Carry-free adds.  V + s2 (stored value plus packed substitution, s2 <=
+// Carry-free adds, absolute frame.  V + s2 (stored value plus packed substitution, s2 <=
 // 16*256), z + idx (z = 0x8000 - 16 thr per half) and r + (z + idx) are
 // plain 32-bit adds: by the ranges above no low half, read unsigned,
 // reaches 2^16, so nothing carries into the high half.
 //
-// Window edges.  Live values are > 0 and pruned ones 0, so a half is live
-// iff it is nonzero.  The edges are tested once per pair of diagonals,
+// Window edges (both frames).  The edges are tested once per pair of diagonals,
 // after the even one: no live cell of diagonals d+1, d+2 can leave the
 // window unless E's top slot (diagonal d) or O's top slot (d-1) is live,
 // or E's bottom slot is.  The window then shifts up one slot if E's two
@@ -167,6 +213,26 @@ __device__ __forceinline__ uint32_t tree_max2(const uint32_t (&k)[N])
     }
 }
 
+template <int N>
+__device__ __forceinline__ uint32_t tree_max2s(const uint32_t (&k)[N])
+{
+    if constexpr (N == 1) {
+        return k[0];
+    } else if constexpr (N == 2) {
+        return __vmaxs2(k[0], k[1]);
+    } else {
+        constexpr int M = (N + 2) / 3;
+        uint32_t r[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            if (3 * i + 2 < N) r[i] = __vimax3_s16x2(k[3 * i], k[3 * i + 1], k[3 * i + 2]);
+            else if (3 * i + 1 < N) r[i] = __vmaxs2(k[3 * i], k[3 * i + 1]);
+            else r[i] = k[3 * i];
+        }
+        return tree_max2s<M>(r);
+    }
+}
+
 // A slot is live iff its half is nonzero (pruned slots hold 0).
 __device__ __forceinline__ bool live_lo(uint32_t v) { return (v & 0xFFFFu) != 0; }
 __device__ __forceinline__ bool live_hi(uint32_t v) { return (v >> 16) != 0; }
@@ -236,6 +302,87 @@ __device__ __forceinline__ uint32_t dp16(uint32_t (&V)[C2], const uint32_t (&U)[
     return max(kk >> 16, kk & 0xFFFFu);
 }
 
+// ---- relative frame (see the header comment) ----
+
+constexpr uint32_t kDead2 = 0xC000C000u;  // a pruned slot, both halves
+
+// Match-bit positions.  A lane's shifted flag word puts register t's two
+// flags at bits pos and pos + 16.  Lanes of 32 slots (KS = 32) serve three
+// registers with one shift (positions 1, 3, 5), the others two (1, 3).
+template <int C2>
+__host__ __device__ constexpr int rel_group() { return C2 == 16 ? 3 : 2; }
+template <int C2>
+__host__ __device__ constexpr int rel_pos(int t) { return 1 + 2 * ((t % 8) % rel_group<C2>()); }
+
+// The flag bits of slots lo .. hi of a 16-slot flag word.
+__device__ __forceinline__ uint32_t flag_range(int32_t lo, int32_t hi)
+{
+    uint32_t below, upto;
+    asm("shl.b32 %0, 0xFFFFFFFF, %1;" : "=r"(below) : "r"(2 * min(max(lo, 0), 16)));
+    asm("shl.b32 %0, 0xFFFFFFFF, %1;" : "=r"(upto) : "r"(2 * min(max(hi + 1, 0), 16)));
+    return below & ~upto;
+}
+
+// Slots of register t outside lo .. hi, to the pruned value.
+template <int C2>
+__device__ __forceinline__ uint32_t keep_range(uint32_t v, int t, int32_t lo, int32_t hi)
+{
+    const uint32_t l = (t >= lo && t <= hi) ? 0x0000FFFFu : 0u;
+    const uint32_t h = (t + C2 >= lo && t + C2 <= hi) ? 0xFFFF0000u : 0u;
+    return (v & (l | h)) | (kDead2 & ~(l | h));
+}
+
+// Per-group constants of the substitution: k[q] multiplies a flag at bit
+// 1 + 2q into the match bonus, c[q] (both halves) the mismatch score when
+// the scoring allows it (else 0, and mi2 is added).
+struct RelSubst {
+    uint32_t k[3], c[3];
+    uint32_t mi2;
+};
+
+// One anti-diagonal for one lane in the relative frame.  V: diagonal d-2 (in
+// its own frame), overwritten with d; U: diagonal d-1 plus the threshold
+// step from d-2 to d-1, so both predecessors are in the frame of d-2.
+// nstep: minus the threshold step from d-2 to d, per half.
+template <int C2, bool ODD, bool ADD>
+__device__ __forceinline__ uint32_t dp16r(uint32_t (&V)[C2], const uint32_t (&U)[C2],
+                                          uint32_t edge, uint32_t eq7, uint32_t eqh,
+                                          const RelSubst &sb, uint32_t nstep, uint32_t one)
+{
+    constexpr int G = rel_group<C2>();
+    constexpr int NS = (8 + G - 1) / G;  // shifts per flag word of 8 registers
+    constexpr int NE = C2 == 16 ? 2 : 1;
+    uint32_t e[NE];  // slot t's flag at 2t+1, slot t+C2's at 2t+17
+    if constexpr (C2 == 2) e[0] = (eq7 & 0xFu) | (eq7 << 12);
+    else if constexpr (C2 == 4) e[0] = prmt(eq7, eq7, 0x2100);
+    else if constexpr (C2 == 8) e[0] = eq7;
+    else { e[0] = prmt(eq7, eqh, 0x5410); e[1] = prmt(eq7, eqh, 0x7632); }
+    uint32_t es[NE][NS];
+#pragma unroll
+    for (int h = 0; h < NE; ++h)
+#pragma unroll
+        for (int q = 0; q < NS; ++q) es[h][q] = e[h] >> (2 * G * q);
+    uint32_t key[C2];
+#pragma unroll
+    for (int t = 0; t < C2; ++t) {
+        uint32_t sh;
+        if (ODD) sh = (t + 1 < C2) ? U[t + 1] : prmt(U[0], edge, 0x5432);
+        else sh = (t > 0) ? U[t - 1] : prmt(edge, U[C2 - 1], 0x5432);
+        constexpr uint32_t kBit = 0x00010001u;
+        const int q = (t % 8) % G;
+        const uint32_t w = (es[t / 8][(t % 8) / G] & (kBit << rel_pos<C2>(t))) | sb.c[q];
+        uint32_t cand = fma_add(w, sb.k[q], V[t]);
+        if (ADD) cand = fma_add(cand, one, sb.mi2);
+        const uint32_t r = __vimax3_s16x2(cand, U[t], sh);
+        // r - threshold step: a live cell stays >= 0; below the threshold it
+        // wraps to an unsigned value above kDead, which the minimum replaces
+        const uint32_t v = __viaddmin_u16x2(r, nstep, kDead2);
+        V[t] = v;
+        key[t] = fma_add(v, one, idx2<C2>(t));
+    }
+    return tree_max2s<C2>(key);
+}
+
 }  // namespace p16
 
 __host__ __device__ inline bool packed16_ok(const Scoring &sc)
@@ -262,8 +409,41 @@ __host__ __device__ inline int32_t rebase_step16(const Scoring &sc)
     return (0x8000 / p16::key_scale<S>() - 8) - 3 * sc.match + 3 * sc.gap;
 }
 
-// one: 1 (see fma_add).
-template <int L, int C2, class Src>
+// The relative frame on lanes of S slots: every value a step forms from a
+// live one, at most x + 2 match + 2|gap| in units of KS, stays below 2^15.
+// Lanes of up to 16 slots hold every scoring of packed16_ok.
+template <int S>
+__host__ __device__ inline bool relative_ok(const Scoring &sc)
+{
+    return packed16_ok(sc) &&
+           (sc.x + 2 * sc.match - 2 * sc.gap + 1) * p16::key_scale<S>() <= 0x8000;
+}
+
+// Whether the mismatch score can ride on the flag word (RelSubst::c): c =
+// 2 mm / bonus at flag bit 1 (mm = mismatch + 2|gap|, bonus = match -
+// mismatch) must be whole, leave the flag bit free and fit its half.
+__host__ __device__ inline bool subst_folds(const Scoring &sc)
+{
+    const int32_t mm = sc.mismatch - 2 * sc.gap, bonus = sc.match - sc.mismatch;
+    const int32_t c = 2 * mm / bonus;
+    return c * bonus == 2 * mm && !(c & 2) && c < 0x800;
+}
+
+// Pairs of diagonals after which pruned slots must be lifted back to the
+// pruned value: one may sink by the threshold's growth, at most match +
+// |gap|, on every diagonal, and by two such steps at once, and has 2^14 of
+// room.
+template <int S>
+__host__ __device__ inline int32_t lift_period(const Scoring &sc)
+{
+    const int32_t step = (sc.match - sc.gap) * p16::key_scale<S>();
+    const int32_t p = ((1 << 14) / step - 2) / 2;
+    return p < 1 ? 1 : p;
+}
+
+// REL: the relative frame (the scoring passes relative_ok<2 * C2>); else the
+// absolute one.  one: 1 (see fma_add).
+template <int L, int C2, bool REL, class Src>
 __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, int64_t nw,
                                                 uint32_t one)
 {
@@ -276,7 +456,10 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
     constexpr uint32_t SMASK = (1u << SB) - 1u;
     // -KS * 0x10001: z = 0x80008000 - KS thr in both halves
     constexpr uint32_t ZMUL = 0u - (uint32_t)key_scale<S>() * 0x10001u;
-    static_assert(S <= 32 && 32 % L == 0 && L >= 2 && C2 % 4 == 0, "packed tile shape");
+    static_assert(S <= 32 && 32 % L == 0 && L >= 2 && C2 % 2 == 0, "packed tile shape");
+    static_assert(REL || C2 % 4 == 0, "packed tile shape, absolute frame");
+    constexpr uint32_t KS = (uint32_t)key_scale<S>();
+    constexpr uint32_t kPruned = REL ? kDead2 : 0u;  // a pruned slot, both halves
     const int lane = threadIdx.x & 31;
     const int glane = lane % L;
     const int gbase = lane - glane;
@@ -285,7 +468,13 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
     // per-lane constants: 0/1 factors that clear the shuffled-in edge
     // beyond the group, and the halves the window-edge test reads
     const uint32_t keep_up = top_lane ? 0u : 1u, keep_dn = bot_lane ? 0u : 1u;
-    const uint32_t tmask = top_lane ? 0xFFFF0000u : 0u, bmask = bot_lane ? 0x0000FFFFu : 0u;
+    const uint32_t edge_up = top_lane ? kPruned : 0u, edge_dn = bot_lane ? kPruned : 0u;
+    const uint32_t tmask = top_lane ? (REL ? 0x80000000u : 0xFFFF0000u) : 0u;
+    const uint32_t bmask = bot_lane ? (REL ? 0x00008000u : 0x0000FFFFu) : 0u;
+    // a slot is live iff its half is nonzero (absolute frame) or not
+    // negative (relative frame)
+    auto lo_live = [](uint32_t v) { return REL ? (v & 0x8000u) == 0u : live_lo(v); };
+    auto hi_live = [](uint32_t v) { return REL ? (int32_t)v >= 0 : live_hi(v); };
 
     // Per-group task state (uniform within a group).
     bool active = false, exhausted = false;
@@ -302,17 +491,24 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
     int32_t ng = 1;                     // |gap|
     uint32_t mi2 = 0;                   // packed 16 * (mismatch + 2|gap|)
     uint32_t k13 = 0, k15 = 0;          // 16 (match - mismatch) << 19, << 17
+    RelSubst rs = {{0, 0, 0}, {0, 0, 0}, 0};  // relative frame: substitution constants
+    uint32_t dA = 0, dB = 0;            // relative frame: threshold steps d-2 -> d-1, d-1 -> d
+    uint32_t ngp = 0;                   // |gap| * KS in both halves
+    int32_t lift = 1 << 20;             // relative frame: lift_period of the group's scoring
+    int32_t lift_n = 1 << 20;           // warp-uniform: pairs until the next lift
+    bool add_mi = false;                // the group's scoring needs rs.mi2 added
+    bool generic = false;               // warp-uniform: some group's does
     bool prev_dead = false, fin = false, rb = false;
     uint32_t E[C2], O[C2];
 #pragma unroll
-    for (int t = 0; t < C2; ++t) { E[t] = 0u; O[t] = 0u; }
+    for (int t = 0; t < C2; ++t) { E[t] = kPruned; O[t] = kPruned; }
     // base windows (slots 0-15; Aw1, Bw1: slots 16-31 of 32-slot lanes) and
     // the lookahead words
     uint32_t Aw = 0, Aw1 = 0, LA = 0, Bw = 0, Bw1 = 0, LB = 0;
     int la_n = 16;        // warp-uniform: diagonal pairs the lookahead words still cover
     int32_t budget = 0;   // warp-uniform: diagonal pairs known to stay inside every rectangle
     // (31 - lane) * 16, less the key offset's share of the group key
-    const int32_t lane_bits = ((31 - glane) << SB) - (0x8000 << 5);
+    const int32_t lane_bits = ((31 - glane) << SB) - (REL ? 0 : (0x8000 << 5));
 
     auto retire = [&](bool overflow) {
         if (bd > 0) {
@@ -322,6 +518,8 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
         if (glane == 0) src.retire(gj, task, overflow, T, bi, bj);
         active = false;
         ng = 0;  // the frame offset stays put while the group waits
+        add_mi = false;
+        lift = 1 << 20;
     };
 
     // Diagonal pairs until a cell of this group's window can leave the
@@ -348,11 +546,11 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
     // One anti-diagonal and the bookkeeping that cannot wait for the end of
     // the pair: T and the best cell.  Returns the group key (negative iff
     // every cell of the diagonal was pruned) and the diagonal's threshold.
-    auto diag = [&](auto odd_tag, auto masked_tag, int32_t &thr) -> int32_t {
+    auto diag = [&](auto odd_tag, auto masked_tag, auto add_tag, int32_t &thr) -> int32_t {
         constexpr bool ODD = decltype(odd_tag)::value;
         constexpr bool MASKED = decltype(masked_tag)::value;
+        constexpr bool ADD = decltype(add_tag)::value;
         ++d;
-        Q += ng;
         if (ODD) {
             ++i0;
             if constexpr (WIDE) {
@@ -368,41 +566,76 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
             Bw = __funnelshift_l(LB, Bw, 2);
             LB <<= 2;
         }
-        thr = T + Q;
-        // 0x8000 - 16 thr in both halves (no borrow: 16 thr <= 0x8000)
-        const uint32_t z = (uint32_t)thr * ZMUL + kKey2;
         // rectangle bounds of this lane's slots, clamped into 16 bits (only
         // the masked copy reads them)
         uint32_t lo1_2 = 0, nhi1_2 = 0;
-        if (MASKED) {
+        if (MASKED && !REL) {
             const int32_t lo = j0 - n, hi = m - i0;
             lo1_2 = pack2(min(max(lo - 1, -1024), 1024));
             nhi1_2 = pack2(min(max(-hi - 1, -1024), 1024));
         }
         const uint32_t xx = Aw ^ Bw;
-        const uint32_t eq7 = ~(xx | (xx << 1));
+        uint32_t eq7 = ~(xx | (xx << 1));
         uint32_t eqh = 0u;
         if constexpr (WIDE) {
             const uint32_t xh = Aw1 ^ Bw1;
             eqh = ~(xh | (xh << 1));
         }
-        uint32_t lk;
-        if (ODD) {
-            const uint32_t edge = fma_add(__shfl_down_sync(FULL, E[0], 1, L), keep_up, 0u);
-            lk = dp16<C2, true, MASKED>(O, E, edge, eq7, eqh, mi2, k13, k15, z, lo1_2, nhi1_2,
-                                        one);
+        if (MASKED && REL) {  // no match outside the rectangle (header comment)
+            const int32_t lo = j0 - n, hi = m - i0;
+            eq7 &= flag_range(lo, hi);
+            if constexpr (WIDE) eqh &= flag_range(lo - 16, hi - 16);
+        }
+        int32_t lk;
+        if constexpr (REL) {
+            // diagonal d-1 in the frame of d-2; both halves of dA and dB are equal
+            const uint32_t nstep = 0x00010000u - (dA + dB);
+            uint32_t U[C2];
+#pragma unroll
+            for (int t = 0; t < C2; ++t) U[t] = fma_add(ODD ? E[t] : O[t], one, dA);
+            uint32_t kk;
+            if (ODD) {
+                const uint32_t edge = fma_add(__shfl_down_sync(FULL, U[0], 1, L), keep_up, edge_up);
+                kk = dp16r<C2, true, ADD>(O, U, edge, eq7, eqh, rs, nstep, one);
+            } else {
+                const uint32_t edge =
+                    fma_add(__shfl_up_sync(FULL, U[C2 - 1], 1, L), keep_dn, edge_dn);
+                kk = dp16r<C2, false, ADD>(E, U, edge, eq7, eqh, rs, nstep, one);
+            }
+            lk = max((int32_t)kk >> 16, (int32_t)(kk << 16) >> 16);
         } else {
-            const uint32_t edge = fma_add(__shfl_up_sync(FULL, O[C2 - 1], 1, L), keep_dn, 0u);
-            lk = dp16<C2, false, MASKED>(E, O, edge, eq7, eqh, mi2, k13, k15, z, lo1_2, nhi1_2,
-                                         one);
+            Q += ng;
+            thr = T + Q;
+            // 0x8000 - 16 thr in both halves (no borrow: 16 thr <= 0x8000)
+            const uint32_t z = (uint32_t)thr * ZMUL + kKey2;
+            if (ODD) {
+                const uint32_t edge = fma_add(__shfl_down_sync(FULL, E[0], 1, L), keep_up, edge_up);
+                lk = (int32_t)dp16<C2, true, MASKED>(O, E, edge, eq7, eqh, mi2, k13, k15, z, lo1_2,
+                                                     nhi1_2, one);
+            } else {
+                const uint32_t edge =
+                    fma_add(__shfl_up_sync(FULL, O[C2 - 1], 1, L), keep_dn, edge_dn);
+                lk = (int32_t)dp16<C2, false, MASKED>(E, O, edge, eq7, eqh, mi2, k13, k15, z, lo1_2,
+                                                      nhi1_2, one);
+            }
         }
         // Group key: value above lane above slot in lane, so one max finds
         // the lowest window slot among the cells holding the maximum.  With
-        // lk = 0x8000 + 2^SB v + i: 32 lk - 31 i = 0x8000 * 32 + 2^VS v + i
-        // (multiply-adds).
-        const int32_t mkey = lockstep_group_max<L>(
-            (int32_t)fma_add(lk, one << 5, fma_add(lk & SMASK, 0u - 31u, (uint32_t)lane_bits)));
-        if (mkey >= xup) {  // best value - thr > x: T rises (decoded at retire)
+        // lk = 2^SB v + i (plus 0x8000 in the absolute frame): 32 lk - 31 i =
+        // 2^VS v + i (plus 0x8000 * 32) (multiply-adds).
+        const int32_t mkey = lockstep_group_max<L>((int32_t)fma_add(
+            (uint32_t)lk, one << 5, fma_add((uint32_t)lk & SMASK, 0u - 31u, (uint32_t)lane_bits)));
+        if constexpr (REL) {
+            const int32_t rise = max((mkey >> VS) - sc.x, 0);  // best value above T
+            dA = dB;
+            dB = (uint32_t)rise * (KS * 0x10001u) + ngp;
+            T += rise;
+            if (rise > 0) {  // decoded at retire
+                bkey = mkey;
+                bi0 = i0;
+                bd = d;
+            }
+        } else if (mkey >= xup) {  // best value - thr > x: T rises (decoded at retire)
             T += (mkey >> VS) - sc.x;
             bkey = mkey;
             bi0 = i0;
@@ -415,20 +648,21 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
     // "something to do" vote: a window edge went live, a task ended, the
     // lookahead words ran out, a frame needs a rebase, the masking-free
     // budget ran out, or a group waits for a task.
-    auto pair = [&](auto masked_tag) -> bool {
+    auto pair = [&](auto masked_tag, auto add_tag) -> bool {
         constexpr bool MASKED = decltype(masked_tag)::value;
-        int32_t thr_o, thr_e;
-        const int32_t key_o = diag(std::true_type{}, masked_tag, thr_o);
-        const int32_t key_e = diag(std::false_type{}, masked_tag, thr_e);
+        int32_t thr_o = 0, thr_e = 0;
+        const int32_t key_o = diag(std::true_type{}, masked_tag, add_tag, thr_o);
+        const int32_t key_e = diag(std::false_type{}, masked_tag, add_tag, thr_e);
         const bool dead_o = key_o < 0, dead_e = key_e < 0;
         fin = active && ((dead_o && (prev_dead || dead_e)) || d >= mn);
         prev_dead = dead_e;
         --budget;
         --la_n;
-        rb = active && thr_o >= kRL;
+        if constexpr (!REL) rb = active && thr_o >= kRL;
         // window edges: this group's bottom lane tests E's bottom slot, its
-        // top lane the top slots of E and O (a nonzero half is live)
-        const uint32_t ew = ((E[C2 - 1] | O[C2 - 1]) & tmask) | (E[0] & bmask);
+        // top lane the top slots of E and O
+        const uint32_t ew = REL ? (~(E[C2 - 1] & O[C2 - 1]) & tmask) | (~E[0] & bmask)
+                                : ((E[C2 - 1] | O[C2 - 1]) & tmask) | (E[0] & bmask);
         const bool edge = active && ew != 0u;
         bool ev = edge || fin || rb || la_n == 0 || (!active && !exhausted);
         if (!MASKED) ev = ev || budget < 1;
@@ -442,13 +676,13 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
     auto handle = [&](const bool masked) -> bool {
         bool ovf = false;
         const bool go = active && !fin;
-        const bool need_dn_l = bot_lane && live_lo(E[0]);
-        const bool need_up_l = top_lane && (live_hi(E[C2 - 1]) || live_hi(O[C2 - 1]));
+        const bool need_dn_l = bot_lane && lo_live(E[0]);
+        const bool need_up_l = top_lane && (hi_live(E[C2 - 1]) || hi_live(O[C2 - 1]));
         if (__any_sync(FULL, go && (need_dn_l || need_up_l))) {
             // Per group: the decision of its bottom and top lanes.
-            const bool blk_up_l = live_lo(E[0]) || live_lo(E[1]) || live_lo(O[0]);
-            const bool blk_dn_l = live_hi(E[C2 - 1]) || live_hi(O[C2 - 1]) ||
-                                  live_hi(E[C2 - 2]) || live_hi(O[C2 - 2]);
+            const bool blk_up_l = lo_live(E[0]) || lo_live(E[1]) || lo_live(O[0]);
+            const bool blk_dn_l = hi_live(E[C2 - 1]) || hi_live(O[C2 - 1]) ||
+                                  hi_live(E[C2 - 2]) || hi_live(O[C2 - 2]);
             // every lane takes part in every shuffle (no short-circuit
             // around a warp-wide collective)
             const bool up_g = __shfl_sync(FULL, (int)need_up_l, L - 1, L) != 0;
@@ -463,7 +697,7 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
             if (__any_sync(FULL, su)) {
                 uint32_t ne = __shfl_down_sync(FULL, E[0], 1, L);
                 uint32_t no = __shfl_down_sync(FULL, O[0], 1, L);
-                if (top_lane) { ne = 0u; no = 0u; }
+                if (top_lane) { ne = kPruned; no = kPruned; }
                 if (su) {
                     const uint32_t te = prmt(E[0], ne, 0x5432), to = prmt(O[0], no, 0x5432);
 #pragma unroll
@@ -477,7 +711,7 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
             if (__any_sync(FULL, sd)) {
                 uint32_t pe = __shfl_up_sync(FULL, E[C2 - 1], 1, L);
                 uint32_t po = __shfl_up_sync(FULL, O[C2 - 1], 1, L);
-                if (bot_lane) { pe = 0u; po = 0u; }
+                if (bot_lane) { pe = kPruned; po = kPruned; }
                 if (sd) {
                     const uint32_t te = prmt(pe, E[C2 - 1], 0x5432);
                     const uint32_t to = prmt(po, O[C2 - 1], 0x5432);
@@ -501,10 +735,33 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
             LB = back16_u(pk, nw, sb0, dir, j0 + 16);
             la_n = 16;
         }
-        // Every live value of the pair is >= 16 thr of its odd diagonal:
+        if constexpr (REL) {
+            if (refill && masked) {  // end what lives outside the rectangle
+                const int32_t lo = j0 - n, hi = m - i0;
+#pragma unroll
+                for (int t = 0; t < C2; ++t) {
+                    E[t] = keep_range<C2>(E[t], t, lo, hi);
+                    O[t] = keep_range<C2>(O[t], t, lo - 1, hi);  // one diagonal earlier
+                }
+            }
+            // lift the pruned slots back up (lift_period)
+            if (refill) {
+                lift_n -= 16;
+                if (lift_n < 16) {
+#pragma unroll
+                    for (int t = 0; t < C2; ++t) {
+                        E[t] = __vmaxs2(E[t], kDead2);
+                        O[t] = __vmaxs2(O[t], kDead2);
+                    }
+                    lift_n = __reduce_min_sync(FULL, lift);
+                    la_n = min(16, lift_n);
+                }
+            }
+        }
+        // Absolute frame: every live value of the pair is >= 16 thr of its odd diagonal:
         // once that threshold reaches kR + match + 1, take kR off the frame
         // (pruned halves stay 0; no half borrows).
-        if (active && rb) {
+        if (!REL && active && rb) {
             const uint32_t mr = pack2(kScale * kR);
 #pragma unroll
             for (int t = 0; t < C2; ++t) {
@@ -547,7 +804,7 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
                     exhausted = true;
                 } else if (r > 0) {
                     const Ext e = src.open(gj, task, sc);
-                    if (e.ok && !(WIDE ? packed32_ok(sc) : packed16_ok(sc))) {
+                    if (e.ok && !(REL ? relative_ok<S>(sc) : packed32_ok(sc))) {
                         // A scoring 16-bit cells cannot hold exactly (a serving
                         // request's own): hand the task to the next, 32-bit tier.
                         if (glane == 0) src.retire(gj, task, true, 0, 0, 0);
@@ -559,30 +816,48 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
                         n = e.n;
                         mn = m + n;
                         ng = -sc.gap;
-                        kR = rebase_step16<S>(sc);
-                        kRL = kR + sc.match + 1;
-                        xup = (sc.x + 1) << VS;
-                        mi2 = pack2(kScale * (sc.mismatch + 2 * ng));
-                        k13 = (uint32_t)(kScale * (sc.match - sc.mismatch)) << 19;
-                        k15 = (uint32_t)(kScale * (sc.match - sc.mismatch)) << 17;
-                        // origin (H = 0) at window slot W/2, stored as
-                        // 16 * (x + beta), beta = match + |gap| + 1
-                        const int32_t beta = sc.match + ng + 1;
-                        const uint32_t orig = (uint32_t)(kScale * (sc.x + beta));
+                        uint32_t orig;
+                        if constexpr (REL) {
+                            // origin (H = 0) at window slot W/2, x above the threshold
+                            orig = (uint32_t)sc.x * KS;
+                            const int32_t mm = sc.mismatch + 2 * ng, bonus = sc.match - sc.mismatch;
+                            const bool folds = subst_folds(sc);
+                            add_mi = !folds;
+                            rs.mi2 = folds ? 0u : pack2(mm * (int32_t)KS);
+                            const uint32_t c = folds ? (uint32_t)(2 * mm / bonus) * 0x10001u : 0u;
+#pragma unroll
+                            for (int q = 0; q < 3; ++q) {
+                                rs.k[q] = (uint32_t)bonus * KS >> (1 + 2 * q);
+                                rs.c[q] = c << (2 * q);
+                            }
+                            ngp = (uint32_t)ng * (KS * 0x10001u);
+                            dA = dB = ngp;
+                            lift = lift_period<S>(sc);
+                        } else {
+                            kR = rebase_step16<S>(sc);
+                            kRL = kR + sc.match + 1;
+                            xup = (sc.x + 1) << VS;
+                            mi2 = pack2(kScale * (sc.mismatch + 2 * ng));
+                            k13 = (uint32_t)(kScale * (sc.match - sc.mismatch)) << 19;
+                            k15 = (uint32_t)(kScale * (sc.match - sc.mismatch)) << 17;
+                            // origin (H = 0) at window slot W/2, stored as
+                            // 16 * (x + beta), beta = match + |gap| + 1
+                            Q = sc.match + ng + 1;
+                            orig = (uint32_t)(kScale * (sc.x + Q));
+                        }
 #pragma unroll
                         for (int t = 0; t < C2; ++t) {
                             const int slo = glane * S + t, shi = slo + C2;
-                            const uint32_t lo = (slo == W / 2) ? orig : 0u;
-                            const uint32_t hi = (shi == W / 2) ? orig : 0u;
+                            const uint32_t lo = (slo == W / 2) ? orig : (kPruned & 0xFFFFu);
+                            const uint32_t hi = (shi == W / 2) ? orig : (kPruned >> 16);
                             E[t] = lo | (hi << 16);
-                            O[t] = 0u;
+                            O[t] = kPruned;
                         }
                         i0 = -(W / 2) + glane * S;
                         j0 = (W / 2) - glane * S;
                         load_windows();
                         d = 0;
                         T = 0;
-                        Q = beta;
                         bi = 0;
                         bj = 0;
                         bd = 0;
@@ -598,13 +873,24 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
             continue;
         }
         refresh_budget();
+        if constexpr (REL) {
+            generic = __any_sync(FULL, add_mi);
+            lift_n = min(lift_n, __reduce_min_sync(FULL, lift));
+            la_n = min(la_n, lift_n);
+        }
         if (budget >= 1) {
-            for (;;) {  // no cell of any window can leave its rectangle
-                if (pair(T0{}) && handle(false)) break;
+            if (REL && generic) {
+                for (;;) {
+                    if (pair(T0{}, T1{}) && handle(false)) break;
+                }
+            } else {
+                for (;;) {  // no cell of any window can leave its rectangle
+                    if (pair(T0{}, T0{}) && handle(false)) break;
+                }
             }
         } else {
             for (;;) {
-                if (pair(T1{}) && handle(true)) break;
+                if (pair(T1{}, T1{}) && handle(true)) break;
             }
         }
     }
@@ -615,13 +901,13 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
 // lane (five such blocks fit an SM, 20 warps) and 128 with 32 (four blocks),
 // and that measured faster than capping the registers for more warps.
 constexpr int kPackedThreads = 128;
-template <int L, int C2>
+template <int L, int C2, bool REL = true>
 __global__ void __launch_bounds__(kPackedThreads)
 lockstep16_kernel(const Job *jp, const uint32_t *order, const uint32_t *n_tasks_ptr,
                   uint32_t *counter, Spill spill, uint32_t one)
 {
     BatchSrc src{jp, order, *n_tasks_ptr, counter, spill};
-    lockstep16_loop<L, C2>(src, jp->packed, jp->n_words, one);
+    lockstep16_loop<L, C2, REL>(src, jp->packed, jp->n_words, one);
 }
 
 }  // namespace xd

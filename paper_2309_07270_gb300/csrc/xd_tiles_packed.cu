@@ -7,20 +7,21 @@
 
 namespace xd {
 
-template <int L, int C2>
+template <int L, int C2, bool REL = true>
 static cudaError_t packed_impl(int grid, const Job *jp, const uint32_t *order, const uint32_t *n,
                                uint32_t *ctr, Spill sp, cudaStream_t s)
 {
     (void)cudaGetLastError();
-    lockstep16_kernel<L, C2><<<grid, kPackedThreads, 0, s>>>(jp, order, n, ctr, sp, 1u);
+    lockstep16_kernel<L, C2, REL><<<grid, kPackedThreads, 0, s>>>(jp, order, n, ctr, sp, 1u);
     return cudaGetLastError();
 }
 
-template <int L, int C2>
+template <int L, int C2, bool REL = true>
 static int packed_occupancy_impl()
 {
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lockstep16_kernel<L, C2>, kPackedThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lockstep16_kernel<L, C2, REL>, kPackedThreads,
+                                                  0);
     return b;
 }
 
@@ -30,6 +31,10 @@ cudaError_t launch_persistent_packed(Tile t, int grid, const Job *jp, const uint
 {
     *handled = true;
     if (t.packed) {
+        if (t.absolute && t.c == 32) {
+            if (t.lanes == 2) return packed_impl<2, 16, false>(grid, jp, order, n, ctr, sp, s);
+            if (t.lanes == 4) return packed_impl<4, 16, false>(grid, jp, order, n, ctr, sp, s);
+        }
         if (t.lanes == 4 && t.c == 8) return packed_impl<4, 4>(grid, jp, order, n, ctr, sp, s);
         if (t.lanes == 2 && t.c == 16) return packed_impl<2, 8>(grid, jp, order, n, ctr, sp, s);
         if (t.lanes == 4 && t.c == 16) return packed_impl<4, 8>(grid, jp, order, n, ctr, sp, s);
@@ -46,6 +51,10 @@ cudaError_t launch_persistent_packed(Tile t, int grid, const Job *jp, const uint
 int occupancy_packed(Tile t)
 {
     if (!t.packed) return -1;
+    if (t.absolute && t.c == 32) {
+        if (t.lanes == 2) return packed_occupancy_impl<2, 16, false>();
+        if (t.lanes == 4) return packed_occupancy_impl<4, 16, false>();
+    }
     if (t.lanes == 4 && t.c == 8) return packed_occupancy_impl<4, 4>();
     if (t.lanes == 2 && t.c == 16) return packed_occupancy_impl<2, 8>();
     if (t.lanes == 4 && t.c == 16) return packed_occupancy_impl<4, 8>();
@@ -64,9 +73,17 @@ bool packed_tile_ok(Tile t, const Scoring &sc)
     return t.packed && (t.c == 32 ? packed32_ok(sc) : packed16_ok(sc));
 }
 
+// Lanes of 32 slots hold x + match <= 1022 (packed32_ok) in the absolute
+// frame; the relative one needs x + 2 match + 2|gap| < 1024 there.
+Tile in_frame(Tile t, const Scoring &sc)
+{
+    t.absolute = t.packed && t.c == 32 && !relative_ok<32>(sc);
+    return t;
+}
+
 Tile usable_tile(Tile t, const Scoring &sc)
 {
-    if (!t.packed || packed_tile_ok(t, sc)) return t;
+    if (!t.packed || packed_tile_ok(t, sc)) return in_frame(t, sc);
     if (t.c == 32) {  // the 16-slot tile of the same width, or its 32-bit twin
         const Tile h{2 * t.lanes, 16, true};
         return packed16_ok(sc) ? h : Tile{h.lanes, 16, false};
