@@ -246,7 +246,8 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st);
 /* Packed tiles: 16-bit cells, two per 32-bit register, for scorings with
  * match - gap <= 128, mismatch >= -128, mismatch - 2*gap >= 0 and
  * x + match <= 1536, and x + match <= 1022 for the tiles of 32 cells per
- * lane (results identical to the 32-bit tiles; other scorings run the
+ * lane (x + 2 match + 2|gap| <= 1023 for 1x32, <= 511 with match + |gap| <= 64
+ * for 2x64; results identical to the 32-bit tiles; other scorings run the
  * packed 16-cell tile of the same width, else the 32-bit tile of that
  * shape).  Set in `cells` of xdrop_set_tile. */
 #define XDROP_TILE_PACKED16 0x100
@@ -260,10 +261,11 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st);
  * submit).  The first submit with a new key times the first-tier tiles on
  * a stratified random sample of its pairs (one pair of every 3 with the
  * packed tiles when the scoring fits them, else one of every 8 with the
- * 32-bit tiles) and keeps the fastest for that key.  Tiles: 4x16, 8x8, 16x4,
+ * 32-bit tiles; widths far from x / |gap| are left out) and keeps the
+ * fastest for that key.  Tiles: 4x16, 8x8, 16x4,
  * 8x16, 16x8, 32x4, and packed (cells | XDROP_TILE_PACKED16) 4x8, 2x16,
- * 4x16, 8x8, 2x32, 8x16, 16x8, 4x32.  Returns XDROP_EINVAL for another
- * shape.  Serving mode (set the tile before the first xdrop_submit_pairs)
+ * 4x16, 8x8, 2x32, 8x16, 16x8, 4x32, 1x32, 2x64.  Returns XDROP_EINVAL for
+ * another shape.  Serving mode (set the tile before the first xdrop_submit_pairs)
  * runs packed 4x16 by default (a packed tile of 32 cells per lane serves as
  * the 16-cell tile of its width); with a packed first tier, requests whose
  * scoring does not fit 16 bits run on the serving kernel's 32-bit second

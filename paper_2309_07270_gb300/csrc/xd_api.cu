@@ -268,7 +268,8 @@ int enqueue_batched(xdrop_ctx *c, Tile t0, int bps, bool main_events, uint32_t *
 // the packed 16-bit ones only for scorings they hold exactly.
 const Tile kTuneTiles[] = {{4, 16}, {8, 8}, {16, 4}, {8, 16}, {16, 8}, {32, 4}};
 const Tile kPackedTiles[] = {{4, 8, true},  {2, 16, true}, {4, 16, true}, {8, 8, true},
-                             {2, 32, true}, {8, 16, true}, {16, 8, true}, {4, 32, true}};
+                             {2, 32, true}, {8, 16, true}, {16, 8, true}, {4, 32, true},
+                             {1, 32, true}, {2, 64, true}};
 
 // The first tile for a submit: the forced one (unpacked when the scoring
 // does not fit 16 bits) or the tuned one for this scoring.
@@ -309,6 +310,13 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
+    // Widths worth timing: a gap step costs |gap| and moves half a slot, so
+    // a live band spans at most about x / |gap| slots.  A window under 3/4 of
+    // that overflows too often to win, one over 3 times it computes mostly
+    // dead slots.
+    const int64_t span = job.sc.x / -(int64_t)job.sc.gap;
+    const int64_t min_w = std::min<int64_t>(128, span * 3 / 4);
+    const int64_t max_w = std::max<int64_t>(64, span * 3);
     float best_ms = 1e30f;
     *best = Tile{0, 0};
     std::vector<Tile> cands;
@@ -317,10 +325,12 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     for (const Tile &cand : cands) {
         if (cand.packed && !packed_tile_ok(cand, job.sc)) continue;
         const Tile t = in_frame(cand, job.sc);
+        if (t.width() < min_w || t.width() > max_w) continue;
         const int bps = persistent_blocks_per_sm(t);
         if (bps <= 0) continue;
         float tmin = 1e30f;
         for (int rep = 0; rep < 2; ++rep) {
+            if (rep && tmin > 1.25f * best_ms) break;  // far behind after one run
             CK(cudaEventRecord(e0, s));
             int rc = enqueue_batched(c, t, bps, false, nullptr);
             if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }

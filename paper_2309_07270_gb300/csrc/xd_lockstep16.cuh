@@ -5,16 +5,23 @@
 // It is exact whenever the scoring passes packed16_ok():
 //   match - gap <= 128, mismatch >= -128, mismatch + 2|gap| >= 0,
 //   x + match <= 1536,
-// and, for lanes of 32 slots, packed32_ok(): also x + match <= 1022.
+// and, for lanes of 32 and 64 slots, relative_ok().
 //
 // What bounds it: integer issue.  Byte permutes, logic, minima, maxima and
 // DPX instructions issue on the ALU pipe and multiply-adds on the FMA pipe,
 // two cycles each per warp, so the count of instructions per register and
-// their split over the two pipes decide the time.
+// their split over the two pipes decide the time, and the bookkeeping of a
+// diagonal (base windows, lane and group maximum, T, events), which is per
+// lane: lanes of more slots spread it over more cells (29x, first tier: x = 50
+// 4x16 51.6 ms, 2x32 45.0, 1x64 50.6; x = 100 4x32 88.6, 2x64 84.9; x = 15 2x16
+// 25.7, 1x32 23.0).  Rare events cost as a group's event stops the whole warp:
+// shifts by an eighth of the window instead of one slot, on registers moved
+// directly and with bases loaded once for both directions, took 1x64 from
+// 90 to 50 ms and 2x32 from 50.2 to 46.0.
 //
-// Relative frame (REL).  A live cell of anti-diagonal d is kept as its
-// height above the diagonal's X-drop threshold,
-//   v = KS * (H - (T_{d-1} - x)) >= 0        (KS = 16 or 32, see Key),
+// Relative frame.  A live cell of anti-diagonal d is kept as its height
+// above the diagonal's X-drop threshold,
+//   v = KS * (H - (T_{d-1} - x)) >= 0        (KS = 16, 32 or 64, see Key),
 // and a pruned one as a negative half, kDead = -2^14 or below.  In the
 // normalised score H + d*|gap| the threshold grows by step(d) = |gap| + the
 // rise of T on diagonal d, gap predecessors enter unchanged and diagonal
@@ -27,16 +34,16 @@
 // as an unsigned half and becomes kDead.  No threshold, mask or rebase per
 // cell.  Per register: a LOP3, a three-way maximum, the add-minimum and half
 // a key maximum on the ALU pipe; the substitution, the step and the key on
-// the FMA pipe: 6.5 instructions, 3.5 of them ALU.  The absolute frame below
-// takes 8.5 and 4.5.  Measured on 304,178 pairs of 29x reads, first tier,
-// 2x32 tile, x = 50: 64.3 ms in the absolute frame, 50.2 ms in this one (x =
-// 100, 4x32: 122.8 and 94.8 ms; x = 15, 2x16: 35.3 and 31.3 ms).
+// the FMA pipe: 6.5 instructions, 3.5 of them ALU (the absolute frame of
+// xd_lockstep16_abs.cuh takes 8.5 and 4.5).  Measured on 304,178 pairs of 29x
+// reads, first tier: x = 50 (2x32) 64.3 ms in the absolute frame, 50.2 ms in
+// this one; x = 100 (4x32) 122.8 and 94.8 ms; x = 15 (2x16) 35.3 and 31.3 ms.
 //   Ranges.  Every half formed from a live one is at most KS * (x + 2 match +
 // 2|gap|) + KS - 1 < 2^15 (relative_ok).  A pruned half sinks by at most one
 // step per diagonal; every lift_period pairs the pruned halves are lifted
-// back to kDead, before one can wrap.  s' and steps are at most 256 and 128
-// units, so a pruned half never reaches 0 by them either, and the plain
-// 32-bit adds never carry from the low half (it stays below 0xE000 when
+// back to kDead, before one can wrap.  s' and steps add less than 2^14 to a
+// half, so a pruned half never reaches 0 by them either, and the plain
+// 32-bit adds never carry from the low half (it stays below 2^16 when
 // pruned and below 2^15 when live).
 //   Substitution.  One XOR of the 2-bit base windows gives a flag per slot
 // (bit 2s+1).  A shift shared by two or three registers brings register
@@ -44,174 +51,52 @@
 // adds a constant c, and w * k + V adds the match bonus and, through c, the
 // mismatch score s'(mismatch) = k c / KS (subst_folds; other scorings take
 // one more add).
+//   Chain.  The keys are taken from r, before the prune, so the maximum of a
+// diagonal does not wait for the maximum of the one before it.
 //   Rectangle ends.  Cells with i > m or j > n are not masked; their match
 // flags are cleared instead.  Without matches no such cell exceeds T, and none
 // leads back inside, so scores, positions and the two-dead-diagonal end
 // are those of the cells inside.  They can only keep a finished extension
-// running, so every 16 pairs they are pruned explicitly.  Per-register
-// masks took 5 more instructions per register on a quarter of the
-// diagonals: 58.1 -> 52 ms of the first tier.
-//   Key.  v + (S-1-slot) per half, compared signed; then as below.
-//
-// Absolute frame (!REL; only lanes of 32 slots with x + 2 match + 2|gap| >=
-// 1023).  A live cell on anti-diagonal d holds
-//   r = H + x + d*|gap| - B + beta     (B: the rebase steps taken off,
-//                                       beta = match + |gap| + 1)
-// stored as 16*r in an unsigned half; a pruned cell holds 0.  The two gap
-// predecessors enter unchanged and the diagonal one with s + 2|gap| >= 0:
-//   r(d) = max(r_diag(d-2) + s + 2|gap|,  r_up(d-1),  r_left(d-1)),
-// one 32-bit add (both halves at once, see below) and one u16x2 three-way
-// max per register (two cells).  The X-drop threshold of diagonal d (T of
-// d-1 minus x) becomes thr = T + d*|gap| - B + beta, a cell is live iff
-// r >= thr, and r - thr <= x + match.  Every threshold is at least
-// match + 2|gap| + 1, so a pruned predecessor (0, or 16*(s + 2|gap|) after
-// the diagonal add) can never lift a cell to its threshold: a cell with no
-// live predecessor stays pruned, and one with a live predecessor takes the
-// same maximum as the recurrence over live predecessors.
-//
-// Key.  One more 32-bit multiply-add gives each slot's key
-//   0x8000 + KS*(r - thr) + (S-1-slot),
-// with KS = 16 key units per unit of r for lanes of up to 16 slots (a
-// 4-bit slot index; the add takes the stored 16 r as it is) and KS = 32
-// for lanes of 32 (a 5-bit index; the multiply-add doubles 16 r).  Bit 15
-// is set exactly for the live cells (a byte permute spreads that bit into
-// the mask that zeroes the pruned ones) and, for live cells, the key
-// orders by value and then by lowest slot.  The lane's best key becomes
-// value * 2^(SB+5) + (31 - lane) * 2^SB + slot bits in 32 bits (SB = 4 or
-// 5 slot bits), so one group max gives the largest value and, among equal
-// values, the lowest window slot: the first cell in order of increasing i
-// on the diagonal.
-//
-// Substitution, absolute frame.  The match bits of each 16 slots of a lane come from one
-// XOR of two 2-bit base-window words (a lane of 32 slots keeps two words
-// per read, and byte permutes merge its two match words for each half of
-// its 16 registers).  For register t the two bits (slots t and t+C2) are
-// moved to bits p and p+16, p = 13 or 15, by a left shift (a multiply on
-// the FMA pipe) and masked; a high multiply by 16 (match - mismatch) *
-// 2^(32-p) turns them into the per-half match bonus, and its addend is the
-// mismatch substitution.  One ALU instruction (the mask) per register.
+// running, so every 16 pairs they are pruned explicitly.  (Per-register
+// masks take 5 more instructions per register, on a quarter of the pairs.)
+//   Key.  r + (S-1-slot) per half, compared signed, KS = 2^(slot bits): for
+// live cells it orders by value and then by lowest slot.  Across lanes the
+// key becomes value * 2^(SB+5) + (31 - lane) * 2^SB + slot bits, so one group
+// maximum gives the largest value and, among equal ones, the lowest window
+// slot: the first cell in order of increasing i on the diagonal.
 //
 // Layout.  Lane g of a group of L lanes holds the window slots g*S .. g*S+S-1
 // (S = 2*C2 slots).  Register t holds slot t in its low half and slot t+C2
 // in its high half, so the neighbour slot s+1 (s-1) of every slot in
 // register t sits in register t+1 (t-1) at the same half; only the end
-// registers need a byte permute and one shuffle per diagonal.
+// registers need a byte permute and, between lanes, one shuffle.
 //
-// Ranges, absolute frame, in units of r, with kR = (0x8000 / KS - 8) - 3 match - 3|gap|
-// the rebase step (rebase_step16: at least 1656 for KS = 16 and 632 for
-// KS = 32 inside the ranges above, and at least match + 2|gap|, the most
-// one pair of diagonals can raise a threshold); the figures below are for
-// KS = 16, and for KS = 32 they halve (thresholds <= 1016, keys below
-// 2^16 by x + match <= 1022, 32 r below 2^16).
-// After every pair of diagonals (odd d-1, even d) the frame is rebased by
-// kR once thr of d-1 reaches kR + match + 1.  Every live value of d-1 and d
-// is at least that threshold, so it stays above match + 1 > 0 after the
-// rebase, and the next threshold is again at least match + 2|gap| + 1.
-// thr grows by at most 3|gap| + 2 match over the three diagonals between
-// two tests, so thr <= 2040 always (16 thr < 0x8000: the key's pruned
-// range stays non-negative) and every live value is at most
-// thr + x + match <= 3576 (16 times that < 2^16).
-//
-// Carry-free adds, absolute frame.  V + s2 (stored value plus packed substitution, s2 <=
-// 16*256), z + idx (z = 0x8000 - 16 thr per half) and r + (z + idx) are
-// plain 32-bit adds: by the ranges above no low half, read unsigned,
-// reaches 2^16, so nothing carries into the high half.
-//
-// Window edges (both frames).  The edges are tested once per pair of diagonals,
-// after the even one: no live cell of diagonals d+1, d+2 can leave the
-// window unless E's top slot (diagonal d) or O's top slot (d-1) is live,
-// or E's bottom slot is.  The window then shifts up one slot if E's two
-// bottom slots and O's bottom slot are dead, or down one slot if the two
-// top slots of E and of O are dead; otherwise the band has outgrown the
-// window and the task goes to a wider tier.
+// Window edges.  The edges are tested once per pair of diagonals, after the
+// even one: no live cell of diagonals d+1, d+2 can leave the window unless
+// E's top slot (diagonal d) or O's top slot (d-1) is live, or E's bottom slot
+// is.  The window can then shift up by k slots if E's k+1 bottom slots and
+// O's k bottom slots are dead, or down by k if the k+1 top slots of E and of
+// O are dead; it shifts by NSH slots (an eighth of the window, at most a
+// quarter lane) if it can, since a band that drifts by chance comes back to
+// such an edge far less often than to one shifted by one slot, else by one
+// slot; otherwise the band has outgrown the window and the task goes to a
+// wider tier.
 #pragma once
 #include <stdint.h>
 
 #include <type_traits>
 
 #include "xd_device.cuh"
+#include "xd_lockstep16_abs.cuh"
 
 namespace xd {
 
 namespace p16 {
 
-constexpr int32_t kScale = 16;       // stored value = 16 * r
-constexpr uint32_t kKey2 = 0x80008000u;  // key offset in both halves: live iff bit 15
+constexpr uint32_t kDead2 = 0xC000C000u;  // a pruned slot, both halves
 
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
-{
-    uint32_t r;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
-    return r;
-}
-
-__host__ __device__ inline uint32_t pack2(int32_t v) { return ((uint32_t)v & 0xFFFFu) * 0x10001u; }
-
-// a * one + b with one == 1 at run time: the same value as a + b (and as
-// a << s for one << s), issued as a multiply-add on the FMA pipe.  Every DPX,
-// byte-permute, logic and min/max instruction of the loop issues on the ALU
-// pipe, which bounds it; the compiler would issue these adds and shifts there
-// too.  `one` is a kernel argument, so the compiler cannot fold the multiply.
-__device__ __forceinline__ uint32_t fma_add(uint32_t a, uint32_t one, uint32_t b)
-{
-    uint32_t r;
-    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(one), "r"(b));
-    return r;
-}
-
-// The high word of a * b, plus c (FMA pipe).
-__device__ __forceinline__ uint32_t mad_hi(uint32_t a, uint32_t b, uint32_t c)
-{
-    uint32_t r;
-    asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
-    return r;
-}
-
-template <int C2>
-__host__ __device__ constexpr uint32_t idx2(int t)
-{
-    return (uint32_t)(2 * C2 - 1 - t) | ((uint32_t)(2 * C2 - 1 - (t + C2)) << 16);
-}
-
-// Lane slots of register t (low: t, high: t + C2) and their negations.
-template <int C2>
-__host__ __device__ constexpr uint32_t slot2(int t)
-{
-    return (uint32_t)t | ((uint32_t)(t + C2) << 16);
-}
-template <int C2>
-__host__ __device__ constexpr uint32_t nslot2(int t)
-{
-    return ((uint32_t)(-t) & 0xFFFFu) | (((uint32_t)(-(t + C2)) & 0xFFFFu) << 16);
-}
-
-// Register t's match bits: shifted left by 12 - 4 (t >> 1) they sit at
-// bits p and p + 16, p = 13 + 2 (t & 1) (see the header).
-__host__ __device__ constexpr int subst_shift(int t) { return 12 - 4 * (t >> 1); }
-__host__ __device__ constexpr uint32_t subst_mask(int t)
-{
-    return (1u << (13 + 2 * (t & 1))) | (1u << (29 + 2 * (t & 1)));
-}
-
-template <int N>
-__device__ __forceinline__ uint32_t tree_max2(const uint32_t (&k)[N])
-{
-    if constexpr (N == 1) {
-        return k[0];
-    } else if constexpr (N == 2) {
-        return __vmaxu2(k[0], k[1]);
-    } else {
-        constexpr int M = (N + 2) / 3;
-        uint32_t r[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            if (3 * i + 2 < N) r[i] = __vimax3_u16x2(k[3 * i], k[3 * i + 1], k[3 * i + 2]);
-            else if (3 * i + 1 < N) r[i] = __vmaxu2(k[3 * i], k[3 * i + 1]);
-            else r[i] = k[3 * i];
-        }
-        return tree_max2<M>(r);
-    }
-}
+__device__ __forceinline__ bool rel_live_lo(uint32_t v) { return (v & 0x8000u) == 0u; }
+__device__ __forceinline__ bool rel_live_hi(uint32_t v) { return (int32_t)v >= 0; }
 
 template <int N>
 __device__ __forceinline__ uint32_t tree_max2s(const uint32_t (&k)[N])
@@ -233,84 +118,11 @@ __device__ __forceinline__ uint32_t tree_max2s(const uint32_t (&k)[N])
     }
 }
 
-// A slot is live iff its half is nonzero (pruned slots hold 0).
-__device__ __forceinline__ bool live_lo(uint32_t v) { return (v & 0xFFFFu) != 0; }
-__device__ __forceinline__ bool live_hi(uint32_t v) { return (v >> 16) != 0; }
-
-// Key units per unit of r, and slot bits of a key: lanes of up to 16 slots
-// keep 16 r and a 4-bit slot index; lanes of 32 slots a 5-bit index, with
-// keys in units of 32 r (the key add doubles the stored value).
-template <int S>
-__host__ __device__ constexpr int key_scale() { return S <= 16 ? 16 : 32; }
-template <int S>
-__host__ __device__ constexpr int slot_bits() { return S <= 16 ? 4 : 5; }
-
-// One anti-diagonal for one lane: V (diagonal d-2, overwritten with d) and
-// U (d-1).  edge: the neighbouring lane's end register of U (next lane's
-// register 0 on odd diagonals, previous lane's register C2-1 on even ones),
-// 0 beyond the group.  eq7: bit 2s+1 set iff slot s's bases match (slots
-// 0-15); eqh: the same for slots 16-31 (C2 = 16 only).  k13, k15:
-// 16 (match - mismatch) << 19 and << 17; mi2: the packed mismatch
-// substitution 16 (mismatch + 2|gap|); z: 0x8000 - KS thr in both halves
-// (KS = key_scale).  Returns the lane's largest key (0 .. 0xFFFF; below
-// 0x8000 iff every slot was pruned).
-template <int C2, bool ODD, bool MASKED>
-__device__ __forceinline__ uint32_t dp16(uint32_t (&V)[C2], const uint32_t (&U)[C2],
-                                         uint32_t edge, uint32_t eq7, uint32_t eqh,
-                                         uint32_t mi2, uint32_t k13, uint32_t k15, uint32_t z,
-                                         uint32_t lo1_2, uint32_t nhi1_2, uint32_t one)
-{
-    static_assert(C2 == 4 || C2 == 8 || C2 == 16, "packed registers per lane");
-    constexpr int NE = C2 == 16 ? 2 : 1;
-    // e[h]: slot t's match bit at 2t+1, slot t+C2's at 2t+17 (registers
-    // 8h .. 8h+7)
-    uint32_t e[NE];
-    if constexpr (C2 == 4) e[0] = prmt(eq7, eq7, 0x2100);
-    else if constexpr (C2 == 8) e[0] = eq7;
-    else { e[0] = prmt(eq7, eqh, 0x5410); e[1] = prmt(eq7, eqh, 0x7632); }
-    uint32_t es[4 * NE];
-#pragma unroll
-    for (int h = 0; h < NE; ++h) {
-        es[4 * h] = fma_add(e[h], one << 12, 0u);
-        es[4 * h + 1] = fma_add(e[h], one << 8, 0u);
-        es[4 * h + 2] = fma_add(e[h], one << 4, 0u);
-        es[4 * h + 3] = e[h];
-    }
-    uint32_t key[C2];
-#pragma unroll
-    for (int t = 0; t < C2; ++t) {
-        uint32_t sh;
-        if (ODD) sh = (t + 1 < C2) ? U[t + 1] : prmt(U[0], edge, 0x5432);
-        else sh = (t > 0) ? U[t - 1] : prmt(edge, U[C2 - 1], 0x5432);
-        const uint32_t w = es[t >> 1] & subst_mask(t);
-        const uint32_t s2 = mad_hi(w, (t & 1) ? k15 : k13, mi2);
-        uint32_t r = __vimax3_u16x2(fma_add(V[t], one, s2), U[t], sh);  // carry-free (header)
-        if (MASKED) {
-            // slot s lies in the rectangle iff lo <= s <= hi (lo = j0 - n,
-            // hi = m - i0): max(s - hi - 1, lo - 1 - s) < 0, per half
-            const uint32_t c = __viaddmax_s16x2(nslot2<C2>(t), lo1_2, 0x80008000u);
-            const uint32_t u = __viaddmax_s16x2(slot2<C2>(t), nhi1_2, c);
-            r &= prmt(u, u, 0xBB99);  // 0xFFFF where inside
-        }
-        // 0x8000 + KS*(r - thr) + (S-1-slot): bit 15 set iff live
-        const uint32_t k = fma_add(r, (key_scale<2 * C2>() == 16) ? one : one << 1,
-                                   fma_add(z, one, idx2<C2>(t)));
-        V[t] = r & prmt(k, k, 0xBB99);
-        key[t] = k;
-    }
-    const uint32_t kk = tree_max2<C2>(key);
-    return max(kk >> 16, kk & 0xFFFFu);
-}
-
-// ---- relative frame (see the header comment) ----
-
-constexpr uint32_t kDead2 = 0xC000C000u;  // a pruned slot, both halves
-
 // Match-bit positions.  A lane's shifted flag word puts register t's two
-// flags at bits pos and pos + 16.  Lanes of 32 slots (KS = 32) serve three
-// registers with one shift (positions 1, 3, 5), the others two (1, 3).
+// flags at bits pos and pos + 16.  With KS >= 32 one shift serves three
+// registers (positions 1, 3, 5), else two (1, 3).
 template <int C2>
-__host__ __device__ constexpr int rel_group() { return C2 == 16 ? 3 : 2; }
+__host__ __device__ constexpr int rel_group() { return C2 >= 16 ? 3 : 2; }
 template <int C2>
 __host__ __device__ constexpr int rel_pos(int t) { return 1 + 2 * ((t % 8) % rel_group<C2>()); }
 
@@ -332,6 +144,61 @@ __device__ __forceinline__ uint32_t keep_range(uint32_t v, int t, int32_t lo, in
     return (v & (l | h)) | (kDead2 & ~(l | h));
 }
 
+// N words of 16 bases each from consecutive base positions, word k starting
+// 16 * step * k bases (step = 1 or -1) after base pos of word w0 of the packed
+// buffer, its 16 fields in reverse order with rev.  One code path for
+// both directions (groups of one warp differ in theirs) in 32-bit
+// arithmetic; words outside the buffer are clamped (ld_word).
+template <int N>
+__device__ __forceinline__ void load_words(const uint32_t *pk, int32_t last, int32_t w0,
+                                           int32_t pos, int step, bool rev, uint32_t (&out)[N])
+{
+    const int32_t w = w0 + (pos >> 4) + (step < 0 ? 1 : 0);
+    const uint32_t sh = 2u * (uint32_t)(pos & 15);
+    uint32_t r[N + 1];
+#pragma unroll
+    for (int k = 0; k <= N; ++k) r[k] = __ldg(pk + min(max(w + step * k, 0), last));
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const uint32_t v = __funnelshift_r(step > 0 ? r[k] : r[k + 1], step > 0 ? r[k + 1] : r[k], sh);
+        out[k] = rev ? rev16(v) : v;
+    }
+}
+
+// V moved by K slots towards lane 0 (UP: slot s takes slot s + K) or away
+// from it, where mine; the slots that enter come from the neighbouring lane,
+// pruned beyond the group.  Every lane of the warp takes part.
+template <int L, int C2, int K, bool UP>
+__device__ __forceinline__ void shift_slots(uint32_t (&V)[C2], bool mine, bool edge_lane)
+{
+    static_assert(K < C2, "shift within a register's reach");
+    uint32_t in[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        in[q] = kDead2;
+        if constexpr (L > 1) {
+            in[q] = UP ? __shfl_down_sync(FULL, V[q], 1, L) : __shfl_up_sync(FULL, V[C2 - 1 - q], 1, L);
+            if (edge_lane) in[q] = kDead2;
+        }
+    }
+    if (!mine) return;
+    uint32_t e[K];  // the registers whose slots cross a half
+#pragma unroll
+    for (int q = 0; q < K; ++q)
+        e[q] = UP ? prmt(V[q], in[q], 0x5432) : prmt(in[q], V[C2 - 1 - q], 0x5432);
+    if (UP) {
+#pragma unroll
+        for (int t = 0; t < C2 - K; ++t) V[t] = V[t + K];
+#pragma unroll
+        for (int q = 0; q < K; ++q) V[C2 - K + q] = e[q];
+    } else {
+#pragma unroll
+        for (int t = C2 - 1; t >= K; --t) V[t] = V[t - K];
+#pragma unroll
+        for (int q = 0; q < K; ++q) V[K - 1 - q] = e[q];
+    }
+}
+
 // Per-group constants of the substitution: k[q] multiplies a flag at bit
 // 1 + 2q into the match bonus, c[q] (both halves) the mismatch score when
 // the scoring allows it (else 0, and mi2 is added).
@@ -340,83 +207,66 @@ struct RelSubst {
     uint32_t mi2;
 };
 
-// One anti-diagonal for one lane in the relative frame.  V: diagonal d-2 (in
-// its own frame), overwritten with d; U: diagonal d-1 plus the threshold
-// step from d-2 to d-1, so both predecessors are in the frame of d-2.
-// nstep: minus the threshold step from d-2 to d, per half.
-template <int C2, bool ODD, bool ADD>
+// One anti-diagonal for one lane.  V: diagonal d-2 (in its own frame),
+// overwritten with d; U: diagonal d-1 plus the threshold step from d-2 to
+// d-1, so both predecessors are in the frame of d-2.  edge: the neighbouring
+// lane's end register of U.  eq[w]: bit 2s+1 set iff the bases of slot
+// 16w + s match.  nstep: minus the threshold step from d-2 to d, per half.
+// Returns the largest keys of the low and of the high halves, in the frame
+// of d-2 and before the prune: they do not wait for the threshold of d, which
+// the previous diagonal's maximum decides, so the two diagonals' chains
+// overlap.
+template <int C2, int NW, bool ODD, bool ADD>
 __device__ __forceinline__ uint32_t dp16r(uint32_t (&V)[C2], const uint32_t (&U)[C2],
-                                          uint32_t edge, uint32_t eq7, uint32_t eqh,
+                                          uint32_t edge, const uint32_t (&eq)[NW],
                                           const RelSubst &sb, uint32_t nstep, uint32_t one)
 {
     constexpr int G = rel_group<C2>();
     constexpr int NS = (8 + G - 1) / G;  // shifts per flag word of 8 registers
-    constexpr int NE = C2 == 16 ? 2 : 1;
-    uint32_t e[NE];  // slot t's flag at 2t+1, slot t+C2's at 2t+17
-    if constexpr (C2 == 2) e[0] = (eq7 & 0xFu) | (eq7 << 12);
-    else if constexpr (C2 == 4) e[0] = prmt(eq7, eq7, 0x2100);
-    else if constexpr (C2 == 8) e[0] = eq7;
-    else { e[0] = prmt(eq7, eqh, 0x5410); e[1] = prmt(eq7, eqh, 0x7632); }
+    constexpr int NE = C2 >= 16 ? C2 / 8 : 1;
+    // registers 8h .. 8h+7: slot t's flag at 2(t-8h)+1, slot t+C2's 16 bits on
     uint32_t es[NE][NS];
 #pragma unroll
-    for (int h = 0; h < NE; ++h)
+    for (int h = 0; h < NE; ++h) {
+        uint32_t e;
+        if constexpr (C2 == 2) e = (eq[0] & 0xFu) | (eq[0] << 12);
+        else if constexpr (C2 == 4) e = prmt(eq[0], eq[0], 0x2100);
+        else if constexpr (C2 == 8) e = eq[0];
+        else e = prmt(eq[h / 2], eq[NW / 2 + h / 2], (h & 1) ? 0x7632 : 0x5410);
 #pragma unroll
-        for (int q = 0; q < NS; ++q) es[h][q] = e[h] >> (2 * G * q);
+        for (int q = 0; q < NS; ++q) es[h][q] = e >> (2 * G * q);
+    }
     uint32_t key[C2];
 #pragma unroll
     for (int t = 0; t < C2; ++t) {
         uint32_t sh;
         if (ODD) sh = (t + 1 < C2) ? U[t + 1] : prmt(U[0], edge, 0x5432);
         else sh = (t > 0) ? U[t - 1] : prmt(edge, U[C2 - 1], 0x5432);
-        constexpr uint32_t kBit = 0x00010001u;
         const int q = (t % 8) % G;
-        const uint32_t w = (es[t / 8][(t % 8) / G] & (kBit << rel_pos<C2>(t))) | sb.c[q];
+        const uint32_t w = (es[t / 8][(t % 8) / G] & (0x00010001u << rel_pos<C2>(t))) | sb.c[q];
         uint32_t cand = fma_add(w, sb.k[q], V[t]);
         if (ADD) cand = fma_add(cand, one, sb.mi2);
         const uint32_t r = __vimax3_s16x2(cand, U[t], sh);
         // r - threshold step: a live cell stays >= 0; below the threshold it
         // wraps to an unsigned value above kDead, which the minimum replaces
-        const uint32_t v = __viaddmin_u16x2(r, nstep, kDead2);
-        V[t] = v;
-        key[t] = fma_add(v, one, idx2<C2>(t));
+        V[t] = __viaddmin_u16x2(r, nstep, kDead2);
+        key[t] = fma_add(r, one, idx2<C2>(t));
     }
     return tree_max2s<C2>(key);
 }
 
 }  // namespace p16
 
-__host__ __device__ inline bool packed16_ok(const Scoring &sc)
-{
-    return sc.match - sc.gap <= 128 && sc.mismatch >= -128 && sc.mismatch - 2 * sc.gap >= 0 &&
-           sc.x >= 0 && sc.x + sc.match <= 1536;
-}
-
-// Lanes of 32 slots keep keys in units of 32 r, so their keys (0x8000 +
-// 32 (x + match) + 31 at most) need x + match <= 1022 as well.
-__host__ __device__ inline bool packed32_ok(const Scoring &sc)
-{
-    return packed16_ok(sc) && sc.x + sc.match <= 1022;
-}
-
-// Frame step of one rebase (units of r) for a scoring that passes
-// packed16_ok: the threshold cap 0x8000 / KS - 8 (2040 or 1016) less
-// 3 match + 3|gap|, so between 1656 and 2033 for lanes of up to 16 slots
-// and between 632 and 1009 for lanes of 32 (see the header comment's
-// ranges).
-template <int S>
-__host__ __device__ inline int32_t rebase_step16(const Scoring &sc)
-{
-    return (0x8000 / p16::key_scale<S>() - 8) - 3 * sc.match + 3 * sc.gap;
-}
-
 // The relative frame on lanes of S slots: every value a step forms from a
 // live one, at most x + 2 match + 2|gap| in units of KS, stays below 2^15.
-// Lanes of up to 16 slots hold every scoring of packed16_ok.
+// Lanes of up to 16 slots hold every scoring of packed16_ok.  With KS = 64
+// the steps are kept below 2^12, so that pruned slots sink slowly enough.
 template <int S>
 __host__ __device__ inline bool relative_ok(const Scoring &sc)
 {
     return packed16_ok(sc) &&
-           (sc.x + 2 * sc.match - 2 * sc.gap + 1) * p16::key_scale<S>() <= 0x8000;
+           (sc.x + 2 * sc.match - 2 * sc.gap + 1) * p16::key_scale<S>() <= 0x8000 &&
+           (S < 64 || sc.match - sc.gap <= 64);
 }
 
 // Whether the mismatch score can ride on the flag word (RelSubst::c): c =
@@ -441,85 +291,82 @@ __host__ __device__ inline int32_t lift_period(const Scoring &sc)
     return p < 1 ? 1 : p;
 }
 
-// REL: the relative frame (the scoring passes relative_ok<2 * C2>); else the
-// absolute one.  one: 1 (see fma_add).
-template <int L, int C2, bool REL, class Src>
+// one: 1 (see fma_add).
+template <int L, int C2, class Src>
 __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, int64_t nw,
                                                 uint32_t one)
 {
     using namespace p16;
     constexpr int S = 2 * C2;  // slots per lane
     constexpr int W = L * S;
-    constexpr bool WIDE = S == 32;              // two base-window words per read
-    constexpr int SB = slot_bits<S>();          // slot bits of a key
-    constexpr int VS = SB + 5;                  // value shift of a group key
+    constexpr int NW = S > 16 ? S / 16 : 1;      // base-window words per read
+    constexpr int SB = slot_bits<S>();           // slot bits of a key
+    constexpr int VS = L == 1 ? SB : SB + 5;     // value shift of a group key
     constexpr uint32_t SMASK = (1u << SB) - 1u;
-    // -KS * 0x10001: z = 0x80008000 - KS thr in both halves
-    constexpr uint32_t ZMUL = 0u - (uint32_t)key_scale<S>() * 0x10001u;
-    static_assert(S <= 32 && 32 % L == 0 && L >= 2 && C2 % 2 == 0, "packed tile shape");
-    static_assert(REL || C2 % 4 == 0, "packed tile shape, absolute frame");
     constexpr uint32_t KS = (uint32_t)key_scale<S>();
-    constexpr uint32_t kPruned = REL ? kDead2 : 0u;  // a pruned slot, both halves
+    // slots of a long window shift
+    constexpr int NSH = S / 4 < 2 ? 1 : S / 4 < W / 8 ? S / 4 : W / 8;
+    constexpr int32_t kForever = 1 << 20;
+    using T0 = std::integral_constant<bool, false>;
+    using T1 = std::integral_constant<bool, true>;
+    static_assert(S <= 64 && 32 % L == 0 && (C2 == 2 || C2 == 4 || C2 == 8 || C2 % 16 == 0),
+                  "packed tile shape");
     const int lane = threadIdx.x & 31;
     const int glane = lane % L;
     const int gbase = lane - glane;
     const unsigned gm = group_mask<L>(gbase);
     const bool bot_lane = glane == 0, top_lane = glane == L - 1;
-    // per-lane constants: 0/1 factors that clear the shuffled-in edge
-    // beyond the group, and the halves the window-edge test reads
+    // per-lane constants: factors and addends that prune the edge beyond
+    // the group
     const uint32_t keep_up = top_lane ? 0u : 1u, keep_dn = bot_lane ? 0u : 1u;
-    const uint32_t edge_up = top_lane ? kPruned : 0u, edge_dn = bot_lane ? kPruned : 0u;
-    const uint32_t tmask = top_lane ? (REL ? 0x80000000u : 0xFFFF0000u) : 0u;
-    const uint32_t bmask = bot_lane ? (REL ? 0x00008000u : 0x0000FFFFu) : 0u;
-    // a slot is live iff its half is nonzero (absolute frame) or not
-    // negative (relative frame)
-    auto lo_live = [](uint32_t v) { return REL ? (v & 0x8000u) == 0u : live_lo(v); };
-    auto hi_live = [](uint32_t v) { return REL ? (int32_t)v >= 0 : live_hi(v); };
+    const uint32_t edge_up = top_lane ? kDead2 : 0u, edge_dn = bot_lane ? kDead2 : 0u;
 
     // Per-group task state (uniform within a group).
     bool active = false, exhausted = false;
     uint32_t task = 0;
     const Job *gj = nullptr;
     Scoring sc{1, -1, -1, 0};
-    int64_t sa0 = 0, sb0 = 0;
+    int32_t aw0 = 0, bw0 = 0, ab0 = 0, bb0 = 0;  // word and base in it of both streams' first base
     int dir = 1;
-    int32_t mn = 0, m = 0, n = 0, d = 0, i0 = 0, j0 = 0, T = 0, bi = 0, bj = 0;
-    int32_t Q = 0;                      // frame offset: thr = T + Q
-    int32_t kR = 0, kRL = 0;            // rebase step, and the threshold that triggers one
-    int32_t xup = 0;                    // (x + 1) << VS: a group key this large raises T
+    int32_t mn = 0, m = 0, n = 0, d = 0, i0 = 0, j0 = 0, T = 0;
     int32_t bkey = 0, bi0 = 0, bd = 0;  // best cell: group key, this lane's i0, diagonal
-    int32_t ng = 1;                     // |gap|
-    uint32_t mi2 = 0;                   // packed 16 * (mismatch + 2|gap|)
-    uint32_t k13 = 0, k15 = 0;          // 16 (match - mismatch) << 19, << 17
-    RelSubst rs = {{0, 0, 0}, {0, 0, 0}, 0};  // relative frame: substitution constants
-    uint32_t dA = 0, dB = 0;            // relative frame: threshold steps d-2 -> d-1, d-1 -> d
+    RelSubst rs = {{0, 0, 0}, {0, 0, 0}, 0};
+    uint32_t dA = 0, dB = 0;            // threshold steps d-2 -> d-1, d-1 -> d
+    int32_t sA = 0, sB = 0;             // the same steps in units of the score
+    int32_t ng = 0;                     // |gap|
     uint32_t ngp = 0;                   // |gap| * KS in both halves
-    int32_t lift = 1 << 20;             // relative frame: lift_period of the group's scoring
-    int32_t lift_n = 1 << 20;           // warp-uniform: pairs until the next lift
+    int32_t lift = kForever;            // lift_period of the group's scoring
     bool add_mi = false;                // the group's scoring needs rs.mi2 added
-    bool generic = false;               // warp-uniform: some group's does
-    bool prev_dead = false, fin = false, rb = false;
+    // event masks, 0 while the group waits: the half of this lane's end
+    // slots the edge test reads, and the sign bit for the end test
+    uint32_t tmask = 0, bmask = 0, amask = 0;
+    int32_t ptop = 0;                   // best value of the last even diagonal
+    uint32_t finw = 0;                  // nonzero: two dead diagonals in a row
     uint32_t E[C2], O[C2];
 #pragma unroll
-    for (int t = 0; t < C2; ++t) { E[t] = kPruned; O[t] = kPruned; }
-    // base windows (slots 0-15; Aw1, Bw1: slots 16-31 of 32-slot lanes) and
-    // the lookahead words
-    uint32_t Aw = 0, Aw1 = 0, LA = 0, Bw = 0, Bw1 = 0, LB = 0;
-    int la_n = 16;        // warp-uniform: diagonal pairs the lookahead words still cover
-    int32_t budget = 0;   // warp-uniform: diagonal pairs known to stay inside every rectangle
-    // (31 - lane) * 16, less the key offset's share of the group key
-    const int32_t lane_bits = ((31 - glane) << SB) - (REL ? 0 : (0x8000 << 5));
+    for (int t = 0; t < C2; ++t) { E[t] = kDead2; O[t] = kDead2; }
+    uint32_t Aw[NW], Bw[NW], LA = 0, LB = 0;  // base windows, lookahead words
+#pragma unroll
+    for (int k = 0; k < NW; ++k) { Aw[k] = 0; Bw[k] = 0; }
+    // Warp-uniform countdowns, in pairs of diagonals.
+    int la_n = 16;             // the lookahead words still cover
+    int32_t budget = 0;        // known to stay inside every rectangle
+    int32_t lift_n = kForever; // until pruned slots must be lifted
+    int32_t ctr = 0, ctr0 = 0; // until the next event that is due anyway, and its start
+    const int32_t lane_bits = (31 - glane) << SB;
 
     auto retire = [&](bool overflow) {
+        int32_t bi = 0, bj = 0;
         if (bd > 0) {
-            bi = (bi0 - glane * S) + (31 - ((bkey >> SB) & 31)) * S + (S - 1 - (int)(bkey & SMASK));
+            const int32_t slot = S - 1 - (int)(bkey & SMASK);
+            bi = L == 1 ? bi0 + slot : (bi0 - glane * S) + (31 - ((bkey >> SB) & 31)) * S + slot;
             bj = bd - bi;
         }
         if (glane == 0) src.retire(gj, task, overflow, T, bi, bj);
         active = false;
-        ng = 0;  // the frame offset stays put while the group waits
+        tmask = bmask = amask = 0;
         add_mi = false;
-        lift = 1 << 20;
+        lift = kForever;
     };
 
     // Diagonal pairs until a cell of this group's window can leave the
@@ -532,211 +379,170 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
 
     // The base windows of this lane's slots at the current i0, j0: slot s
     // holds a[i0 + s] and b[j0 - s]; the lookahead words the next 16 bases.
+    const int32_t last = (int32_t)nw - 1;
+    auto load_ahead = [&]() {
+        uint32_t v[1];
+        const int32_t ia = i0 + 16 * NW;
+        load_words<1>(pk, last, aw0, ab0 + (dir > 0 ? ia - 1 : -ia - 14), 1, dir < 0, v);
+        LA = v[0];
+        load_words<1>(pk, last, bw0, bb0 + (dir > 0 ? j0 : -j0 - 15), 1, dir > 0, v);
+        LB = v[0];
+    };
     auto load_windows = [&]() {
-        Aw = fwd16_u(pk, nw, sa0, dir, i0);
-        Bw = back16_u(pk, nw, sb0, dir, j0);
-        if constexpr (WIDE) {
-            Aw1 = fwd16_u(pk, nw, sa0, dir, i0 + 16);
-            Bw1 = back16_u(pk, nw, sb0, dir, j0 - 16);
-        }
-        LA = fwd16_u(pk, nw, sa0, dir, i0 + (WIDE ? 32 : 16));
-        LB = back16_u(pk, nw, sb0, dir, j0 + 16);
+        uint32_t v[NW + 1];
+        load_words<NW + 1>(pk, last, aw0, ab0 + (dir > 0 ? i0 - 1 : -i0 - 14), dir, dir < 0, v);
+#pragma unroll
+        for (int k = 0; k < NW; ++k) Aw[k] = v[k];
+        LA = v[NW];
+        load_words<NW + 1>(pk, last, bw0, bb0 + (dir > 0 ? j0 : -j0 - 15), -dir, dir > 0, v);
+        LB = v[0];
+#pragma unroll
+        for (int k = 0; k < NW; ++k) Bw[k] = v[k + 1];
     };
 
     // One anti-diagonal and the bookkeeping that cannot wait for the end of
-    // the pair: T and the best cell.  Returns the group key (negative iff
-    // every cell of the diagonal was pruned) and the diagonal's threshold.
-    auto diag = [&](auto odd_tag, auto masked_tag, auto add_tag, int32_t &thr) -> int32_t {
+    // the pair: T and the best cell.  Returns the best value above the
+    // threshold (negative iff every cell of the diagonal was pruned).
+    auto diag = [&](auto odd_tag, auto masked_tag, auto add_tag) -> int32_t {
         constexpr bool ODD = decltype(odd_tag)::value;
         constexpr bool MASKED = decltype(masked_tag)::value;
         constexpr bool ADD = decltype(add_tag)::value;
         ++d;
         if (ODD) {
             ++i0;
-            if constexpr (WIDE) {
-                Aw = __funnelshift_r(Aw, Aw1, 2);
-                Aw1 = __funnelshift_r(Aw1, LA, 2);
-            } else {
-                Aw = __funnelshift_r(Aw, LA, 2);
-            }
+#pragma unroll
+            for (int k = 0; k < NW; ++k)
+                Aw[k] = __funnelshift_r(Aw[k], k + 1 < NW ? Aw[k + 1] : LA, 2);
             LA >>= 2;
         } else {
             ++j0;
-            if constexpr (WIDE) Bw1 = __funnelshift_l(Bw, Bw1, 2);
-            Bw = __funnelshift_l(LB, Bw, 2);
+#pragma unroll
+            for (int k = NW - 1; k > 0; --k) Bw[k] = __funnelshift_l(Bw[k - 1], Bw[k], 2);
+            Bw[0] = __funnelshift_l(LB, Bw[0], 2);
             LB <<= 2;
         }
-        // rectangle bounds of this lane's slots, clamped into 16 bits (only
-        // the masked copy reads them)
-        uint32_t lo1_2 = 0, nhi1_2 = 0;
-        if (MASKED && !REL) {
-            const int32_t lo = j0 - n, hi = m - i0;
-            lo1_2 = pack2(min(max(lo - 1, -1024), 1024));
-            nhi1_2 = pack2(min(max(-hi - 1, -1024), 1024));
-        }
-        const uint32_t xx = Aw ^ Bw;
-        uint32_t eq7 = ~(xx | (xx << 1));
-        uint32_t eqh = 0u;
-        if constexpr (WIDE) {
-            const uint32_t xh = Aw1 ^ Bw1;
-            eqh = ~(xh | (xh << 1));
-        }
-        if (MASKED && REL) {  // no match outside the rectangle (header comment)
-            const int32_t lo = j0 - n, hi = m - i0;
-            eq7 &= flag_range(lo, hi);
-            if constexpr (WIDE) eqh &= flag_range(lo - 16, hi - 16);
-        }
-        int32_t lk;
-        if constexpr (REL) {
-            // diagonal d-1 in the frame of d-2; both halves of dA and dB are equal
-            const uint32_t nstep = 0x00010000u - (dA + dB);
-            uint32_t U[C2];
+        uint32_t eq[NW];
 #pragma unroll
-            for (int t = 0; t < C2; ++t) U[t] = fma_add(ODD ? E[t] : O[t], one, dA);
-            uint32_t kk;
-            if (ODD) {
-                const uint32_t edge = fma_add(__shfl_down_sync(FULL, U[0], 1, L), keep_up, edge_up);
-                kk = dp16r<C2, true, ADD>(O, U, edge, eq7, eqh, rs, nstep, one);
-            } else {
-                const uint32_t edge =
-                    fma_add(__shfl_up_sync(FULL, U[C2 - 1], 1, L), keep_dn, edge_dn);
-                kk = dp16r<C2, false, ADD>(E, U, edge, eq7, eqh, rs, nstep, one);
-            }
-            lk = max((int32_t)kk >> 16, (int32_t)(kk << 16) >> 16);
-        } else {
-            Q += ng;
-            thr = T + Q;
-            // 0x8000 - 16 thr in both halves (no borrow: 16 thr <= 0x8000)
-            const uint32_t z = (uint32_t)thr * ZMUL + kKey2;
-            if (ODD) {
-                const uint32_t edge = fma_add(__shfl_down_sync(FULL, E[0], 1, L), keep_up, edge_up);
-                lk = (int32_t)dp16<C2, true, MASKED>(O, E, edge, eq7, eqh, mi2, k13, k15, z, lo1_2,
-                                                     nhi1_2, one);
-            } else {
-                const uint32_t edge =
-                    fma_add(__shfl_up_sync(FULL, O[C2 - 1], 1, L), keep_dn, edge_dn);
-                lk = (int32_t)dp16<C2, false, MASKED>(E, O, edge, eq7, eqh, mi2, k13, k15, z, lo1_2,
-                                                      nhi1_2, one);
-            }
+        for (int k = 0; k < NW; ++k) {
+            const uint32_t xx = Aw[k] ^ Bw[k];
+            eq[k] = ~(xx | (xx << 1));
+            if (MASKED) eq[k] &= flag_range(j0 - n - 16 * k, m - i0 - 16 * k);
         }
-        // Group key: value above lane above slot in lane, so one max finds
-        // the lowest window slot among the cells holding the maximum.  With
-        // lk = 2^SB v + i (plus 0x8000 in the absolute frame): 32 lk - 31 i =
-        // 2^VS v + i (plus 0x8000 * 32) (multiply-adds).
-        const int32_t mkey = lockstep_group_max<L>((int32_t)fma_add(
-            (uint32_t)lk, one << 5, fma_add((uint32_t)lk & SMASK, 0u - 31u, (uint32_t)lane_bits)));
-        if constexpr (REL) {
-            const int32_t rise = max((mkey >> VS) - sc.x, 0);  // best value above T
-            dA = dB;
-            dB = (uint32_t)rise * (KS * 0x10001u) + ngp;
-            T += rise;
-            if (rise > 0) {  // decoded at retire
-                bkey = mkey;
-                bi0 = i0;
-                bd = d;
-            }
-        } else if (mkey >= xup) {  // best value - thr > x: T rises (decoded at retire)
-            T += (mkey >> VS) - sc.x;
+        const uint32_t nstep = 0x00010000u - (dA + dB);  // both halves of dA and dB are equal
+        uint32_t U[C2];
+#pragma unroll
+        for (int t = 0; t < C2; ++t) U[t] = fma_add(ODD ? E[t] : O[t], one, dA);
+        uint32_t kk;
+        if (ODD) {
+            uint32_t edge = kDead2;
+            if constexpr (L > 1)
+                edge = fma_add(__shfl_down_sync(FULL, U[0], 1, L), keep_up, edge_up);
+            kk = dp16r<C2, NW, true, ADD>(O, U, edge, eq, rs, nstep, one);
+        } else {
+            uint32_t edge = kDead2;
+            if constexpr (L > 1)
+                edge = fma_add(__shfl_up_sync(FULL, U[C2 - 1], 1, L), keep_dn, edge_dn);
+            kk = dp16r<C2, NW, false, ADD>(E, U, edge, eq, rs, nstep, one);
+        }
+        int32_t mkey = max((int32_t)kk >> 16, (int32_t)(kk << 16) >> 16);
+        // with key = 2^SB v + i: 32 key - 31 i = 2^VS v + i (multiply-adds)
+        if constexpr (L > 1)
+            mkey = lockstep_group_max<L>((int32_t)fma_add(
+                (uint32_t)mkey, one << 5,
+                fma_add((uint32_t)mkey & SMASK, 0u - 31u, (uint32_t)lane_bits)));
+        // the best value above the diagonal's threshold, and above T
+        const int32_t top = (mkey >> VS) - (sA + sB);
+        const int32_t rise = max(top - sc.x, 0);
+        dA = dB;
+        dB = (uint32_t)rise * (KS * 0x10001u) + ngp;
+        sA = sB;
+        sB = rise + ng;
+        T += rise;
+        if (rise > 0) {  // decoded at retire
             bkey = mkey;
             bi0 = i0;
             bd = d;
         }
-        return mkey;
+        return top;
     };
 
     // One pair of anti-diagonals (odd, then even).  Returns the warp-wide
-    // "something to do" vote: a window edge went live, a task ended, the
-    // lookahead words ran out, a frame needs a rebase, the masking-free
-    // budget ran out, or a group waits for a task.
+    // "something to do" vote: a window edge went live, a task ended, or the
+    // countdown ran out.
     auto pair = [&](auto masked_tag, auto add_tag) -> bool {
         constexpr bool MASKED = decltype(masked_tag)::value;
-        int32_t thr_o = 0, thr_e = 0;
-        const int32_t key_o = diag(std::true_type{}, masked_tag, add_tag, thr_o);
-        const int32_t key_e = diag(std::false_type{}, masked_tag, add_tag, thr_e);
-        const bool dead_o = key_o < 0, dead_e = key_e < 0;
-        fin = active && ((dead_o && (prev_dead || dead_e)) || d >= mn);
-        prev_dead = dead_e;
-        --budget;
-        --la_n;
-        if constexpr (!REL) rb = active && thr_o >= kRL;
+        const int32_t top_o = diag(std::true_type{}, masked_tag, add_tag);
+        const int32_t top_e = diag(std::false_type{}, masked_tag, add_tag);
+        // sign bits: the odd diagonal is dead, and so is the even one before or after it
+        finw = (uint32_t)top_o & (uint32_t)(ptop | top_e) & amask;
+        if (MASKED && d >= mn) finw = amask;
+        ptop = top_e;
         // window edges: this group's bottom lane tests E's bottom slot, its
         // top lane the top slots of E and O
-        const uint32_t ew = REL ? (~(E[C2 - 1] & O[C2 - 1]) & tmask) | (~E[0] & bmask)
-                                : ((E[C2 - 1] | O[C2 - 1]) & tmask) | (E[0] & bmask);
-        const bool edge = active && ew != 0u;
-        bool ev = edge || fin || rb || la_n == 0 || (!active && !exhausted);
-        if (!MASKED) ev = ev || budget < 1;
-        return __any_sync(FULL, ev);
+        const uint32_t ew = (~(E[C2 - 1] & O[C2 - 1]) & tmask) | (~E[0] & bmask);
+        --ctr;
+        return __any_sync(FULL, (ew | finw) != 0u) || ctr == 0;
     };
 
-    // The rare work behind an event, after the even diagonal of a pair.
-    // Returns true when the loop must go back to the task switch (a group
-    // waits for a task, no group is left running, the masking-free budget
-    // no longer covers a pair, or, masked, it covers one again).
+    // The work behind an event, after the even diagonal of a pair.  Returns
+    // true when the loop must go back to the task switch (a group waits for
+    // a task, no group is left running, the masking-free budget no longer
+    // covers a pair, or, masked, it covers one again).
     auto handle = [&](const bool masked) -> bool {
-        bool ovf = false;
+        la_n -= ctr0 - ctr;
+        bool fin = finw != 0u, ovf = false;
         const bool go = active && !fin;
-        const bool need_dn_l = bot_lane && lo_live(E[0]);
-        const bool need_up_l = top_lane && (hi_live(E[C2 - 1]) || hi_live(O[C2 - 1]));
+        const bool need_dn_l = bot_lane && rel_live_lo(E[0]);
+        const bool need_up_l = top_lane && (rel_live_hi(E[C2 - 1]) || rel_live_hi(O[C2 - 1]));
         if (__any_sync(FULL, go && (need_dn_l || need_up_l))) {
-            // Per group: the decision of its bottom and top lanes.
-            const bool blk_up_l = lo_live(E[0]) || lo_live(E[1]) || lo_live(O[0]);
-            const bool blk_dn_l = hi_live(E[C2 - 1]) || hi_live(O[C2 - 1]) ||
-                                  hi_live(E[C2 - 2]) || hi_live(O[C2 - 2]);
-            // every lane takes part in every shuffle (no short-circuit
-            // around a warp-wide collective)
-            const bool up_g = __shfl_sync(FULL, (int)need_up_l, L - 1, L) != 0;
-            const bool dn_g = __shfl_sync(FULL, (int)need_dn_l, 0, L) != 0;
-            const bool bu = __shfl_sync(FULL, (int)blk_up_l, 0, L) != 0;
-            const bool bdn = __shfl_sync(FULL, (int)blk_dn_l, L - 1, L) != 0;
-            const bool nu = go && up_g;
-            const bool nd = go && dn_g;
-            ovf = (nu && bu) || (!nu && nd && bdn);
-            const bool su = nu && !bu;           // shift up: slot s takes slot s+1
-            const bool sd = !nu && nd && !bdn;   // shift down: slot s takes slot s-1
-            if (__any_sync(FULL, su)) {
-                uint32_t ne = __shfl_down_sync(FULL, E[0], 1, L);
-                uint32_t no = __shfl_down_sync(FULL, O[0], 1, L);
-                if (top_lane) { ne = kPruned; no = kPruned; }
-                if (su) {
-                    const uint32_t te = prmt(E[0], ne, 0x5432), to = prmt(O[0], no, 0x5432);
+            // dead slots at both ends of this lane: k + 1 of E (and of O at
+            // the top, k at the bottom), for k = 1 and k = NSH
+            uint32_t lo1 = E[0] & E[1] & O[0], hi1 = E[C2 - 1] & O[C2 - 1] & E[C2 - 2] & O[C2 - 2];
+            uint32_t los = lo1, his = hi1;
 #pragma unroll
-                    for (int t = 0; t < C2 - 1; ++t) { E[t] = E[t + 1]; O[t] = O[t + 1]; }
-                    E[C2 - 1] = te;
-                    O[C2 - 1] = to;
-                    i0 += 1;
-                    j0 -= 1;
+            for (int k = 1; k < NSH; ++k) {
+                los &= E[k + 1] & O[k];
+                his &= E[C2 - 2 - k] & O[C2 - 2 - k];
+            }
+            // bit 0: the lane's edge is live; 1, 2: one slot, NSH slots are free
+            int bot = (rel_live_lo(E[0]) ? 1 : 0) | (rel_live_lo(lo1) ? 0 : 2) |
+                      (rel_live_lo(los) ? 0 : 4);
+            int top = (need_up_l ? 1 : 0) | (rel_live_hi(hi1) ? 0 : 2) | (rel_live_hi(his) ? 0 : 4);
+            if constexpr (L > 1) {  // every lane takes part in every shuffle
+                bot = __shfl_sync(FULL, bot, 0, L);
+                top = __shfl_sync(FULL, top, L - 1, L);
+            }
+            const bool nu = go && (top & 1), nd = go && !(top & 1) && (bot & 1);
+            const int room = nu ? bot : top;  // of the opposite edge
+            ovf = (nu || nd) && !(room & 2);
+            const int by = (nu || nd) && !ovf ? ((room & 4) ? NSH : 1) : 0;
+            auto shift = [&](auto k_tag, auto up_tag) {  // groups that move by k slots
+                constexpr int K = decltype(k_tag)::value;
+                constexpr bool UP = decltype(up_tag)::value;
+                const bool mine = by == K && (UP ? nu : nd);
+                if (!__any_sync(FULL, mine)) return;
+                shift_slots<L, C2, K, UP>(E, mine, UP ? top_lane : bot_lane);
+                shift_slots<L, C2, K, UP>(O, mine, UP ? top_lane : bot_lane);
+                if (mine) {
+                    i0 += UP ? K : -K;
+                    j0 -= UP ? K : -K;
                 }
+            };
+            if constexpr (NSH > 1) {
+                shift(std::integral_constant<int, NSH>{}, T1{});
+                shift(std::integral_constant<int, NSH>{}, T0{});
             }
-            if (__any_sync(FULL, sd)) {
-                uint32_t pe = __shfl_up_sync(FULL, E[C2 - 1], 1, L);
-                uint32_t po = __shfl_up_sync(FULL, O[C2 - 1], 1, L);
-                if (bot_lane) { pe = kPruned; po = kPruned; }
-                if (sd) {
-                    const uint32_t te = prmt(pe, E[C2 - 1], 0x5432);
-                    const uint32_t to = prmt(po, O[C2 - 1], 0x5432);
-#pragma unroll
-                    for (int t = C2 - 1; t > 0; --t) { E[t] = E[t - 1]; O[t] = O[t - 1]; }
-                    E[0] = te;
-                    O[0] = to;
-                    i0 -= 1;
-                    j0 += 1;
-                }
-            }
-            if (su || sd) {
-                load_windows();
-            }
+            shift(std::integral_constant<int, 1>{}, T1{});
+            shift(std::integral_constant<int, 1>{}, T0{});
+            if (by > 0) load_windows();
             fin = fin || ovf;
         }
         if (fin) retire(ovf);
         const bool refill = la_n == 0;
         if (refill) {
-            LA = fwd16_u(pk, nw, sa0, dir, i0 + (WIDE ? 32 : 16));
-            LB = back16_u(pk, nw, sb0, dir, j0 + 16);
+            load_ahead();
             la_n = 16;
-        }
-        if constexpr (REL) {
-            if (refill && masked) {  // end what lives outside the rectangle
+            if (masked) {  // end what lives outside the rectangle
                 const int32_t lo = j0 - n, hi = m - i0;
 #pragma unroll
                 for (int t = 0; t < C2; ++t) {
@@ -744,51 +550,31 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
                     O[t] = keep_range<C2>(O[t], t, lo - 1, hi);  // one diagonal earlier
                 }
             }
-            // lift the pruned slots back up (lift_period)
-            if (refill) {
-                lift_n -= 16;
-                if (lift_n < 16) {
+            lift_n -= 16;
+            if (lift_n < 16) {  // before the next refill: lift the pruned slots
 #pragma unroll
-                    for (int t = 0; t < C2; ++t) {
-                        E[t] = __vmaxs2(E[t], kDead2);
-                        O[t] = __vmaxs2(O[t], kDead2);
-                    }
-                    lift_n = __reduce_min_sync(FULL, lift);
-                    la_n = min(16, lift_n);
+                for (int t = 0; t < C2; ++t) {
+                    E[t] = __vmaxs2(E[t], kDead2);
+                    O[t] = __vmaxs2(O[t], kDead2);
                 }
+                lift_n = __reduce_min_sync(FULL, lift);
+                la_n = min(16, lift_n);
             }
-        }
-        // Absolute frame: every live value of the pair is >= 16 thr of its odd diagonal:
-        // once that threshold reaches kR + match + 1, take kR off the frame
-        // (pruned halves stay 0; no half borrows).
-        if (!REL && active && rb) {
-            const uint32_t mr = pack2(kScale * kR);
-#pragma unroll
-            for (int t = 0; t < C2; ++t) {
-                E[t] = __vmaxu2(E[t], mr) - mr;
-                O[t] = __vmaxu2(O[t], mr) - mr;
-            }
-            Q -= kR;
         }
         if constexpr (Src::kCanAbort) {
             if (__any_sync(FULL, src.aborted())) return true;
         }
         if (__any_sync(FULL, !active && !exhausted) || !__any_sync(FULL, active)) return true;
-        if (!masked) {
+        // Masked pairs are dearer: look every 16 of them (with the refill)
+        // whether the unmasked copy is safe again.
+        if (!masked || refill) {
             refresh_budget();
-            return budget < 1;
+            if (masked ? budget >= 1 : budget < 1) return true;
         }
-        // Masked pairs are dearer: look again every 16 pairs (with the
-        // refill) and go back to the unmasked copy once it is safe.
-        if (refill) {
-            refresh_budget();
-            return budget >= 1;
-        }
+        ctr0 = ctr = masked ? la_n : min(la_n, budget);
         return false;
     };
 
-    using T0 = std::integral_constant<bool, false>;
-    using T1 = std::integral_constant<bool, true>;
     for (;;) {
         // A serving kernel can be told to leave at once (teardown).
         if constexpr (Src::kCanAbort) {
@@ -804,65 +590,55 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
                     exhausted = true;
                 } else if (r > 0) {
                     const Ext e = src.open(gj, task, sc);
-                    if (e.ok && !(REL ? relative_ok<S>(sc) : packed32_ok(sc))) {
+                    if (e.ok && !relative_ok<S>(sc)) {
                         // A scoring 16-bit cells cannot hold exactly (a serving
                         // request's own): hand the task to the next, 32-bit tier.
                         if (glane == 0) src.retire(gj, task, true, 0, 0, 0);
                     } else if (e.ok) {
-                        sa0 = e.A.s0;
-                        sb0 = e.B.s0;
+                        aw0 = (int32_t)(e.A.s0 >> 4);
+                        ab0 = (int32_t)(e.A.s0 & 15);
+                        bw0 = (int32_t)(e.B.s0 >> 4);
+                        bb0 = (int32_t)(e.B.s0 & 15);
                         dir = e.A.dir;
                         m = e.m;
                         n = e.n;
                         mn = m + n;
                         ng = -sc.gap;
-                        uint32_t orig;
-                        if constexpr (REL) {
-                            // origin (H = 0) at window slot W/2, x above the threshold
-                            orig = (uint32_t)sc.x * KS;
-                            const int32_t mm = sc.mismatch + 2 * ng, bonus = sc.match - sc.mismatch;
-                            const bool folds = subst_folds(sc);
-                            add_mi = !folds;
-                            rs.mi2 = folds ? 0u : pack2(mm * (int32_t)KS);
-                            const uint32_t c = folds ? (uint32_t)(2 * mm / bonus) * 0x10001u : 0u;
+                        const int32_t mm = sc.mismatch + 2 * ng;
+                        const int32_t bonus = sc.match - sc.mismatch;
+                        const bool folds = subst_folds(sc);
+                        add_mi = !folds;
+                        rs.mi2 = folds ? 0u : pack2(mm * (int32_t)KS);
+                        const uint32_t c = folds ? (uint32_t)(2 * mm / bonus) * 0x10001u : 0u;
 #pragma unroll
-                            for (int q = 0; q < 3; ++q) {
-                                rs.k[q] = (uint32_t)bonus * KS >> (1 + 2 * q);
-                                rs.c[q] = c << (2 * q);
-                            }
-                            ngp = (uint32_t)ng * (KS * 0x10001u);
-                            dA = dB = ngp;
-                            lift = lift_period<S>(sc);
-                        } else {
-                            kR = rebase_step16<S>(sc);
-                            kRL = kR + sc.match + 1;
-                            xup = (sc.x + 1) << VS;
-                            mi2 = pack2(kScale * (sc.mismatch + 2 * ng));
-                            k13 = (uint32_t)(kScale * (sc.match - sc.mismatch)) << 19;
-                            k15 = (uint32_t)(kScale * (sc.match - sc.mismatch)) << 17;
-                            // origin (H = 0) at window slot W/2, stored as
-                            // 16 * (x + beta), beta = match + |gap| + 1
-                            Q = sc.match + ng + 1;
-                            orig = (uint32_t)(kScale * (sc.x + Q));
+                        for (int q = 0; q < 3; ++q) {
+                            rs.k[q] = (uint32_t)bonus * KS >> (1 + 2 * q);
+                            rs.c[q] = c << (2 * q);
                         }
+                        ngp = (uint32_t)ng * (KS * 0x10001u);
+                        dA = dB = ngp;
+                        sA = sB = ng;
+                        lift = lift_period<S>(sc);
+                        // origin (H = 0, x above the threshold) at window slot W/2
 #pragma unroll
                         for (int t = 0; t < C2; ++t) {
                             const int slo = glane * S + t, shi = slo + C2;
-                            const uint32_t lo = (slo == W / 2) ? orig : (kPruned & 0xFFFFu);
-                            const uint32_t hi = (shi == W / 2) ? orig : (kPruned >> 16);
-                            E[t] = lo | (hi << 16);
-                            O[t] = kPruned;
+                            const uint32_t orig = (uint32_t)sc.x * KS, dead = kDead2 & 0xFFFFu;
+                            E[t] = (slo == W / 2 ? orig : dead) |
+                                   ((shi == W / 2 ? orig : dead) << 16);
+                            O[t] = kDead2;
                         }
                         i0 = -(W / 2) + glane * S;
                         j0 = (W / 2) - glane * S;
                         load_windows();
                         d = 0;
                         T = 0;
-                        bi = 0;
-                        bj = 0;
                         bd = 0;
-                        prev_dead = false;
+                        ptop = 0;
                         active = true;
+                        tmask = top_lane ? 0x80000000u : 0u;
+                        bmask = bot_lane ? 0x00008000u : 0u;
+                        amask = 0x80000000u;
                     }
                 }
             }
@@ -873,41 +649,41 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
             continue;
         }
         refresh_budget();
-        if constexpr (REL) {
-            generic = __any_sync(FULL, add_mi);
-            lift_n = min(lift_n, __reduce_min_sync(FULL, lift));
-            la_n = min(la_n, lift_n);
-        }
-        if (budget >= 1) {
-            if (REL && generic) {
-                for (;;) {
-                    if (pair(T0{}, T1{}) && handle(false)) break;
-                }
-            } else {
-                for (;;) {  // no cell of any window can leave its rectangle
-                    if (pair(T0{}, T0{}) && handle(false)) break;
-                }
-            }
-        } else {
+        lift_n = min(lift_n, __reduce_min_sync(FULL, lift));
+        la_n = min(la_n, lift_n);
+        // a group that still waits for a task asks again after every pair
+        const bool waits = __any_sync(FULL, !active && !exhausted);
+        ctr0 = ctr = waits ? 1 : budget >= 1 ? min(la_n, budget) : la_n;
+        if (budget < 1) {
             for (;;) {
                 if (pair(T1{}, T1{}) && handle(true)) break;
+            }
+        } else if (__any_sync(FULL, add_mi)) {
+            for (;;) {
+                if (pair(T0{}, T1{}) && handle(false)) break;
+            }
+        } else {
+            for (;;) {  // no cell of any window can leave its rectangle
+                if (pair(T0{}, T0{}) && handle(false)) break;
             }
         }
     }
 }
 
 // Batched form of the packed kernel (same task source as lockstep_kernel).
-// 128-thread blocks: the loop holds about 96 registers with 16 slots per
-// lane (five such blocks fit an SM, 20 warps) and 128 with 32 (four blocks),
-// and that measured faster than capping the registers for more warps.
-constexpr int kPackedThreads = 128;
-template <int L, int C2, bool REL = true>
-__global__ void __launch_bounds__(kPackedThreads)
+// Blocks of 128 threads.  The registers are capped for 3 blocks per SM with 32
+// or 64 slots per lane, 4 with 16 and 5 with fewer: more warps at fewer
+// registers measured slower (29x, x = 50, first tier: 2x32 at 3, 4 and 5
+// blocks 45.8, 46.0 and 48.8 ms; 4x16 at 4, 5 and 6 blocks 52.0, 54.2 and 57.7).
+template <int C2>
+__host__ __device__ constexpr int packed_min_blocks() { return C2 >= 16 ? 3 : C2 == 8 ? 4 : 5; }
+template <int L, int C2>
+__global__ void __launch_bounds__(kPackedThreads, packed_min_blocks<C2>())
 lockstep16_kernel(const Job *jp, const uint32_t *order, const uint32_t *n_tasks_ptr,
                   uint32_t *counter, Spill spill, uint32_t one)
 {
     BatchSrc src{jp, order, *n_tasks_ptr, counter, spill};
-    lockstep16_loop<L, C2, REL>(src, jp->packed, jp->n_words, one);
+    lockstep16_loop<L, C2>(src, jp->packed, jp->n_words, one);
 }
 
 }  // namespace xd

@@ -563,7 +563,7 @@ template <int L1, int C2a, int L2, int C2>
 __global__ void __launch_bounds__(256, 2)
 serve16_kernel(ServeArgs a, const uint32_t *pk, int64_t nw)
 {
-    serve_warp(a, [&](RingSrc &src) { lockstep16_loop<L1, C2a, true>(src, pk, nw, a.one); },
+    serve_warp(a, [&](RingSrc &src) { lockstep16_loop<L1, C2a>(src, pk, nw, a.one); },
                [&](SpillSrc &src) { lockstep_loop<L2, C2>(src, pk, nw); });
 }
 

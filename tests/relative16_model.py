@@ -1,8 +1,8 @@
 """Bit-level CPU model of the packed band kernel's relative frame (test infrastructure).
 
 Restates, in plain Python integers, the arithmetic of ``lockstep16_loop`` in
-``paper_2309_07270_gb300/csrc/xd_lockstep16.cuh`` for one group of lanes when
-the cells are kept relative to each diagonal's X-drop threshold (``REL``):
+``paper_2309_07270_gb300/csrc/xd_lockstep16.cuh`` for one group of lanes, with
+the cells kept relative to each diagonal's X-drop threshold:
 the substitution folded into one multiply-add, signed three-way maxima, the
 prune by an unsigned add-and-minimum, the plain slot keys, the lift of
 pruned slots and the window shifts.  Every add is checked: a half that
@@ -10,15 +10,24 @@ carries into the other one, or leaves the signed 16-bit range where the
 kernel compares signed, raises Wrap.  Any change to the kernel's arithmetic
 must be made here too.
 """
-from packed16_model import Wrap, fits, key_scale, mk, pack2, prmt, s16, slot_bits, uhalves, umk
+from packed16_model import Wrap, fits, mk, pack2, prmt, s16, uhalves, umk
 
 DEAD = 0xC000
 DEAD2 = 0xC000C000
 
 
+def key_scale(slots):
+    return max(slots, 16)
+
+
+def slot_bits(slots):
+    return {16: 4, 32: 5, 64: 6}[key_scale(slots)]
+
+
 def relative_ok(match, mismatch, gap, x, slots):
     return (fits(match, mismatch, gap, x)
-            and (x + 2 * match - 2 * gap + 1) * key_scale(slots) <= 0x8000)
+            and (x + 2 * match - 2 * gap + 1) * key_scale(slots) <= 0x8000
+            and (slots < 64 or match - gap <= 64))
 
 
 def subst_folds(match, mismatch, gap):
@@ -60,16 +69,16 @@ def addmin_u(a, b, c):
 
 def flags(eqs, t, C2):
     """Register t's flag word and the bit of its low flag (rel_pos)."""
-    eq7, eqh = eqs[0], eqs[-1]
     if C2 == 2:
-        e = (eq7 & 0xF) | (eq7 << 12 & 0xFFFFFFFF)
+        e = (eqs[0] & 0xF) | (eqs[0] << 12 & 0xFFFFFFFF)
     elif C2 == 4:
-        e = prmt(eq7, eq7, 0x2100)
+        e = prmt(eqs[0], eqs[0], 0x2100)
     elif C2 == 8:
-        e = eq7
+        e = eqs[0]
     else:
-        e = prmt(eq7, eqh, 0x5410) if t < 8 else prmt(eq7, eqh, 0x7632)
-    G = 3 if C2 == 16 else 2
+        h = t // 8
+        e = prmt(eqs[h // 2], eqs[len(eqs) // 2 + h // 2], 0x7632 if h & 1 else 0x5410)
+    G = 3 if C2 >= 16 else 2
     q = (t % 8) % G
     return e >> (2 * G * ((t % 8) // G)), q
 
@@ -81,7 +90,9 @@ def extend(a, b, match, mismatch, gap, x, lanes=2, regs=16, stats=None):
         stats.setdefault(k, 0)
     C2, S = regs, 2 * regs
     KS, SB = key_scale(S), slot_bits(S)
+    VS = SB if lanes == 1 else SB + 5
     W, m, n, ng = lanes * S, len(a), len(b), -gap
+    NSH = max(min(S // 4, W // 8), 1)
     assert relative_ok(match, mismatch, gap, x, S)
     mm, bonus = mismatch + 2 * ng, match - mismatch
     folds = subst_folds(match, mismatch, gap)
@@ -156,21 +167,22 @@ def extend(a, b, match, mismatch, gap, x, lanes=2, regs=16, stats=None):
                 v = addmin_u(r, nstep, DEAD2)
                 row.append(v)
                 idx = (S - 1 - t) | ((S - 1 - (t + C2)) << 16)
-                key = add(v, idx)
+                key = add(r, idx)
                 lane = max(lane, s16(key), s16(key >> 16))
             newV.append(row)
             mask = (1 << SB) - 1
-            mkey = 32 * lane - 31 * (lane & mask) + ((31 - g) << SB)
-            assert mkey >> (SB + 5) == lane >> SB
+            mkey = lane if lanes == 1 else 32 * lane - 31 * (lane & mask) + ((31 - g) << SB)
+            assert mkey >> VS == lane >> SB
             group = mkey if group is None else max(group, mkey)
         for g in range(lanes):
             V[g][:] = newV[g]
-        rise = max((group >> (SB + 5)) - x, 0)
+        above = (group >> VS) - (st["dA"] + st["dB"])
+        rise = max(above - x, 0)
         st["T"] += rise
         st["dA"], st["dB"] = st["dB"], ng + rise
         if rise:
             st["best"] = (group, i0[0], st["d"])
-        return group
+        return above
 
     def shift(up):
         for X in (E, O):
@@ -205,17 +217,26 @@ def extend(a, b, match, mismatch, gap, x, lanes=2, regs=16, stats=None):
             if st["best"] is None:
                 return st["T"], 0, 0, False
             key, ibase, bd = st["best"]
-            bi = ibase + (31 - ((key >> SB) & 31)) * S + (S - 1 - (key & ((1 << SB) - 1)))
+            bi = ibase + S - 1 - (key & ((1 << SB) - 1))
+            bi += 0 if lanes == 1 else (31 - ((key >> SB) & 31)) * S
             return st["T"], bi, bd - bi, False
         need_up = hi_live(E[top][C2 - 1]) or hi_live(O[top][C2 - 1])
         need_dn = lo_live(E[0][0])
-        blk_up = lo_live(E[0][0]) or lo_live(E[0][1]) or lo_live(O[0][0])
-        blk_dn = need_up or hi_live(E[top][C2 - 2]) or hi_live(O[top][C2 - 2])
-        if (need_up and blk_up) or (need_dn and not need_up and blk_dn):
-            return st["T"], 0, 0, True
+
+        def free_bottom(k):
+            return not any(lo_live(E[0][q]) for q in range(k + 1)) and \
+                not any(lo_live(O[0][q]) for q in range(k))
+
+        def free_top(k):
+            return not any(hi_live(X[top][C2 - 1 - q]) for X in (E, O) for q in range(k + 1))
         if need_up or need_dn:
-            stats["up" if need_up else "down"] += 1
-            shift(need_up)
+            free = free_bottom if need_up else free_top
+            if not free(1):
+                return st["T"], 0, 0, True
+            by = NSH if free(NSH) else 1
+            stats["up" if need_up else "down"] += by
+            for _ in range(by):
+                shift(need_up)
             budget = margin()
         refill -= 1
         if refill == 0:

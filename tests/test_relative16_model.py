@@ -22,7 +22,7 @@ SCORINGS = [
     (1, -1, -1, 50), (1, 0, -1, 20), (2, -3, -2, 30), (1, -2, -1, 100),
     (64, -128, -64, 1472), (64, -128, -64, 767),  # largest of 16- and of 32-slot lanes
     (3, -2, -125, 100), (127, -1, -1, 1409), (127, -1, -1, 767),
-    (1, -2, -1, 1535), (1, -2, -1, 1019), (7, -1, -2, 0), (4, -4, -3, 40),
+    (1, -2, -1, 1535), (1, -2, -1, 1019), (1, -2, -1, 507), (32, -64, -32, 383), (7, -1, -2, 0), (4, -4, -3, 40),
 ]
 
 
@@ -36,7 +36,7 @@ def cases(seed, n, slots):
         yield scorings[(k // 3) % len(scorings)], t[:la], b[:lb]
 
 
-@pytest.mark.parametrize("lanes,regs", [(4, 4), (4, 8), (2, 16), (4, 16), (8, 2)])
+@pytest.mark.parametrize("lanes,regs", [(4, 4), (4, 8), (2, 16), (4, 16), (32, 2), (1, 16), (1, 32), (2, 32)])
 def test_model_matches_oracle(orc, lanes, regs):
     done = 0
     for sc, a, b in cases(lanes * regs, 42, 2 * regs):
@@ -59,7 +59,7 @@ def test_long_reads_sink_and_lift_pruned_slots(orc, lanes, regs, sc):
     assert st["lift"] >= 1500 // R.lift_period(sc[0], sc[2], 2 * regs) - 1
 
 
-@pytest.mark.parametrize("lanes,regs", [(4, 8), (2, 16), (16, 2)])
+@pytest.mark.parametrize("lanes,regs", [(4, 8), (2, 16), (1, 32), (16, 2)])
 def test_drifting_band_shifts_the_window(orc, lanes, regs):
     rng = np.random.default_rng(17)
     t = rng.integers(0, 4, 480).astype(np.uint8)
@@ -78,13 +78,13 @@ int main(void)
 {
     const int match[] = {1, 2, 3, 7, 64, 127, 128}, gap[] = {-1, -2, -3, -64, -127, -128};
     const int mis[] = {0, -1, -2, -3, -4, -127, -128, -129};
-    const int x[] = {0, 1, 50, 765, 766, 767, 1017, 1018, 1019, 1020, 1535, 1536};
+    const int x[] = {0, 1, 50, 505, 506, 507, 765, 766, 767, 1017, 1018, 1019, 1020, 1535, 1536};
     for (int a : match) for (int g : gap) for (int b : mis) for (int c : x) {
         const xd::Scoring sc{a, b, g, c};
         if (!xd::packed16_ok(sc)) continue;
-        printf("%d %d %d %d %d %d %d %d %d\n", a, b, g, c, (int)xd::relative_ok<16>(sc),
-               (int)xd::relative_ok<32>(sc), (int)xd::subst_folds(sc), xd::lift_period<16>(sc),
-               xd::lift_period<32>(sc));
+        printf("%d %d %d %d %d %d %d %d %d %d\n", a, b, g, c, (int)xd::relative_ok<16>(sc),
+               (int)xd::relative_ok<32>(sc), (int)xd::relative_ok<64>(sc),
+               (int)xd::subst_folds(sc), xd::lift_period<16>(sc), xd::lift_period<32>(sc));
     }
     return 0;
 }
@@ -102,11 +102,12 @@ def test_kernel_rules_equal_the_model(tmp_path):
                     os.path.join(ROOT, "include"), "-o", str(exe), str(src)], check=True)
     rows = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout
     n = 0
-    for m, mis, g, x, ok16, ok32, folds, p16, p32 in (map(int, r.split()) for r in
+    for m, mis, g, x, ok16, ok32, ok64, folds, p16, p32 in (map(int, r.split()) for r in
                                                       rows.splitlines()):
         assert bool(ok16) == R.relative_ok(m, mis, g, x, 16) and ok16  # every packed scoring
         assert bool(ok32) == R.relative_ok(m, mis, g, x, 32)
         assert not ok32 or P.fits(m, mis, g, x, 32)
+        assert bool(ok64) == R.relative_ok(m, mis, g, x, 64)
         assert bool(folds) == R.subst_folds(m, mis, g)
         assert (p16, p32) == (R.lift_period(m, g, 16), R.lift_period(m, g, 32))
         n += 1
