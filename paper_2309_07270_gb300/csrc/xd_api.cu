@@ -70,9 +70,9 @@ enum : int {
     C_OFFS = 32,         // NBINS
     C_NVALID = 64,
     C_COUNTER = 65,
-    C_SPILL0 = 66,       // spill counts of tiers 0..2
-    C_SPILL1 = 67,
-    C_SPILL2 = 68,
+    C_SPILL0 = 66,       // extensions the first tier handed on
+    C_SPILL1 = 67,       // extensions for the unbounded tier
+    C_WARP = 68,         // work counter of the warp kernel
     C_NBAD = 69,
     C_MAXLEN = 70,
     C_WORDS = 72
@@ -113,7 +113,7 @@ struct xdrop_ctx {
 
     Job *d_job = nullptr;
     uint32_t *d_ctrs = nullptr;
-    DevBuf order, spill[3], wide;
+    DevBuf order, spill[2], wide;
     DevBuf plain_ctl;  // plain mode: task count and work counter per sub-batch
     size_t cap_tasks = 0;
     int64_t wide_per_cta = 0;
@@ -192,8 +192,7 @@ int ensure_scratch(xdrop_ctx *c, size_t n_tasks, uint32_t maxlen)
     if ((rc = dev_alloc(c, c->order, tasks * 4))) return rc;
     for (auto &s : c->spill)
         if ((rc = dev_alloc(c, s, tasks * 4))) return rc;
-    c->cap_tasks = std::min(c->order.cap, std::min(c->spill[0].cap,
-                            std::min(c->spill[1].cap, c->spill[2].cap))) / 4;
+    c->cap_tasks = std::min(c->order.cap, std::min(c->spill[0].cap, c->spill[1].cap)) / 4;
     int64_t per = (int64_t)3 * ((int64_t)maxlen + 1);
     per = (per + 63) / 64 * 64;
     if (per > c->wide_per_cta) {
@@ -221,15 +220,16 @@ Spill spill_of(xdrop_ctx *c, int k)
     return Spill{(uint32_t *)c->spill[k].p, c->d_ctrs + C_SPILL0 + k};
 }
 
-Tile next_tile_after(Tile t)
+// The tiers after a first tier of width w: a warp per extension (windows of
+// 128 slots unless the first tier had them, then 512), then the unbounded
+// tier.
+int enqueue_wider(xdrop_ctx *c, int w, uint64_t n_tasks)
 {
-    // The 128-wide tile for narrower first tiers, then 512.  Its overflow
-    // tier is 32 lanes x 4 cells: the few extensions that reach it run one
-    // per warp, and with half the cells per lane a diagonal takes half as
-    // long, so the tier (which ends when its longest extension does) is
-    // shorter than with 16 lanes x 8 cells.
-    if (t.width() < 128) return Tile{32, 4};
-    return Tile{32, 16};
+    CK(launch_warp(n_tasks, c->sm_count, c->d_job, spill_of(c, 0).list, spill_of(c, 0).count,
+                   c->d_ctrs + C_WARP, w >= 128, nullptr, Spill{}, spill_of(c, 1), c->stream));
+    CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
+                   c->wide_per_cta, c->stream));
+    return XDROP_OK;
 }
 
 // Enqueue the batched launch sequence (graph body) with first tile t0.
@@ -247,21 +247,8 @@ int enqueue_batched(xdrop_ctx *c, Tile t0, int bps, bool main_events, uint32_t *
     CK(launch_persistent(t0, c->sm_count * bps, c->d_job, (uint32_t *)c->order.p,
                          ctr + C_NVALID, ctr + C_COUNTER, spill_of(c, 0), s));
     if (main_events) CK(cudaEventRecordWithFlags(c->ev_main1, s, cudaEventRecordExternal));
-    int n = 4;
-    Tile t1 = next_tile_after(t0);
-    int k = 0;
-    if (t1.width() < 512) {
-        CK(launch_spill(t1, false, c->sm_count * 4, c->d_job, spill_of(c, 0), spill_of(c, 1), s));
-        k = 1;
-        ++n;
-    }
-    CK(launch_spill(Tile{32, 16}, false, c->sm_count * 2, c->d_job, spill_of(c, k),
-                    spill_of(c, k + 1), s));
-    CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, k + 1), (int32_t *)c->wide.p,
-                   c->wide_per_cta, s));
-    n += 2;
-    if (launches) *launches = n;
-    return XDROP_OK;
+    if (launches) *launches = 6;
+    return enqueue_wider(c, t0.width(), c->cap_tasks);
 }
 
 // Candidate first tiles for autotuning (all persistent instantiations);
@@ -459,17 +446,29 @@ int run_plain(xdrop_ctx *c, Ticket *tk, const Job &job)
         CK(launch_persistent(t0, grid, c->d_job, order + 2 * p0, ctl + 2 * k, ctl + 2 * k + 1,
                              spill_of(c, 0), s));
     }
-    tk->launches += (uint32_t)(1 + n_sub);
-    Tile t1 = next_tile_after(t0);
-    int k = 0;
-    if (t1.width() < 512) {
-        CK(launch_spill(t1, false, c->sm_count * 4, c->d_job, spill_of(c, 0), spill_of(c, 1), s));
-        k = 1;
-        tk->launches += 1;
-    }
-    CK(launch_spill(Tile{32, 16}, false, c->sm_count * 2, c->d_job, spill_of(c, k),
-                    spill_of(c, k + 1), s));
-    CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, k + 1), (int32_t *)c->wide.p,
+    tk->launches += (uint32_t)(3 + n_sub);
+    return enqueue_wider(c, t0.width(), 2 * n_pairs);
+}
+
+// A batch of few tasks (at most kWarpTasksPerSm per SM): every extension has a
+// warp of its own from the start, with no order, tuning or graph.
+// Such a batch lasts as long as its longest extension, and the warp kernel
+// has the shortest diagonal.
+constexpr uint64_t kWarpTasksPerSm = 8;
+bool is_small(const xdrop_ctx *c, uint64_t n_pairs)
+{
+    return c->mode != XDROP_MODE_PLAIN && !c->forced.lanes && 2 * n_pairs <= kWarpTasksPerSm * c->sm_count;
+}
+
+int run_small(xdrop_ctx *c, Ticket *tk, const Job &job)
+{
+    cudaStream_t s = c->stream;
+    c->tile0 = Tile{32, 4, warp_packed(job.sc)};
+    CK(cudaMemsetAsync(c->d_ctrs, 0, C_MAXLEN * 4, s));
+    CK(launch_warp(2 * job.n_pairs, c->sm_count, c->d_job, nullptr, nullptr, c->d_ctrs + C_WARP, false,
+                   tk->device_submit ? c->d_ctrs + C_NBAD : nullptr, spill_of(c, 0),
+                   spill_of(c, 1), s));
+    CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
                    c->wide_per_cta, s));
     tk->launches += 2;
     return XDROP_OK;
@@ -497,18 +496,20 @@ int launch_ticket(xdrop_ctx *c, Ticket *tk, const Job &job, uint32_t maxlen)
     *tk->h_job = job;
     CK(cudaMemcpyAsync(c->d_job, tk->h_job, sizeof(Job), cudaMemcpyHostToDevice, s));
     CK(cudaEventRecord(tk->ev_begin, s));
+    const bool small = job.n_pairs && is_small(c, job.n_pairs);
     // the tile first: autotuning uses the result buffer as scratch, and
     // validation then writes every status word
-    if (job.n_pairs && c->mode != XDROP_MODE_PLAIN) {
+    if (job.n_pairs && c->mode != XDROP_MODE_PLAIN && !small) {
         if ((rc = pick_tile(c, tk, job, &c->tile0))) return rc;
     }
-    if (tk->device_submit) {
+    if (tk->device_submit && !small) {
         CK(cudaMemsetAsync(c->d_ctrs + C_NBAD, 0, 4, s));
         CK(launch_validate(c->d_job, job.n_pairs, c->d_ctrs + C_NBAD, s));
         tk->launches += 1;
     }
     if (job.n_pairs) {
-        if (c->mode == XDROP_MODE_PLAIN) rc = run_plain(c, tk, job);
+        if (small) rc = run_small(c, tk, job);
+        else if (c->mode == XDROP_MODE_PLAIN) rc = run_plain(c, tk, job);
         else rc = run_batched(c, tk);
         if (rc) return rc;
     }
@@ -813,8 +814,7 @@ int xdrop_sync(xdrop_ctx *c, xdrop_ticket t, int64_t timeout_ns)
     st.main_kernel_ms = ms_main;
     st.tasks = 2 * (uint64_t)tk->n_pairs;
     st.overflow_tasks = tk->h_ctrs[C_SPILL0];
-    st.wide_tasks = next_tile_after(c->tile0).width() >= 512 ? tk->h_ctrs[C_SPILL1]
-                                                              : tk->h_ctrs[C_SPILL2];
+    st.wide_tasks = tk->h_ctrs[C_SPILL1];
     st.launches = tk->launches;
     st.graph_replays = tk->graph_replays;
     st.tile_lanes = c->tile0.lanes;
@@ -964,10 +964,10 @@ int xdrop_submit_pairs(xdrop_ctx *c, const xdrop_pair *pairs, size_t n_pairs,
     // chunks when the pair table does not fit the device memory budget
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
-    const size_t per_pair = sizeof(xdrop_pair) + sizeof(xdrop_result) + 2 * 4 * 4;  // + task scratch
+    const size_t per_pair = sizeof(xdrop_pair) + sizeof(xdrop_result) + 2 * 3 * 4;  // + task scratch
     size_t chunk = std::max<size_t>(n_pairs, 1);
     if (c->budget && c->mode != XDROP_MODE_PLAIN) {
-        const size_t scratch_now = c->order.cap + c->spill[0].cap + c->spill[1].cap + c->spill[2].cap;
+        const size_t scratch_now = c->order.cap + c->spill[0].cap + c->spill[1].cap;
         const size_t fixed = c->used - scratch_now + 4 * kAlign;
         if (c->budget <= fixed + 1024 * per_pair)
             return fail(c->tickets.empty() ? XDROP_ENOMEM : XDROP_EBUSY,
@@ -978,7 +978,7 @@ int xdrop_submit_pairs(xdrop_ctx *c, const xdrop_pair *pairs, size_t n_pairs,
         if (fit < chunk) {
             chunk = fit;
             // scratch sized for this chunk must not stay larger from before
-            for (DevBuf *b : {&c->order, &c->spill[0], &c->spill[1], &c->spill[2]}) {
+            for (DevBuf *b : {&c->order, &c->spill[0], &c->spill[1]}) {
                 if (b->cap > 2 * chunk * 4) {
                     CK(cudaStreamSynchronize(c->stream));
                     cudaFree(b->p);

@@ -364,43 +364,8 @@ window_kernel(const Job *jp, uint32_t task_base, uint32_t n_tasks, Spill spill)
     }
 }
 
-// Persistent form: groups pull positions of `order` from a global counter
-// until *n_tasks_ptr is reached (order is longest-first in batched mode).
-template <int LANES, int C>
-__global__ void __launch_bounds__(256)
-window_persistent_kernel(const Job *jp, const uint32_t *order, const uint32_t *n_tasks_ptr,
-                         uint32_t *counter, Spill spill)
-{
-    const Job J = *jp;
-    const int lane = threadIdx.x & 31;
-    const int glane = lane % LANES;
-    const int gbase = lane - glane;
-    const unsigned gm = group_mask<LANES>(gbase);
-    const uint32_t n_tasks = *n_tasks_ptr;
-    for (;;) {
-        uint32_t q = 0;
-        if (glane == 0) q = atomicAdd(counter, 1u);
-        q = __shfl_sync(gm, q, gbase);
-        if (q >= n_tasks) break;
-        const uint32_t task = order ? order[q] : q;
-        Ext e = decode(J, task);
-        if (!e.ok) continue;
-        int32_t sc, bi, bj;
-        int64_t cells;
-        int st = extend_window<LANES, C, false>(e, J.sc, glane, gbase, sc, bi, bj, cells);
-        if (glane == 0) {
-            if (st) {
-                uint32_t s = atomicAdd(spill.count, 1u);
-                spill.list[s] = task;
-            } else {
-                write_result(J, e, sc, bi, bj);
-            }
-        }
-    }
-}
-
 // Window kernels take their task list from a spill of the previous tier.
-template <int LANES, int C, bool COUNT>
+template <int LANES, int C>
 __global__ void __launch_bounds__(256)
 window_spill_kernel(const Job *jp, Spill in, Spill out)
 {
@@ -417,13 +382,11 @@ window_spill_kernel(const Job *jp, Spill in, Spill out)
         if (!e.ok) continue;
         int32_t sc, bi, bj;
         int64_t cells;
-        int st = extend_window<LANES, C, COUNT>(e, J.sc, glane, gbase, sc, bi, bj, cells);
+        int st = extend_window<LANES, C, false>(e, J.sc, glane, gbase, sc, bi, bj, cells);
         if (glane == 0) {
             if (st) {
                 uint32_t s = atomicAdd(out.count, 1u);
                 out.list[s] = task;
-            } else if (COUNT) {
-                J.cells[task] = cells;
             } else {
                 write_result(J, e, sc, bi, bj);
             }

@@ -36,9 +36,16 @@ cudaError_t launch_window(Tile t, bool count, const Job *jp, uint32_t task_base,
 cudaError_t launch_persistent(Tile t, int grid, const Job *jp, const uint32_t *order,
                               const uint32_t *n_tasks, uint32_t *counter, Spill spill,
                               cudaStream_t s);
-// Tasks listed in `in`, overflow to `out`.
-cudaError_t launch_spill(Tile t, bool count, int grid, const Job *jp, Spill in, Spill out,
-                         cudaStream_t s);
+// Tasks listed in `in` on windows of 512 slots, overflow to `out`.
+cudaError_t launch_spill_512(int grid, const Job *jp, Spill in, Spill out, cudaStream_t s);
+// A warp per task (xd_warp16.cuh): the tasks of a list (n_tasks bounds their
+// number *n_ptr) or, without one, all tasks of the job; windows of 128 slots
+// (unless skip128), then 512, overflow to `out`.  Without a list: tasks that
+// outgrew 128 slots are also noted in `over`, and n_bad asks for the pairs'
+// status.
+cudaError_t launch_warp(uint64_t n_tasks, int sm_count, const Job *jp, const uint32_t *list,
+                        const uint32_t *n_ptr, uint32_t *counter, bool skip128, uint32_t *n_bad,
+                        Spill over, Spill out, cudaStream_t s);
 // Blocks per SM of a persistent tile at 256 threads per block.
 int persistent_block_threads(Tile t);  // threads per block of the persistent first tier
 int persistent_blocks_per_sm(Tile t);
@@ -51,6 +58,8 @@ bool packed_tile_ok(Tile t, const Scoring &sc);
 // packed 16-slot tile of the same width, else a 32-bit tile of its width.
 Tile usable_tile(Tile t, const Scoring &sc);
 
+// Whether the warp kernel runs this scoring on packed cells.
+bool warp_packed(const Scoring &sc);
 // The tile with the frame its cells need for this scoring (packed tiles).
 Tile in_frame(Tile t, const Scoring &sc);
 

@@ -14,15 +14,7 @@ __global__ void validate_kernel(const Job *jp, uint32_t *n_bad)
     for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < J.n_pairs;
          p += (uint64_t)gridDim.x * blockDim.x) {
         const Pair pr = J.pairs[p];
-        const bool ok = job_pair_ok(J, pr);
-        int32_t *o = J.out + p * 7;
-        if (!ok) {
-            for (int k = 0; k < 6; ++k) o[k] = 0;
-            o[6] = 1;
-            atomicAdd(n_bad, 1u);
-        } else {
-            o[6] = 0;
-        }
+        write_status(J, p, job_pair_ok(J, pr), n_bad);
     }
 }
 

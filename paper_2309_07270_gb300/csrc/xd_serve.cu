@@ -377,7 +377,7 @@ void Server::handle_spills(std::vector<Req *> &sp)
         Spill in{(uint32_t *)(d + r->d_spill), ctr + 1};
         Spill out{(uint32_t *)(d + r->d_spill2), ctr + 2};
         if (e == cudaSuccess)
-            e = launch_spill(Tile{32, 16}, false, 2 * sm_count, d_jobs + r->slot, in, out, s_side);
+            e = launch_spill_512(2 * sm_count, d_jobs + r->slot, in, out, s_side);
         if (e == cudaSuccess)
             e = launch_wide(false, wide_grid, d_jobs + r->slot, out, wide_scratch, wide_per_cta, s_side);
         if (e == cudaSuccess) {

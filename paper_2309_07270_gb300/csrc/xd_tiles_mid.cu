@@ -42,14 +42,6 @@ int occupancy_mid(Tile t)
     return -1;
 }
 
-cudaError_t launch_spill_mid(int grid, const Job *jp, Spill in, Spill out, cudaStream_t s)
-{
-    (void)cudaGetLastError();
-    window_spill_kernel<32, 4, false><<<grid, 256, 0, s>>>(jp, in, out);
-    return cudaGetLastError();
-}
-
-
 template <int L1, int C1, int L2, int C2>
 static cudaError_t serve_impl(int grid, const ServeArgs &a, const uint32_t *pk, int64_t nw,
                               cudaStream_t s)

@@ -6,12 +6,10 @@
 
 namespace xd {
 
-cudaError_t launch_spill_512(bool count, int grid, const Job *jp, Spill in, Spill out,
-                             cudaStream_t s)
+cudaError_t launch_spill_512(int grid, const Job *jp, Spill in, Spill out, cudaStream_t s)
 {
     (void)cudaGetLastError();
-    if (count) window_spill_kernel<32, 16, true><<<grid, 256, 0, s>>>(jp, in, out);
-    else window_spill_kernel<32, 16, false><<<grid, 256, 0, s>>>(jp, in, out);
+    window_spill_kernel<32, 16><<<grid, 256, 0, s>>>(jp, in, out);
     return cudaGetLastError();
 }
 
@@ -135,7 +133,6 @@ int occupancy_packed(Tile);
 cudaError_t launch_serve_packed(Tile, int, const ServeArgs &, const uint32_t *, int64_t,
                                 cudaStream_t, bool *);
 int serve_occupancy_packed(Tile);
-cudaError_t launch_spill_mid(int, const Job *, Spill, Spill, cudaStream_t);
 
 cudaError_t launch_serve_narrow(Tile, int, const ServeArgs &, const uint32_t *, int64_t,
                                 cudaStream_t, bool *);
@@ -207,14 +204,6 @@ int persistent_blocks_per_sm(Tile t)
     int b = occupancy_narrow(t);
     if (b < 0) b = occupancy_mid(t);
     return b;
-}
-
-cudaError_t launch_spill(Tile t, bool count, int grid, const Job *jp, Spill in, Spill out,
-                         cudaStream_t s)
-{
-    if (t.lanes == 32 && t.c == 16) return launch_spill_512(count, grid, jp, in, out, s);
-    if (!count && t.lanes == 32 && t.c == 4) return launch_spill_mid(grid, jp, in, out, s);
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace xd

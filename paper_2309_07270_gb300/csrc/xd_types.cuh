@@ -166,4 +166,16 @@ __device__ __forceinline__ void write_result(const Job &J, const Ext &e,
     }
 }
 
+// Status of a pair of a device submit: zero scores for a pair that fails
+// the limits.
+__device__ __forceinline__ void write_status(const Job &J, uint64_t pair, bool ok, uint32_t *n_bad)
+{
+    int32_t *o = J.out + pair * 7;
+    if (!ok) {
+        for (int k = 0; k < 6; ++k) o[k] = 0;
+        atomicAdd(n_bad, 1u);
+    }
+    o[6] = ok ? 0 : 1;
+}
+
 }  // namespace xd
