@@ -414,9 +414,11 @@ int xdrop_count_cells_device(xdrop_ctx *c, const uint32_t *packed,
  * on a device also loads the library's device code there, so make that
  * first call before any stream capture that should contain later calls.
  * All calls on a device share the array: calls whose work may overlap on
- * the GPU race and must be ordered (same stream, or events).  Every extension runs on the
- * unbounded-band tier (one CTA per extension), which is exact for any band
- * but slower than the batched path.
+ * the GPU race and must be ordered (same stream, or events).  Every
+ * extension has a warp of its own (windows of 128, then 512 slots); wider
+ * bands run on the unbounded tier (one CTA per extension).  While the call's
+ * work runs, a pair's status may hold further bits; they are clear once it
+ * is done.
  *
  * max_read_len must bound every read length; it sizes the per-CTA scratch
  * (3*(max_read_len+1) int32 per extension) and values above 2,796,202

@@ -1,5 +1,6 @@
-// Allocation-free entry point: the unbounded-band tier with its scratch in
-// a file-scope device array instead of memory from cudaMalloc.
+// Allocation-free entry point: a warp per extension with its band in
+// registers, and for bands wider than 512 slots the unbounded tier with its
+// scratch in a file-scope device array instead of memory from cudaMalloc.
 //
 // Some callers cannot allocate device memory at the time they align: a
 // process whose device memory is owned entirely by another allocator (a
@@ -7,13 +8,13 @@
 // that cannot afford cudaMalloc/cudaFree and their implicit device
 // synchronisation, or code that issues its work while a stream is being
 // captured, where allocation calls are not allowed.  xdrop_align_static
-// serves them: it takes the caller's device inputs and output, launches one
-// kernel on the caller's stream, and calls no allocating routine.
+// serves them: it takes the caller's device inputs and output, launches its
+// kernels on the caller's stream, and calls no allocating routine.
 //
 // The scratch is the static array below.  Every GPU that loads this library
 // holds it (32 MiB) until the process exits; all calls on a device share it
-// and it keeps the last call's contents.  The kernel initialises every word
-// it reads, so nothing has to be cleared between calls.  Calls whose work
+// and it keeps the last call's contents.  The kernels initialise every word
+// they read, so nothing has to be cleared between calls.  Calls whose work
 // overlaps on the GPU (different streams, or no ordering between them) race
 // on the array and must not be issued that way.
 #include <cuda_runtime.h>
@@ -22,7 +23,7 @@
 #include <cstdio>
 #include <string>
 
-#include "xd_device.cuh"
+#include "xd_warp16.cuh"
 #include "xdrop.h"
 
 namespace xd {
@@ -32,38 +33,69 @@ constexpr int kStaticMaxCtas = 128;
 
 static __device__ __align__(256) int32_t g_static_scratch[kStaticScratchWords];
 
-// One CTA per task (all 2*n_pairs tasks, grid-stride), each CTA with its
-// own slice of the static scratch.  Pairs that fail the limits get status
-// XDROP_STATUS_INVALID and zero scores; a task whose extension is longer
-// than the slice allows gets status XDROP_STATUS_TOO_LONG and zeros in its
-// side's three fields.
-__global__ void __launch_bounds__(WIDE_THREADS)
-static_wide_kernel(Job J, int32_t *scratch, int64_t per_cta)
+// Status bits of a pair whose left or right extension outgrew the warp
+// kernel's windows: set and cleared inside one call.
+constexpr int32_t kWideLeft = 1 << 8;
+
+// A warp per task (all 2*n_pairs tasks, grid-stride).  Pairs that fail the
+// limits get status XDROP_STATUS_INVALID and zero scores; a task whose
+// extension is longer than a slice of the scratch allows gets status
+// XDROP_STATUS_TOO_LONG and zeros in its side's three fields; a band wider
+// than 512 slots is left to static_wide_kernel (64 pairs of 2-4 kb reads:
+// 5.9 ms with a CTA per task on the scratch alone, 0.4 ms this way).
+__global__ void __launch_bounds__(kWarpThreads)
+static_warp_kernel(Job J, int64_t per_cta)
 {
-    int32_t *diag = scratch + (int64_t)blockIdx.x * per_cta;
-    const uint64_t n_tasks = 2 * J.n_pairs;
-    for (uint64_t t = blockIdx.x; t < n_tasks; t += gridDim.x) {
-        const uint32_t task = (uint32_t)t;
-        const Ext e = decode(J, task);
+    const int lane = threadIdx.x & 31;
+    const uint64_t n_tasks = 2 * J.n_pairs, warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t t = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n_tasks;
+         t += warps) {
+        const Ext e = decode(J, (uint32_t)t);
         int32_t *o = J.out + (size_t)e.pair * 7;
         if (!e.ok) {
-            if (threadIdx.x == 0 && e.side == 0) {
+            if (lane == 0 && e.side == 0) {
                 for (int k = 0; k < 6; ++k) o[k] = 0;
                 o[6] = XDROP_STATUS_INVALID;
             }
             continue;
         }
         if ((int64_t)3 * (e.m + 1) > per_cta) {
-            if (threadIdx.x == 0) {
+            if (lane == 0) {
                 for (int k = 0; k < 3; ++k) o[3 * e.side + k] = 0;
                 atomicOr(&o[6], XDROP_STATUS_TOO_LONG);
             }
             continue;
         }
         int32_t sc, bi, bj;
+        const int st = extend_warp(e, J.sc, false, lane, sc, bi, bj);
+        if (lane == 0) {
+            if (st == 2) atomicOr(&o[6], kWideLeft << e.side);
+            else write_result(J, e, sc, bi, bj);
+        }
+        __syncwarp();
+    }
+}
+
+// The tasks static_warp_kernel left: one CTA per task, each with its own
+// slice of the static scratch.
+__global__ void __launch_bounds__(WIDE_THREADS)
+static_wide_kernel(Job J, int32_t *scratch, int64_t per_cta)
+{
+    int32_t *diag = scratch + (int64_t)blockIdx.x * per_cta;
+    const uint64_t n_tasks = 2 * J.n_pairs;
+    for (uint64_t t = blockIdx.x; t < n_tasks; t += gridDim.x) {
+        int32_t *status = J.out + (size_t)(t >> 1) * 7 + 6;
+        const int32_t mine = kWideLeft << (t & 1);
+        // the other side's CTA changes its own bit only
+        if (!(*(volatile int32_t *)status & mine)) continue;
+        const Ext e = decode(J, (uint32_t)t);
+        int32_t sc, bi, bj;
         int64_t cells;
         extend_wide<false>(e, J.sc, diag, sc, bi, bj, cells);
-        if (threadIdx.x == 0) write_result(J, e, sc, bi, bj);
+        if (threadIdx.x == 0) {
+            write_result(J, e, sc, bi, bj);
+            atomicAnd(status, ~mine);
+        }
         __syncthreads();
     }
 }
@@ -146,6 +178,8 @@ extern "C" int xdrop_align_static(const uint32_t *packed, uint64_t n_words,
     (void)cudaGetLastError();
     const uint64_t cb = (n_pairs + 255) / 256;
     static_clear_status<<<(unsigned)std::min<uint64_t>(cb, 1024), 256, 0, st>>>(J);
+    const uint64_t wb = (2 * n_pairs + kWarpThreads / 32 - 1) / (kWarpThreads / 32);
+    static_warp_kernel<<<(unsigned)std::min<uint64_t>(wb, 4096), kWarpThreads, 0, st>>>(J, per_cta);
     static_wide_kernel<<<grid, WIDE_THREADS, 0, st>>>(J, scratch, per_cta);
     e = cudaGetLastError();
     if (e != cudaSuccess) return static_fail(XDROP_ECUDA, "kernel launch", e);
