@@ -14,12 +14,12 @@
 //      entry per (read pair, shared reliable k-mer); a radix sort by pair, a
 //      gather and a reduce-by-key with xs::CandMerge give one candidate per
 //      pair;
-//   row-wise (default): A's columns (csc_kernel) and rows
-//      (csr_kernel), then row_kernel, one block per read a, accumulates a's
-//      partners b > a in a shared-memory hash table (count + 64-bit minimum
-//      seed key per partner, shared-memory atomics) in one pass, staging up
-//      to 256 partners per read (a second pass rewrites the rare reads with
-//      more); a radix sort of the few candidates orders them.  No per-entry
+//   row-wise (default): A's columns and the place of every occurrence in
+//      them (column_kernel), then row_kernel, one block per read a, accumulates
+//      a's partners b > a in a shared-memory hash table (count + 64-bit
+//      minimum seed key per partner, shared-memory atomics) in one pass,
+//      staging up to 256 partners per read (a second pass rewrites the rare
+//      reads with more); a radix sort of the few candidates orders them.  No per-entry
 //      table exists.  A read with more partners than the table holds makes
 //      the call take the sort-based product instead (same result).
 // The sorts, run-length encoding, scans and reduce-by-key are CUB library
@@ -130,55 +130,76 @@ out_kernel(const uint64_t *__restrict__ keys, const xs::Cand *__restrict__ agg, 
 
 // ------------------------------------------------------ row-wise product
 
-__global__ void __launch_bounds__(kThreads)
-ucount_kernel(const uint32_t *__restrict__ occ, const uint32_t *__restrict__ occ_rd,
-              const int *__restrict__ run_off, const int *__restrict__ run_len, int n_runs,
-              uint32_t lo, uint32_t hi, uint32_t *__restrict__ ucnt)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_runs; i += gridDim.x * blockDim.x)
-        ucnt[i] = xs::run_reads(occ, occ_rd, (uint64_t)run_off[i], (uint32_t)run_len[i], lo, hi);
-}
+// The columns of A (reliable runs) and where their members stand.  A warp
+// takes 32 runs, reserves room for their entries with one atomic (columns
+// may stand in any order, and the entries that are no read's first leave
+// holes after a column), then writes one column after the other, a lane per
+// entry: member words in read order, the last one marked kLast, and for the
+// member's occurrence q, row_of[q] = the member's index.  Rows need no table
+// of their own: row a is the occurrences of read a, in order of position.
+constexpr unsigned long long kLast = 1ull << 63;  // read ids are below 2^31
+constexpr uint32_t kNone = 0xFFFFFFFFu;
 
-// Column i of A (reliable run i) into members[col_end[i-1] .. col_end[i]),
-// with each member's column id; counts each read's row length.
 __global__ void __launch_bounds__(kThreads)
-csc_kernel(const uint32_t *__restrict__ occ, const uint32_t *__restrict__ occ_rd,
-           const uint32_t *__restrict__ fwd_bits, const uint64_t *__restrict__ occ_off,
-           const int *__restrict__ run_off, const int *__restrict__ run_len,
-           const uint32_t *__restrict__ col_end, int n_runs, uint32_t stride,
-           uint64_t *__restrict__ members, uint32_t *__restrict__ col_of,
-           uint32_t *__restrict__ row_cnt)
+column_kernel(const uint32_t *__restrict__ occ, const uint32_t *__restrict__ occ_rd,
+              const uint32_t *__restrict__ fwd_bits, const uint64_t *__restrict__ occ_off,
+              const int *__restrict__ run_off, const int *__restrict__ run_len, int n_runs,
+              uint32_t lo, uint32_t hi, uint32_t stride, uint64_t *__restrict__ members,
+              uint32_t *__restrict__ row_of, uint32_t *__restrict__ cursor,
+              unsigned long long *__restrict__ nonzeros)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_runs; i += gridDim.x * blockDim.x) {
-        const uint32_t c0 = i ? col_end[i - 1] : 0, c1 = col_end[i];
-        if (c1 == c0) continue;
-        xs::run_members(occ, occ_rd, fwd_bits, occ_off, (uint64_t)run_off[i], (uint32_t)run_len[i],
-                        stride, members + c0);
-        for (uint32_t j = c0; j < c1; ++j) {
-            col_of[j] = (uint32_t)i;
-            atomicAdd(&row_cnt[(uint32_t)(members[j] >> 32)], 1u);
+    const uint32_t lane = threadIdx.x & 31;
+    const int warps = (int)((gridDim.x * blockDim.x) >> 5);
+    uint32_t nnz = 0;
+    for (int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w * 32ll < n_runs; w += warps) {
+        const int i = w * 32 + (int)lane;
+        uint32_t cnt = 0, off = 0;
+        if (i < n_runs) {
+            cnt = (uint32_t)run_len[i];
+            off = (uint32_t)run_off[i];
+            if (cnt < lo || cnt > hi) cnt = 0;
+        }
+        uint32_t sum = cnt;  // inclusive scan over the warp's runs
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, sum, d);
+            if (lane >= (uint32_t)d) sum += v;
+        }
+        uint32_t base = 0;
+        if (lane == 31 && sum) base = atomicAdd(cursor, sum);
+        base = __shfl_sync(0xFFFFFFFFu, base, 31) + sum - cnt;
+        for (unsigned todo = __ballot_sync(0xFFFFFFFFu, cnt != 0); todo; todo &= todo - 1) {
+            const int r = __ffs((int)todo) - 1;
+            const uint32_t s0 = __shfl_sync(0xFFFFFFFFu, off, r), n = __shfl_sync(0xFFFFFFFFu, cnt, r);
+            const uint32_t c0 = __shfl_sync(0xFFFFFFFFu, base, r);
+            uint32_t u = 0, before = kNone;  // members so far, read of the last entry
+            for (uint32_t e0 = 0; e0 < n; e0 += 32) {
+                const bool in = e0 + lane < n;
+                const uint32_t q = in ? occ[s0 + e0 + lane] : 0u;
+                const uint32_t rd = in ? occ_rd[q] : kNone;
+                uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, rd, 1);
+                if (lane == 0) prev = before;
+                const bool first = in && rd != prev;  // its read's first occurrence
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, first);
+                if (first) {
+                    const uint32_t j = c0 + u + __popc(m & ((1u << lane) - 1u));
+                    members[j] = xs::member_word(rd, (uint32_t)((q - occ_off[rd]) * stride),
+                                                 xs::fwd_bit(fwd_bits, q));
+                    row_of[q] = j;
+                }
+                u += (uint32_t)__popc(m);
+                before = __shfl_sync(0xFFFFFFFFu, rd, 31);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                members[c0 + u - 1] |= kLast;
+                nnz += u;
+            }
         }
     }
+    if (lane == 0 && nnz) atomicAdd(nonzeros, (unsigned long long)nnz);
 }
 
-// Row a of A: (column, position << 1 | forward) of a's reliable k-mers, in
-// any order within the row.
-__global__ void __launch_bounds__(kThreads)
-csr_kernel(const uint64_t *__restrict__ members, const uint32_t *__restrict__ col_of, uint64_t nnz,
-           const uint32_t *__restrict__ row_end, uint32_t *__restrict__ row_fill,
-           uint32_t *__restrict__ row_col, uint32_t *__restrict__ row_pos)
-{
-    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < nnz;
-         j += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t m = members[j];
-        const uint32_t r = (uint32_t)(m >> 32);
-        const uint32_t e = (r ? row_end[r - 1] : 0) + atomicAdd(&row_fill[r], 1u);
-        row_col[e] = col_of[j];
-        row_pos[e] = (uint32_t)(m & 0xFFFFFFFFu);
-    }
-}
-
-// One block per read a: the partners b > a of a in a shared-memory table.
 // Partners of a read kept in its staging area by the first pass; a read
 // with more goes through the second pass.
 constexpr uint32_t kStage = 256;
@@ -191,18 +212,29 @@ struct Stage {
     uint32_t *cnt;
 };
 
+// One block per read a: the partners b > a of a in a shared-memory table.
+// The members behind a's own in a column are exactly those (columns are in
+// read order), so half of the column is never read.  A warp takes 32
+// positions of a, then a half warp per reliable one walks its column from
+// behind a's member to the one marked kLast, a lane per member.  Positions
+// come in increasing order, so the first term of a partner almost always
+// holds its smallest position and the 64-bit minimum is skipped after it (a
+// stale read of it can only be too large, which costs one atomic).
+//
 // WRITE = false (first pass, block a = read a): cand_cnt[a] = number of
 // partners (0 and the overflow flag when the table is full); up to kStage
 // partners go to a's staging area, a read with more is listed in big.
 // WRITE = true (second pass, block i = read big[i]): the partners' records
 // at cand_end[a-1] ..., in table order.
+constexpr int kRowThreads = 1024;  // two blocks per SM: the longest reads end the kernel
+constexpr int kCols = 2;          // columns in flight per half warp
 template <bool WRITE>
-__global__ void __launch_bounds__(kThreads)
-row_kernel(const uint32_t *__restrict__ row_end, const uint32_t *__restrict__ row_col,
-           const uint32_t *__restrict__ row_pos, const uint32_t *__restrict__ col_end,
+__global__ void __launch_bounds__(kRowThreads)
+row_kernel(const uint64_t *__restrict__ occ_off, const uint32_t *__restrict__ row_of,
            const uint64_t *__restrict__ members, const uint32_t *__restrict__ read_len,
-           uint32_t k, uint32_t nb, uint64_t *__restrict__ cand_cnt,
-           const uint64_t *__restrict__ cand_end, uint32_t *__restrict__ overflow, Stage stage,
+           uint32_t k, uint32_t stride, uint32_t nb, uint64_t n_occ,
+           uint64_t *__restrict__ cand_cnt, const uint64_t *__restrict__ cand_end,
+           uint32_t *__restrict__ overflow, Stage stage,
            uint32_t *__restrict__ big, uint32_t *__restrict__ n_big,
            uint64_t *__restrict__ rkey, unsigned long long *__restrict__ rbest,
            uint32_t *__restrict__ rshared, uint32_t *__restrict__ ridx)
@@ -212,8 +244,8 @@ row_kernel(const uint32_t *__restrict__ row_end, const uint32_t *__restrict__ ro
     __shared__ unsigned long long tbest[kSlots];
     __shared__ uint32_t ovf, cursor;
     const uint32_t a = WRITE ? big[blockIdx.x] : blockIdx.x;
-    const uint32_t e0 = a ? row_end[a - 1] : 0, e1 = row_end[a];
-    if (e0 == e1) {  // a holds no reliable k-mer
+    const uint64_t q0 = occ_off[a], q1 = occ_off[a + 1];
+    if (q0 == q1) {  // a holds no k-mer
         if (!WRITE && threadIdx.x == 0) cand_cnt[a] = 0;
         return;
     }
@@ -229,13 +261,49 @@ row_kernel(const uint32_t *__restrict__ row_end, const uint32_t *__restrict__ ro
     __syncthreads();
     const xs::RowTable t{tkey, tcnt, tbest, xs::kTableLg};
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    // a warp per row entry, its lanes over the entry's column
-    for (uint32_t e = e0 + warp; e < e1; e += n_warps) {
+    const uint32_t half = lane >> 4, hl = lane & 15;
+    for (uint64_t b0 = q0 + 32 * warp; b0 < q1; b0 += 32 * n_warps) {
         if (*(volatile uint32_t *)&ovf) break;
-        const uint32_t col = row_col[e], pw = row_pos[e];
-        const uint32_t c0 = col ? col_end[col - 1] : 0, c1 = col_end[col];
-        for (uint32_t j = c0 + lane; j < c1; j += 32)
-            if (!xs::row_term(t, a, pw >> 1, (pw & 1u) != 0, members[j], read_len, k)) ovf = 1;
+        const uint64_t q = b0 + lane;
+        uint32_t own = q < q1 ? row_of[q] : kNone;
+        uint64_t word = 0;
+        if (own != kNone) {
+            word = members[own];
+            if (word & kLast) own = kNone;  // no read behind a in the column
+        }
+        const uint32_t pw = (uint32_t)word;  // position << 1 | forward
+        unsigned todo = __ballot_sync(0xFFFFFFFFu, own != kNone);
+        while (todo) {  // kCols positions per half warp at a time: their loads overlap
+            uint32_t j[kCols], p[kCols];
+            uint64_t m[kCols];
+            bool more[kCols];
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) {
+                const int s0 = todo ? __ffs((int)todo) - 1 : -1;
+                todo &= todo - 1;
+                const int s1 = todo ? __ffs((int)todo) - 1 : -1;
+                todo &= todo - 1;
+                const int src = half ? s1 : s0;
+                j[c] = __shfl_sync(0xFFFFFFFFu, own, src < 0 ? 0 : src) + 1 + hl;
+                p[c] = __shfl_sync(0xFFFFFFFFu, pw, src < 0 ? 0 : src);
+                more[c] = src >= 0;
+                m[c] = more[c] && j[c] < n_occ ? members[j[c]] : 0ull;
+            }
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) {
+                while (__any_sync(0xFFFFFFFFu, more[c])) {
+                    const unsigned ends =
+                        (__ballot_sync(0xFFFFFFFFu, more[c] && (m[c] & kLast)) >> (16 * half)) & 0xFFFFu;
+                    // members up to the marked one; what follows is another column's
+                    const bool in = more[c] && (!ends || hl <= (uint32_t)__ffs((int)ends) - 1u);
+                    if (in && !xs::row_term(t, a, p[c] >> 1, (p[c] & 1u) != 0, m[c] & ~kLast, read_len, k))
+                        ovf = 1;
+                    more[c] = more[c] && !ends;
+                    j[c] += 16;
+                    m[c] = more[c] && j[c] < n_occ ? members[j[c]] : 0ull;
+                }
+            }
+        }
     }
     __syncthreads();
     if (ovf) {
@@ -394,6 +462,8 @@ struct Front {
     uint64_t *occ_off = nullptr;
     const uint64_t *codes = nullptr;
     const uint32_t *occ = nullptr;
+    uint64_t *spare8 = nullptr;  // the sort's other buffers: n_occ words of 8
+    uint32_t *spare4 = nullptr;  // and of 4 bytes, free after it
     uint32_t *occ_rd = nullptr, *fwd_bits = nullptr;
     int *run_off = nullptr, *run_len = nullptr;
     int n_runs = 0;
@@ -435,6 +505,8 @@ int front(Arena &ar, Front &f, const std::vector<uint64_t> &occ_off)
     XS_CK(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, dk, dv, n, 0, (int)(2 * f.k), ar.s));
     f.codes = dk.Current();
     f.occ = dv.Current();
+    f.spare8 = dk.Alternate();
+    f.spare4 = dv.Alternate();
     // runs of length >= 2 (a k-mer seen once pairs no reads)
     int *d_nruns;
     XS_GET(f.run_off, f.n_occ / 2 + 1);
@@ -543,46 +615,20 @@ int row_product(Arena &ar, const Front &f, std::vector<Pair> &out_pairs,
 {
     *done = false;
     const int n_runs = f.n_runs, n_reads = (int)f.n_reads;
-    // columns: distinct reads per reliable run, scanned
-    uint32_t *ucnt, *col_end;
-    XS_GET(ucnt, n_runs);
-    XS_GET(col_end, n_runs);
-    ucount_kernel<<<grid_for(n_runs, f.sm_count), kThreads, 0, ar.s>>>(
-        f.occ, f.occ_rd, f.run_off, f.run_len, n_runs, f.lo, f.hi, ucnt);
-    XS_CK(cudaGetLastError());
-    size_t bytes = 0;
-    char *tmp;
-    XS_CK(cub::DeviceScan::InclusiveSum(nullptr, bytes, ucnt, col_end, n_runs, ar.s));
-    XS_GET(tmp, bytes);
-    XS_CK(cub::DeviceScan::InclusiveSum(tmp, bytes, ucnt, col_end, n_runs, ar.s));
-    uint32_t nnz = 0;
-    if (int rc = read_back(ar, &nnz, col_end + (n_runs - 1))) return rc;
-    *nonzeros = nnz;
-    if (nnz == 0) {
-        *done = true;
-        return XDROP_OK;
-    }
-    uint64_t *members;
-    uint32_t *col_of, *row_cnt, *row_end, *row_fill, *row_col, *row_pos;
-    XS_GET(members, nnz);
-    XS_GET(col_of, nnz);
-    XS_GET(row_cnt, n_reads);
-    XS_GET(row_end, n_reads);
-    XS_GET(row_fill, n_reads);
-    XS_GET(row_col, nnz);
-    XS_GET(row_pos, nnz);
-    XS_CK(cudaMemsetAsync(row_cnt, 0, (size_t)n_reads * 4, ar.s));
-    XS_CK(cudaMemsetAsync(row_fill, 0, (size_t)n_reads * 4, ar.s));
-    csc_kernel<<<grid_for(n_runs, f.sm_count), kThreads, 0, ar.s>>>(
-        f.occ, f.occ_rd, f.fwd_bits, f.occ_off, f.run_off, f.run_len, col_end, n_runs, f.stride,
-        members, col_of, row_cnt);
-    XS_CK(cudaGetLastError());
-    bytes = 0;
-    XS_CK(cub::DeviceScan::InclusiveSum(nullptr, bytes, row_cnt, row_end, n_reads, ar.s));
-    XS_GET(tmp, bytes);
-    XS_CK(cub::DeviceScan::InclusiveSum(tmp, bytes, row_cnt, row_end, n_reads, ar.s));
-    csr_kernel<<<grid_for(nnz, f.sm_count), kThreads, 0, ar.s>>>(members, col_of, nnz, row_end,
-                                                                 row_fill, row_col, row_pos);
+    // columns and row entries, in the buffers the sort no longer needs (a
+    // column has at most as many members as its run has occurrences)
+    uint64_t *members = f.spare8;
+    uint32_t *row_of = f.spare4;
+    struct Counts {
+        unsigned long long nonzeros;
+        uint32_t cursor, pad;
+    } *counts, h_counts{};
+    XS_GET(counts, 1);
+    XS_CK(cudaMemsetAsync(counts, 0, sizeof(Counts), ar.s));
+    XS_CK(cudaMemsetAsync(row_of, 0xFF, f.n_occ * sizeof(uint32_t), ar.s));
+    column_kernel<<<grid_for(n_runs, f.sm_count), kThreads, 0, ar.s>>>(
+        f.occ, f.occ_rd, f.fwd_bits, f.occ_off, f.run_off, f.run_len, n_runs, f.lo, f.hi, f.stride,
+        members, row_of, &counts->cursor, &counts->nonzeros);
     XS_CK(cudaGetLastError());
     // each read's partners in one pass: counted, and staged when there are
     // at most kStage of them; reads with more are recomputed and written
@@ -598,18 +644,21 @@ int row_product(Arena &ar, const Front &f, std::vector<Pair> &out_pairs,
     XS_GET(stage.best, (uint64_t)n_reads * kStage);
     XS_GET(stage.cnt, (uint64_t)n_reads * kStage);
     XS_CK(cudaMemsetAsync(flags, 0, 8, ar.s));
-    row_kernel<false><<<n_reads, kThreads, 0, ar.s>>>(
-        row_end, row_col, row_pos, col_end, members, f.read_len, f.k, f.nb, cand_cnt, nullptr,
-        flags, stage, big, flags + 1, nullptr, nullptr, nullptr, nullptr);
+    row_kernel<false><<<n_reads, kRowThreads, 0, ar.s>>>(
+        f.occ_off, row_of, members, f.read_len, f.k, f.stride, f.nb, f.n_occ, cand_cnt, nullptr, flags,
+        stage, big, flags + 1, nullptr, nullptr, nullptr, nullptr);
     XS_CK(cudaGetLastError());
-    bytes = 0;
+    size_t bytes = 0;
+    char *tmp;
     XS_CK(cub::DeviceScan::InclusiveSum(nullptr, bytes, cand_cnt, cand_end, n_reads, ar.s));
     XS_GET(tmp, bytes);
     XS_CK(cub::DeviceScan::InclusiveSum(tmp, bytes, cand_cnt, cand_end, n_reads, ar.s));
     uint32_t hflags[2] = {0, 0};
     uint64_t n_cand = 0;
     XS_CK(cudaMemcpyAsync(hflags, flags, 8, cudaMemcpyDeviceToHost, ar.s));
+    XS_CK(cudaMemcpyAsync(&h_counts, counts, sizeof(Counts), cudaMemcpyDeviceToHost, ar.s));
     if (int rc = read_back(ar, &n_cand, cand_end + (n_reads - 1))) return rc;
+    *nonzeros = h_counts.nonzeros;
     const uint32_t ovf = hflags[0], n_big = hflags[1];
     if (ovf) return XDROP_OK;  // not done: the sort-based product takes over
     *done = true;
@@ -631,8 +680,8 @@ int row_product(Arena &ar, const Front &f, std::vector<Pair> &out_pairs,
         cand_cnt, cand_end, stage, (uint32_t)n_reads, f.nb, rk0, rbest, rshared, ri0);
     XS_CK(cudaGetLastError());
     if (n_big) {
-        row_kernel<true><<<n_big, kThreads, 0, ar.s>>>(
-            row_end, row_col, row_pos, col_end, members, f.read_len, f.k, f.nb, nullptr, cand_end,
+        row_kernel<true><<<n_big, kRowThreads, 0, ar.s>>>(
+            f.occ_off, row_of, members, f.read_len, f.k, f.stride, f.nb, f.n_occ, nullptr, cand_end,
             nullptr, stage, big, nullptr, rk0, rbest, rshared, ri0);
         XS_CK(cudaGetLastError());
     }

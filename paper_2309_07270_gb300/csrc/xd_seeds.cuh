@@ -240,43 +240,52 @@ XS_HD uint32_t table_slot(uint32_t b, uint32_t lg)
     return (b * 2654435761u) >> (32 - lg);  // multiplicative hash, top bits
 }
 
-// Adds one shared k-mer of partner b; false when the table is full.  On
-// the device the slots are claimed and updated with shared-memory atomics
+// The slot of partner b, claimed if it has none yet; kEmpty when the table is
+// full.  On the device the slots are claimed with shared-memory atomics
 // (insertions from all threads of the block at once); on the host in order.
-XS_HD bool table_add(const RowTable &t, uint32_t b, uint64_t key)
+XS_HD uint32_t table_find(const RowTable &t, uint32_t b)
 {
     const uint32_t mask = (1u << t.lg) - 1;
     uint32_t h = table_slot(b, t.lg);
     for (uint32_t probe = 0; probe <= mask; ++probe, h = (h + 1) & mask) {
+        uint32_t prev = t.key[h];  // a claimed slot never changes its key
 #if defined(__CUDA_ARCH__)
-        const uint32_t prev = atomicCAS(&t.key[h], kEmpty, b);
+        if (prev == kEmpty) prev = atomicCAS(&t.key[h], kEmpty, b);
 #else
-        const uint32_t prev = t.key[h];
         if (prev == kEmpty) t.key[h] = b;
 #endif
-        if (prev != kEmpty && prev != b) continue;
-#if defined(__CUDA_ARCH__)
-        atomicAdd(&t.cnt[h], 1u);
-        atomicMin(&t.best[h], (unsigned long long)key);
-#else
-        t.cnt[h] += 1;
-        if (key < t.best[h]) t.best[h] = key;
-#endif
-        return true;
+        if (prev == kEmpty || prev == b) return h;
     }
-    return false;
+    return kEmpty;
 }
 
 // One (row entry, column member) product term of read a: a k-mer at
-// position pa of a (forward fa) that read member>>32 also holds.
+// position pa of a (forward fa) that read member>>32 also holds: one more
+// shared k-mer of that partner, and its seed if the position is smaller
+// than every one so far.  False when the table is full.
 XS_HD bool row_term(const RowTable &t, uint32_t a, uint32_t pa, bool fa, uint64_t member,
                     const uint32_t *read_len, uint32_t k)
 {
     const uint32_t b = (uint32_t)(member >> 32);
     if (b <= a) return true;
+    const uint32_t h = table_find(t, b);
+    if (h == kEmpty) return false;
     const uint32_t pb = (uint32_t)(member & 0xFFFFFFFFu) >> 1;
     const bool rc = fa != ((member & 1u) != 0);
-    return table_add(t, b, seed_key(pa, rc ? read_len[b] - k - pb : pb, rc));
+#if defined(__CUDA_ARCH__)
+    atomicAdd(&t.cnt[h], 1u);
+    // The position alone decides (the positions of a pair's shared k-mers in
+    // a are distinct), and it only falls: a stale read of it can only ask for
+    // a minimum too many.
+    if (pa < ((const volatile uint32_t *)&t.best[h])[1])
+        atomicMin(&t.best[h],
+                  (unsigned long long)seed_key(pa, rc ? read_len[b] - k - pb : pb, rc));
+#else
+    t.cnt[h] += 1;
+    const uint64_t key = seed_key(pa, rc ? read_len[b] - k - pb : pb, rc);
+    if (key < t.best[h]) t.best[h] = key;
+#endif
+    return true;
 }
 
 // Bits per read id in a pair key: the smallest nb >= 1 with n_reads <= 2^nb.
