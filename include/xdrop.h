@@ -256,9 +256,8 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st);
  * and `cells` cells per lane (lanes*cells slots per anti-diagonal parity),
  * or pass lanes = 0 to go back to autotuning.  Autotuning (the default)
  * keys the first tile by the scoring and the job's length bucket (the
- * length bin, ceil(log2(max(m, n) + 1)) of an extension, that holds the
- * median of the job's work, read from a device histogram at every batched
- * submit).  The first submit with a new key times the first-tier tiles on
+ * octave of an extension's min(m, n) that holds the median of the job's work,
+ * read from a device histogram at every batched submit).  The first submit with a new key times the first-tier tiles on
  * a stratified random sample of its pairs (one pair of every 3 with the
  * packed tiles when the scoring fits them, else one of every 8 with the
  * 32-bit tiles; widths far from x / |gap| are left out) and keeps the

@@ -66,16 +66,23 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 // Counter block layout (uint32 words) in device memory.
 enum : int {
-    C_HIST = 0,          // NBINS
-    C_OFFS = 32,         // NBINS
-    C_NVALID = 64,
-    C_COUNTER = 65,
-    C_SPILL0 = 66,       // extensions the first tier handed on
-    C_SPILL1 = 67,       // extensions for the unbounded tier
-    C_WARP = 68,         // work counter of the warp kernel
-    C_NBAD = 69,
-    C_MAXLEN = 70,
-    C_WORDS = 72
+    C_HIST = 0,               // NBINS
+    C_OFFS = NBINS,           // NBINS
+    C_NVALID = 2 * NBINS,
+    C_COUNTER,                // first tier's work counter
+    C_SPILL0,                 // extensions the first tier handed on
+    C_SPILL1,                 // extensions for the unbounded tier
+    C_WARP,                   // work counter of the warp kernel
+    C_ROLE,                   // the words of a WarpRole, but for err
+    C_GROWN = C_ROLE + 5,     // longest tasks that outgrew a warp's first window
+    C_BRIEF,                  // short overflow, the second group tier's tasks
+    C_COUNTER2,               // its work counter
+    C_SPILL2,                 // its overflow
+    C_ROLE2,                  // the words of its WarpRole
+    C_NBAD = C_ROLE2 + 6,    // kept by the launch sequence's memset, as the next two
+    C_MAXLEN,
+    C_ROLE_ERR,               // sticky: a lost overflow entry
+    C_WORDS
 };
 
 struct DevBuf {
@@ -113,7 +120,7 @@ struct xdrop_ctx {
 
     Job *d_job = nullptr;
     uint32_t *d_ctrs = nullptr;
-    DevBuf order, spill[2], wide;
+    DevBuf order, spill[3], wide;
     DevBuf plain_ctl;  // plain mode: task count and work counter per sub-batch
     size_t cap_tasks = 0;
     int64_t wide_per_cta = 0;
@@ -132,6 +139,8 @@ struct xdrop_ctx {
     cudaGraphExec_t gexec = nullptr;
     cudaEvent_t ev_main0 = nullptr, ev_main1 = nullptr;  // recorded inside the graph
     Tile graph_tile = {0, 0};
+    bool graph_brief = false;
+    uint32_t graph_launches = 0;
     uint64_t graph_version = ~0ull;
 
     xdrop_stats last = {};
@@ -192,7 +201,8 @@ int ensure_scratch(xdrop_ctx *c, size_t n_tasks, uint32_t maxlen)
     if ((rc = dev_alloc(c, c->order, tasks * 4))) return rc;
     for (auto &s : c->spill)
         if ((rc = dev_alloc(c, s, tasks * 4))) return rc;
-    c->cap_tasks = std::min(c->order.cap, std::min(c->spill[0].cap, c->spill[1].cap)) / 4;
+    c->cap_tasks = std::min(c->order.cap, std::min(c->spill[0].cap,
+                            std::min(c->spill[1].cap, c->spill[2].cap))) / 4;
     int64_t per = (int64_t)3 * ((int64_t)maxlen + 1);
     per = (per + 63) / 64 * 64;
     if (per > c->wide_per_cta) {
@@ -220,35 +230,80 @@ Spill spill_of(xdrop_ctx *c, int k)
     return Spill{(uint32_t *)c->spill[k].p, c->d_ctrs + C_SPILL0 + k};
 }
 
-// The tiers after a first tier of width w: a warp per extension (windows of
-// 128 slots unless the first tier had them, then 512), then the unbounded
-// tier.
+// The tiers after a first tier of width w: a warp per extension (the wider
+// ones of windows of 128, 256 and 512 slots), then the unbounded tier.
 int enqueue_wider(xdrop_ctx *c, int w, uint64_t n_tasks)
 {
     CK(launch_warp(n_tasks, c->sm_count, c->d_job, spill_of(c, 0).list, spill_of(c, 0).count,
-                   c->d_ctrs + C_WARP, w >= 128, nullptr, Spill{}, spill_of(c, 1), c->stream));
+                   c->d_ctrs + C_WARP, w, nullptr, Spill{}, spill_of(c, 1), c->stream));
     CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
                    c->wide_per_cta, c->stream));
     return XDROP_OK;
 }
 
+// The words of the single-warp part of a first tier that has one.
+WarpRole role_of(xdrop_ctx *c, Tile t)
+{
+    if (!has_warp_role(t)) return WarpRole{};
+    uint32_t *w = c->d_ctrs + C_ROLE;
+    return WarpRole{w, w + 1, w + 2, w + 3, w + 4, c->d_ctrs + C_GROWN, c->d_ctrs + C_ROLE_ERR,
+                    spill_of(c, 1), 0};
+}
+
+bool has_brief(Tile t0, const Scoring &sc)
+{
+    const Tile t{4, 32, true};
+    return has_warp_role(t0) && t0.width() < 128 && packed_tile_ok(t, sc) &&
+           has_warp_role(in_frame(t, sc));
+}
+
+// The second group tier, for the short overflow of a first tier narrower than
+// 128 slots: 4x32 on the list, its own overflow (kept where the order was) to
+// single warps, as are all its tasks if there are few.
+int enqueue_brief(xdrop_ctx *c)
+{
+    const Tile t{4, 32, true};
+    const int bps = persistent_blocks_per_sm(t);
+    if (bps <= 0) return fail(XDROP_ECUDA, "tile 4x32 not available");
+    uint32_t *ctr = c->d_ctrs, *w = ctr + C_ROLE2, *list = (uint32_t *)c->order.p;
+    const int grid = c->sm_count * bps;
+    const uint32_t few = (uint32_t)(grid * persistent_block_threads(t) / 32);
+    const WarpRole role{w, w + 1, w + 2, w + 3, w + 4, w + 5, ctr + C_ROLE_ERR, spill_of(c, 1), few};
+    CK(cudaMemsetAsync(list, 0xFF, c->cap_tasks * 4, c->stream));
+    CK(launch_persistent(t, grid, c->d_job, (uint32_t *)c->spill[2].p, ctr + C_BRIEF,
+                         ctr + C_COUNTER2, Spill{list, ctr + C_SPILL2}, Spill{}, role, c->stream));
+    return XDROP_OK;
+}
+
 // Enqueue the batched launch sequence (graph body) with first tile t0.
-int enqueue_batched(xdrop_ctx *c, Tile t0, int bps, bool main_events, uint32_t *launches)
+int enqueue_batched(xdrop_ctx *c, Tile t0, int bps, const Scoring &sc, bool main_events,
+                    uint32_t *launches)
 {
     cudaStream_t s = c->stream;
     uint32_t *ctr = c->d_ctrs;
     CK(cudaMemsetAsync(ctr, 0, C_NBAD * 4, s));  // keep NBAD / MAXLEN
     const int bgrid = c->sm_count * 4;
-    CK(launch_binning(c->d_job, 0, bgrid, ctr + C_HIST, ctr + C_OFFS, ctr + C_NVALID,
-                      (uint32_t *)c->order.p, s));
+    const WarpRole role = role_of(c, t0);
+    Spill brief{};
+    if (has_brief(t0, sc)) brief = Spill{(uint32_t *)c->spill[2].p, ctr + C_BRIEF};
+    // overflow entries are read while the first tier runs: mark them unwritten
+    if (role.n_long) CK(cudaMemsetAsync(c->spill[0].p, 0xFF, c->cap_tasks * 4, s));
+    CK(launch_binning(c->d_job, bgrid, ctr + C_HIST, ctr + C_OFFS, ctr + C_NVALID, ctr + C_COUNTER,
+                      (uint32_t *)c->order.p, t0, c->sm_count * bps, role, !c->forced.lanes, s));
     if (bps <= 0) return fail(XDROP_ECUDA, "tile %dx%d not available", t0.lanes, t0.c);
     // External record nodes, so the events are really recorded on replay.
     if (main_events) CK(cudaEventRecordWithFlags(c->ev_main0, s, cudaEventRecordExternal));
     CK(launch_persistent(t0, c->sm_count * bps, c->d_job, (uint32_t *)c->order.p,
-                         ctr + C_NVALID, ctr + C_COUNTER, spill_of(c, 0), s));
+                         ctr + C_NVALID, ctr + C_COUNTER, spill_of(c, 0), brief, role, s));
     if (main_events) CK(cudaEventRecordWithFlags(c->ev_main1, s, cudaEventRecordExternal));
-    if (launches) *launches = 6;
-    return enqueue_wider(c, t0.width(), c->cap_tasks);
+    if (launches) *launches = (role.n_long ? 5 : 6) + (brief.list ? 1 : 0);
+    if (brief.list) {
+        if (int rc = enqueue_brief(c)) return rc;
+    }
+    if (!role.n_long) return enqueue_wider(c, t0.width(), c->cap_tasks);
+    CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
+                   c->wide_per_cta, s));
+    return XDROP_OK;
 }
 
 // Candidate first tiles for autotuning (all persistent instantiations);
@@ -304,6 +359,11 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     const int64_t span = job.sc.x / -(int64_t)job.sc.gap;
     const int64_t min_w = std::min<int64_t>(128, span * 3 / 4);
     const int64_t max_w = std::max<int64_t>(64, span * 3);
+    // Lanes of 32 slots beat 4x8, 8x8 and 4x16 wherever they hold the scoring
+    // (29x, first tier: x = 15 4x8 42.1, 1x32 23.0 ms; x = 50 8x8 83.4, 4x16
+    // 51.6, 2x32 45.0), and 8x16 beats 16x8 (1M uneven pairs 18.6, 25.3 ms).
+    const bool long_lanes = packed && has_warp_role(in_frame(Tile{2, 32, true}, job.sc)) &&
+                            packed_tile_ok(Tile{2, 32, true}, job.sc);
     float best_ms = 1e30f;
     *best = Tile{0, 0};
     std::vector<Tile> cands;
@@ -313,13 +373,14 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
         if (cand.packed && !packed_tile_ok(cand, job.sc)) continue;
         const Tile t = in_frame(cand, job.sc);
         if (t.width() < min_w || t.width() > max_w) continue;
+        if (long_lanes && (t.c < 16 || (t.c == 16 && t.lanes == 4))) continue;
         const int bps = persistent_blocks_per_sm(t);
         if (bps <= 0) continue;
         float tmin = 1e30f;
         for (int rep = 0; rep < 2; ++rep) {
             if (rep && tmin > 1.25f * best_ms) break;  // far behind after one run
             CK(cudaEventRecord(e0, s));
-            int rc = enqueue_batched(c, t, bps, false, nullptr);
+            int rc = enqueue_batched(c, t, bps, job.sc, false, nullptr);
             if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
             CK(cudaEventRecord(e1, s));
             CK(cudaEventSynchronize(e1));
@@ -339,24 +400,24 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     return best->lanes ? XDROP_OK : fail(XDROP_ECUDA, "no tile could be timed");
 }
 
-// Length bucket of a job (the tuning key beside the scoring): the length
-// bin ceil(log2(max(m, n) + 1)) holding the median of the job's work, each
-// task weighted by 2^bin (about its length), from a device histogram read
-// back synchronously.  Workloads of different length mixes tune apart.
+// Length bucket of a job (the tuning key beside the scoring): the octave of
+// min(m, n) holding the median of the job's work, each task weighted by its
+// bin's diagonals, from a device histogram read back synchronously.
+// Workloads of different length mixes tune apart.
 int length_bucket(xdrop_ctx *c, Ticket *tk, int *bucket)
 {
     cudaStream_t s = c->stream;
-    CK(cudaMemsetAsync(c->d_ctrs + C_HIST, 0, 32 * 4, s));
+    CK(cudaMemsetAsync(c->d_ctrs + C_HIST, 0, NBINS * 4, s));
     CK(launch_length_hist(c->d_job, c->sm_count * 4, c->d_ctrs + C_HIST, s));
-    CK(cudaMemcpyAsync(tk->h_ctrs, c->d_ctrs + C_HIST, 32 * 4, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(tk->h_ctrs, c->d_ctrs + C_HIST, NBINS * 4, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     double total = 0, run = 0;
-    for (int b = 0; b < 32; ++b) total += (double)tk->h_ctrs[b] * std::ldexp(1.0, b);
+    for (int b = 0; b < NBINS; ++b) total += (double)tk->h_ctrs[b] * bin_diagonals(b);
     *bucket = 0;
-    for (int b = 0; b < 32; ++b) {
-        run += (double)tk->h_ctrs[b] * std::ldexp(1.0, b);
+    for (int b = 0; b < NBINS; ++b) {
+        run += (double)tk->h_ctrs[b] * bin_diagonals(b);
         if (run * 2 >= total && total > 0) {
-            *bucket = b;
+            *bucket = b / 4;
             break;
         }
     }
@@ -385,10 +446,10 @@ int pick_tile(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *out)
     return XDROP_OK;
 }
 
-int run_batched(xdrop_ctx *c, Ticket *tk)
+int run_batched(xdrop_ctx *c, Ticket *tk, const Scoring &sc)
 {
     if (!c->gexec || c->graph_version != c->scratch_version ||
-        !c->graph_tile.same(c->tile0)) {
+        !c->graph_tile.same(c->tile0) || c->graph_brief != has_brief(c->tile0, sc)) {
         c->tile0_bps = persistent_blocks_per_sm(c->tile0);
         if (c->gexec) {
             cudaGraphExecDestroy(c->gexec);
@@ -397,7 +458,7 @@ int run_batched(xdrop_ctx *c, Ticket *tk)
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
         uint32_t launches = 0;
-        int rc = enqueue_batched(c, c->tile0, c->tile0_bps, true, &launches);
+        int rc = enqueue_batched(c, c->tile0, c->tile0_bps, sc, true, &launches);
         cudaError_t ce = cudaStreamEndCapture(c->stream, &g);
         if (rc) {
             if (g) cudaGraphDestroy(g);
@@ -409,11 +470,12 @@ int run_batched(xdrop_ctx *c, Ticket *tk)
         if (ce != cudaSuccess) return fail(XDROP_ECUDA, "graph instantiate: %s", cudaGetErrorString(ce));
         c->graph_version = c->scratch_version;
         c->graph_tile = c->tile0;
-        c->last.launches = launches;
+        c->graph_brief = has_brief(c->tile0, sc);
+        c->graph_launches = launches;
     }
     CK(cudaGraphLaunch(c->gexec, c->stream));
     tk->graph_replays += 1;
-    tk->launches += c->last.launches;
+    tk->launches += c->graph_launches;
     return XDROP_OK;
 }
 
@@ -444,7 +506,7 @@ int run_plain(xdrop_ctx *c, Ticket *tk, const Job &job)
         const uint64_t blocks = (2 * np + groups_per_block - 1) / groups_per_block;
         const int grid = (int)std::min<uint64_t>(blocks, (uint64_t)c->sm_count * bps);
         CK(launch_persistent(t0, grid, c->d_job, order + 2 * p0, ctl + 2 * k, ctl + 2 * k + 1,
-                             spill_of(c, 0), s));
+                             spill_of(c, 0), Spill{}, WarpRole{}, s));
     }
     tk->launches += (uint32_t)(3 + n_sub);
     return enqueue_wider(c, t0.width(), 2 * n_pairs);
@@ -465,7 +527,7 @@ int run_small(xdrop_ctx *c, Ticket *tk, const Job &job)
     cudaStream_t s = c->stream;
     c->tile0 = Tile{32, 4, warp_packed(job.sc)};
     CK(cudaMemsetAsync(c->d_ctrs, 0, C_MAXLEN * 4, s));
-    CK(launch_warp(2 * job.n_pairs, c->sm_count, c->d_job, nullptr, nullptr, c->d_ctrs + C_WARP, false,
+    CK(launch_warp(2 * job.n_pairs, c->sm_count, c->d_job, nullptr, nullptr, c->d_ctrs + C_WARP, 0,
                    tk->device_submit ? c->d_ctrs + C_NBAD : nullptr, spill_of(c, 0),
                    spill_of(c, 1), s));
     CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
@@ -510,7 +572,7 @@ int launch_ticket(xdrop_ctx *c, Ticket *tk, const Job &job, uint32_t maxlen)
     if (job.n_pairs) {
         if (small) rc = run_small(c, tk, job);
         else if (c->mode == XDROP_MODE_PLAIN) rc = run_plain(c, tk, job);
-        else rc = run_batched(c, tk);
+        else rc = run_batched(c, tk, job.sc);
         if (rc) return rc;
     }
     CK(cudaEventRecord(tk->ev_end, s));
@@ -549,7 +611,7 @@ int launch_ticket_chunked(xdrop_ctx *c, Ticket *tk, const xdrop_pair *h_pairs, s
         if (k == 0) {  // first tile: as for an unchunked submit
             if ((rc = pick_tile(c, tk, job, &c->tile0))) return rc;
         }
-        if ((rc = run_batched(c, tk))) return rc;
+        if ((rc = run_batched(c, tk, job.sc))) return rc;
         CK(cudaMemcpyAsync(tk->h_out + p0, d_out, np * sizeof(xdrop_result), cudaMemcpyDeviceToHost, s));
     }
     CK(cudaEventRecord(tk->ev_end, s));
@@ -813,7 +875,7 @@ int xdrop_sync(xdrop_ctx *c, xdrop_ticket t, int64_t timeout_ns)
     st.kernel_ms = ms;
     st.main_kernel_ms = ms_main;
     st.tasks = 2 * (uint64_t)tk->n_pairs;
-    st.overflow_tasks = tk->h_ctrs[C_SPILL0];
+    st.overflow_tasks = tk->h_ctrs[C_SPILL0] + tk->h_ctrs[C_BRIEF] + tk->h_ctrs[C_GROWN];
     st.wide_tasks = tk->h_ctrs[C_SPILL1];
     st.launches = tk->launches;
     st.graph_replays = tk->graph_replays;
@@ -821,7 +883,9 @@ int xdrop_sync(xdrop_ctx *c, xdrop_ticket t, int64_t timeout_ns)
     st.tile_cells = c->tile0.c | (c->tile0.packed ? XDROP_TILE_PACKED16 : 0);
     c->last = st;
     const uint32_t nbad = tk->device_submit ? tk->h_ctrs[C_NBAD] : 0;
+    const bool lost = tk->h_ctrs[C_ROLE_ERR] != 0;
     free_ticket(c, tk);
+    if (lost) return fail(XDROP_ECUDA, "an overflow entry never appeared");
     if (nbad) return fail(XDROP_EINVAL, "%u pairs failed validation (status set)", nbad);
     return XDROP_OK;
 }
@@ -964,10 +1028,10 @@ int xdrop_submit_pairs(xdrop_ctx *c, const xdrop_pair *pairs, size_t n_pairs,
     // chunks when the pair table does not fit the device memory budget
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
-    const size_t per_pair = sizeof(xdrop_pair) + sizeof(xdrop_result) + 2 * 3 * 4;  // + task scratch
+    const size_t per_pair = sizeof(xdrop_pair) + sizeof(xdrop_result) + 2 * 4 * 4;  // + task scratch
     size_t chunk = std::max<size_t>(n_pairs, 1);
     if (c->budget && c->mode != XDROP_MODE_PLAIN) {
-        const size_t scratch_now = c->order.cap + c->spill[0].cap + c->spill[1].cap;
+        const size_t scratch_now = c->order.cap + c->spill[0].cap + c->spill[1].cap + c->spill[2].cap;
         const size_t fixed = c->used - scratch_now + 4 * kAlign;
         if (c->budget <= fixed + 1024 * per_pair)
             return fail(c->tickets.empty() ? XDROP_ENOMEM : XDROP_EBUSY,
@@ -978,7 +1042,7 @@ int xdrop_submit_pairs(xdrop_ctx *c, const xdrop_pair *pairs, size_t n_pairs,
         if (fit < chunk) {
             chunk = fit;
             // scratch sized for this chunk must not stay larger from before
-            for (DevBuf *b : {&c->order, &c->spill[0], &c->spill[1]}) {
+            for (DevBuf *b : {&c->order, &c->spill[0], &c->spill[1], &c->spill[2]}) {
                 if (b->cap > 2 * chunk * 4) {
                     CK(cudaStreamSynchronize(c->stream));
                     cudaFree(b->p);
@@ -1206,11 +1270,18 @@ int xdrop_last_spills(xdrop_ctx *c, uint32_t *dst, size_t cap, size_t *n)
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
     CK(cudaStreamSynchronize(c->stream));
-    uint32_t cnt = 0;
-    CK(cudaMemcpy(&cnt, c->d_ctrs + C_SPILL0, 4, cudaMemcpyDeviceToHost));
-    *n = cnt;
-    size_t k = std::min<size_t>(cap, cnt);
-    if (k) CK(cudaMemcpy(dst, c->spill[0].p, k * 4, cudaMemcpyDeviceToHost));
+    // the long overflow of the first tier, then the short
+    const int word[2] = {C_SPILL0, C_BRIEF}, list[2] = {0, 2};
+    size_t total = 0;
+    for (int k = 0; k < 2; ++k) {
+        uint32_t cnt = 0;
+        CK(cudaMemcpy(&cnt, c->d_ctrs + word[k], 4, cudaMemcpyDeviceToHost));
+        const size_t take = total < cap ? std::min<size_t>(cap - total, cnt) : 0;
+        if (take)
+            CK(cudaMemcpy(dst + total, c->spill[list[k]].p, take * 4, cudaMemcpyDeviceToHost));
+        total += cnt;
+    }
+    *n = total;
     return XDROP_OK;
 }
 

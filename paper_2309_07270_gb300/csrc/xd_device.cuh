@@ -535,6 +535,7 @@ struct BatchSrc {
     uint32_t n_tasks;
     uint32_t *counter;
     Spill spill;
+    Spill brief = {};  // with a list: overflow of short extensions goes there
 
     // Warp-level fetch, executed by every lane: the leaders of the groups
     // that need a task are the set bits of needm.  Returns, for this lane's
@@ -564,8 +565,13 @@ struct BatchSrc {
                                            int32_t bi, int32_t bj)
     {
         if (overflow) {
-            const uint32_t q = atomicAdd(spill.count, 1u);
-            spill.list[q] = task;
+            Spill to = spill;
+            if (brief.list) {
+                const Ext e = decode(*gj, task);
+                if (2 * min(e.m, e.n) <= kBriefDiagonals) to = brief;
+            }
+            const uint32_t q = atomicAdd(to.count, 1u);
+            *(volatile uint32_t *)&to.list[q] = task;
         } else {
             store_result(*gj, task, T, bi, bj);
         }

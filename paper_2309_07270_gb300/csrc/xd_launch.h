@@ -33,18 +33,23 @@ bool tile_supported(Tile t, bool persistent);
 cudaError_t launch_window(Tile t, bool count, const Job *jp, uint32_t task_base,
                           uint32_t n_tasks, Spill spill, cudaStream_t s);
 // Persistent: positions of `order` pulled from *counter up to *n_tasks.
+// role: single-warp extensions beside the tier (all null: none; only for
+// tiles with has_warp_role, whose overflow the kernel then finishes itself,
+// but for what goes to `brief`).
 cudaError_t launch_persistent(Tile t, int grid, const Job *jp, const uint32_t *order,
-                              const uint32_t *n_tasks, uint32_t *counter, Spill spill,
-                              cudaStream_t s);
+                              const uint32_t *n_tasks, uint32_t *counter, Spill spill, Spill brief,
+                              WarpRole role, cudaStream_t s);
+bool has_warp_role(Tile t);
+void tile_rates(Tile t, float *rate, float *group_ns);
 // Tasks listed in `in` on windows of 512 slots, overflow to `out`.
 cudaError_t launch_spill_512(int grid, const Job *jp, Spill in, Spill out, cudaStream_t s);
 // A warp per task (xd_warp16.cuh): the tasks of a list (n_tasks bounds their
-// number *n_ptr) or, without one, all tasks of the job; windows of 128 slots
-// (unless skip128), then 512, overflow to `out`.  Without a list: tasks that
+// number *n_ptr) or, without one, all tasks of the job; windows of 128, 256 and
+// 512 slots, from the first wider than `from`, overflow to `out`.  Without a list: tasks that
 // outgrew 128 slots are also noted in `over`, and n_bad asks for the pairs'
 // status.
 cudaError_t launch_warp(uint64_t n_tasks, int sm_count, const Job *jp, const uint32_t *list,
-                        const uint32_t *n_ptr, uint32_t *counter, bool skip128, uint32_t *n_bad,
+                        const uint32_t *n_ptr, uint32_t *counter, int from, uint32_t *n_bad,
                         Spill over, Spill out, cudaStream_t s);
 // Blocks per SM of a persistent tile at 256 threads per block.
 int persistent_block_threads(Tile t);  // threads per block of the persistent first tier
@@ -66,11 +71,15 @@ Tile in_frame(Tile t, const Scoring &sc);
 cudaError_t launch_wide(bool count, int grid, const Job *jp, Spill in, int32_t *scratch,
                         int64_t scratch_per_cta, cudaStream_t s);
 cudaError_t launch_validate(const Job *jp, uint64_t n_pairs, uint32_t *n_bad, cudaStream_t s);
-cudaError_t launch_binning(const Job *jp, uint64_t n_pairs, int grid, uint32_t *hist,
-                           uint32_t *offs, uint32_t *n_valid, uint32_t *order,
-                           cudaStream_t s);
-// Task length histogram of a job: hist[b] += tasks with
-// ceil(log2(max(m, n) + 1)) = b (32 bins, invalid pairs left out).
+// The longest-first order of a job's tasks (hist zeroed before), their number
+// and, with a role, the first tasks (none unless `longest`) and blocks that go
+// to single warps beside a first tier of tile t on first_grid blocks; *counter
+// starts behind them.
+cudaError_t launch_binning(const Job *jp, int grid, uint32_t *hist, uint32_t *offs,
+                           uint32_t *n_valid, uint32_t *counter, uint32_t *order, Tile t,
+                           int first_grid, WarpRole role, bool longest, cudaStream_t s);
+// Task length histogram of a job: hist[b] += tasks in length bin b (invalid
+// pairs left out).
 cudaError_t launch_length_hist(const Job *jp, int grid, uint32_t *hist, cudaStream_t s);
 // Stratified random sample of a pair table: dst[j] is one pair of the block
 // [j*stride, (j+1)*stride), chosen by a hash of j and seed; m blocks.

@@ -670,20 +670,4 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
     }
 }
 
-// Batched form of the packed kernel (same task source as lockstep_kernel).
-// Blocks of 128 threads.  The registers are capped for 3 blocks per SM with 32
-// or 64 slots per lane, 4 with 16 and 5 with fewer: more warps at fewer
-// registers measured slower (29x, x = 50, first tier: 2x32 at 3, 4 and 5
-// blocks 45.8, 46.0 and 48.8 ms; 4x16 at 4, 5 and 6 blocks 52.0, 54.2 and 57.7).
-template <int C2>
-__host__ __device__ constexpr int packed_min_blocks() { return C2 >= 16 ? 3 : C2 == 8 ? 4 : 5; }
-template <int L, int C2>
-__global__ void __launch_bounds__(kPackedThreads, packed_min_blocks<C2>())
-lockstep16_kernel(const Job *jp, const uint32_t *order, const uint32_t *n_tasks_ptr,
-                  uint32_t *counter, Spill spill, uint32_t one)
-{
-    BatchSrc src{jp, order, *n_tasks_ptr, counter, spill};
-    lockstep16_loop<L, C2>(src, jp->packed, jp->n_words, one);
-}
-
 }  // namespace xd

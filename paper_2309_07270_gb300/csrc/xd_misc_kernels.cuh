@@ -19,19 +19,17 @@ __global__ void validate_kernel(const Job *jp, uint32_t *n_bad)
 }
 
 // ---------------------------------------------------------------------------
-// Length binning (batched form): tasks sorted into bins by
-// ceil(log2(max(m, n) + 1)), bins laid out longest first, so the persistent
-// kernel starts the longest extensions first.
+// Length binning (batched form): tasks sorted into bins by min(m, n), four
+// bins an octave, bins laid out longest first, so the persistent kernel
+// starts the longest extensions first.  A band follows the main diagonal, so
+// the shorter side ends an extension, after about 2 min(m, n) diagonals.
 // ---------------------------------------------------------------------------
-constexpr int NBINS = 32;
 constexpr int BIN_THREADS = 256;
 
 __device__ __forceinline__ int task_bin(const Job &J, uint32_t task)
 {
     Ext e = decode(J, task);
-    if (!e.ok) return -1;
-    uint32_t w = (uint32_t)(e.m > e.n ? e.m : e.n);
-    return 32 - __clz(w);
+    return e.ok ? length_bin((uint32_t)min(e.m, e.n)) : -1;
 }
 
 // hist[b] += tasks in bin b.  Block-local counts first, one global atomic
@@ -54,15 +52,66 @@ bin_count_kernel(const Job *jp, uint32_t *hist)
 }
 
 // offs[b] = start of bin b in the longest-first order; *n_valid = total.
-__global__ void bin_scan_kernel(const uint32_t *hist, uint32_t *offs, uint32_t *n_valid)
+// With a WarpRole, also how many of the longest tasks get a warp each, on how
+// many blocks: a first tier runs the many at rate diagonals per ns, but one
+// of its extensions takes group_ns per diagonal where a warp of its own takes
+// kWarpNs.  Thread b prices the cut behind bin b (all tasks of longer bins
+// to warps) for a few block counts by the longer of the two parts, each the
+// larger of its total work and its longest task; the cheapest wins.  Without
+// `longest` only overflow goes to warps.
+constexpr float kWarpNs = 75.f;  // measured: 57 ns alone on its scheduler
+
+__global__ void __launch_bounds__(NBINS)
+bin_scan_kernel(const uint32_t *hist, uint32_t *offs, uint32_t *n_valid, uint32_t *counter,
+                WarpRole role, bool longest, uint32_t blocks, uint32_t warps_per_block,
+                float rate, float group_ns)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        uint32_t run = 0;
-        for (int b = NBINS - 1; b >= 0; --b) {
-            offs[b] = run;
-            run += hist[b];
+    __shared__ uint32_t h[NBINS];
+    __shared__ unsigned long long best;
+    const int b = threadIdx.x;
+    h[b] = hist[b];
+    if (b == 0) best = ~0ull;
+    __syncthreads();
+    uint32_t before = 0, total = 0;  // tasks of longer bins, of all
+    float d_long = 0.f, d_rest = 0.f, l_long = 0.f, l_rest = 0.f;
+    for (int k = NBINS - 1; k >= 0; --k) {
+        const float l = (float)bin_diagonals(k), d = l * (float)h[k];
+        total += h[k];
+        if (k > b) {
+            before += h[k];
+            d_long += d;
+            if (h[k] && l_long == 0.f) l_long = l;
+        } else {
+            d_rest += d;
+            if (h[k] && l_rest == 0.f) l_rest = l;
         }
-        *n_valid = run;
+    }
+    offs[b] = before;
+    if (b == 0) {
+        *n_valid = total;
+        *counter = 0;
+    }
+    if (!role.n_long) return;
+    // cost (ns), then the block count's index and the cut, in one word
+    unsigned long long mine = ~0ull;
+    const uint32_t share[6] = {blocks / 128, blocks / 24, blocks / 6,
+                               blocks / 3,   blocks / 2,  blocks * 2 / 3};
+    for (int k = 0; k < (longest ? 6 : 1); ++k) {
+        const float nb = (float)max(share[k], 1u), nw = nb * (float)warps_per_block;
+        const float t_long = fmaxf(l_long * kWarpNs, d_long * kWarpNs / nw);
+        const float t_rest = fmaxf(d_rest / rate + t_long * nb / (float)blocks, l_rest * group_ns);
+        const float cost = fminf(fmaxf(t_long, t_rest), 1e18f);
+        const unsigned long long w = ((unsigned long long)cost << 12) |
+                                     ((unsigned long long)k << 8) | (unsigned long long)(NBINS - 1 - b);
+        mine = w < mine ? w : mine;
+    }
+    if (!longest && b < NBINS - 1) mine = ~0ull;  // no cut: overflow only
+    atomicMin(&best, mine);
+    __syncthreads();
+    if (mine == best) {  // the bin and block count make the word unique
+        *role.n_long = before;
+        *role.n_blocks = max(share[(best >> 8) & 15], 1u);
+        *counter = before;
     }
 }
 

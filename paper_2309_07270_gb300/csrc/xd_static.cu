@@ -67,9 +67,9 @@ static_warp_kernel(Job J, int64_t per_cta)
             continue;
         }
         int32_t sc, bi, bj;
-        const int st = extend_warp(e, J.sc, false, lane, sc, bi, bj);
+        const int st = extend_warp(e, J.sc, 0, lane, sc, bi, bj);
         if (lane == 0) {
-            if (st == 2) atomicOr(&o[6], kWideLeft << e.side);
+            if (st < 0) atomicOr(&o[6], kWideLeft << e.side);
             else write_result(J, e, sc, bi, bj);
         }
         __syncwarp();

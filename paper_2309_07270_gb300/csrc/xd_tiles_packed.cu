@@ -5,23 +5,162 @@
 // against 45.0 ms, 29x, x = 50: twice the events per warp, half the warps).
 #include "xd_launch.h"
 #include "xd_serve_kernels.cuh"
+#include "xd_warp16.cuh"
 
 namespace xd {
 
-template <class K>
-static cudaError_t launch_impl(K kernel, int grid, const Job *jp, const uint32_t *order,
-                               const uint32_t *n, uint32_t *ctr, Spill sp, cudaStream_t s)
+// The single-extension part of a group tier's kernel (WarpRole): first the
+// n_long longest tasks of the order, then the tier's overflow, with wait
+// until the tier is done or none came for kRoleIdleNs (the warp then joins
+// the tier), else what there is now.  Entries of the overflow list start as
+// kNoTask and appear right after their position was reserved, so the wait
+// for one is short; it is bounded all the same.
+constexpr unsigned long long kRoleIdleNs = 300000;
+constexpr int kEntryTries = 1 << 20;
+
+static __device__ __noinline__ void run_warp_role(const Job *jp, const uint32_t *order, Spill spill,
+                                           WarpRole role, uint32_t n_long, int width, bool wait,
+                                           uint32_t first_warps)
+{
+    const Job J = *jp;
+    const int lane = threadIdx.x & 31;
+    bool longest = n_long > 0;
+    const uint32_t all_warps = gridDim.x * (blockDim.x >> 5);
+    unsigned long long idle = 0;
+    for (;;) {
+        enum { kAgain = 0, kTask = 1, kLeave = 2 };
+        int act = kAgain;
+        uint32_t task = kNoTask;
+        if (lane == 0) {
+            if (longest) {
+                const uint32_t k = atomicAdd(role.long_ctr, 1u);
+                if (k < n_long) {
+                    task = order[k];
+                    act = kTask;
+                } else {
+                    longest = false;
+                }
+            }
+            if (act == kAgain) {
+                // done before count: what the last warp handed on is seen
+                const uint32_t done = *(volatile uint32_t *)role.done;
+                __threadfence();
+                uint32_t t = *(volatile uint32_t *)role.taken;
+                bool empty = false;
+                for (int tries = 0; tries < 4 && act == kAgain; ++tries) {
+                    const uint32_t count = *(volatile uint32_t *)spill.count;
+                    if (t >= count) {
+                        empty = true;
+                        break;
+                    }
+                    // An add claims an entry for certain while there are more
+                    // than warps that can add at once; near the end a
+                    // compare-and-swap, which loses to every other claim.
+                    uint32_t got;
+                    if (count - t > all_warps) got = t = atomicAdd(role.taken, 1u);
+                    else got = atomicCAS(role.taken, t, t + 1);
+                    if (got == t) {
+                        for (int spin = 0; spin < kEntryTries && task == kNoTask; ++spin) {
+                            task = *(volatile uint32_t *)&spill.list[t];
+                            if (task == kNoTask) __nanosleep(32);
+                        }
+                        if (task == kNoTask) *role.err = 1u;
+                        act = kTask;
+                    }
+                    t = got;
+                }
+                if (act == kAgain && empty) {
+                    if (!wait || done >= first_warps) {
+                        act = kLeave;
+                    } else {
+                        unsigned long long now;
+                        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                        if (idle == 0) idle = now;
+                        if (now - idle > kRoleIdleNs) act = kLeave;
+                        else __nanosleep(1000);
+                    }
+                } else if (act == kAgain) {
+                    __nanosleep(200 + 37 * (blockIdx.x & 31));  // lost every race
+                }
+            }
+        }
+        act = __shfl_sync(FULL, act, 0);
+        if (act == kLeave) return;
+        if (act == kAgain) continue;
+        idle = 0;
+        task = __shfl_sync(FULL, task, 0);
+        const bool whole = __shfl_sync(FULL, (int)longest, 0) != 0;
+        if (task == kNoTask) continue;
+        const Ext e = decode(J, task);
+        if (!e.ok) continue;
+        int32_t sc, bi, bj;
+        const int st = extend_warp(e, J.sc, whole ? 0 : width, lane, sc, bi, bj);
+        if (lane == 0) {
+            if (whole && st) atomicAdd(role.grown, 1u);
+            if (st < 0) role.wide.list[atomicAdd(role.wide.count, 1u)] = task;
+            else write_result(J, e, sc, bi, bj);
+        }
+        __syncwarp();
+    }
+}
+
+// Batched form of the packed kernel (same task source as lockstep_kernel).
+// With a WarpRole the first blocks give their warps to single extensions
+// first: a launch ends with its longest extension, and one that outgrew the
+// window would start over only after the launch.  Every warp that runs out of
+// tasks takes overflow too, so none is left when the kernel ends (short
+// overflow, which can be plentiful, goes to `brief`, the tasks of a second,
+// wider group tier: a warp each costs it four times as much).
+// Blocks of 128 threads.  The registers are capped for 3 blocks per SM with 32
+// or 64 slots per lane, 4 with 16 and 5 with fewer: more warps at fewer
+// registers measured slower (29x, x = 50, first tier: 2x32 at 3, 4 and 5
+// blocks 45.8, 46.0 and 48.8 ms; 4x16 at 4, 5 and 6 blocks 52.0, 54.2 and 57.7).
+template <int C2>
+__host__ __device__ constexpr int packed_min_blocks() { return C2 >= 16 ? 3 : C2 == 8 ? 4 : 5; }
+template <int L, int C2>
+__global__ void __launch_bounds__(kPackedThreads, packed_min_blocks<C2>())
+lockstep16_kernel(const Job *jp, const uint32_t *order, const uint32_t *n_tasks_ptr,
+                  uint32_t *counter, Spill spill, Spill brief, uint32_t one, WarpRole role)
+{
+    constexpr int W = L * 2 * C2;
+    const uint32_t n_tasks = *n_tasks_ptr;
+    if (role.n_long) {
+        const uint32_t mine = *role.n_blocks;
+        const bool all = n_tasks <= role.few;
+        if (all || blockIdx.x < mine)
+            run_warp_role(jp, order, spill, role, all ? n_tasks : *role.n_long, all ? W / 2 : W,
+                          !all, (gridDim.x - mine) * (kPackedThreads / 32));
+        if (all) return;
+    }
+    BatchSrc src{jp, order, n_tasks, counter, spill, brief};
+    lockstep16_loop<L, C2>(src, jp->packed, jp->n_words, one);
+    if (role.n_long) {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0 && blockIdx.x >= *role.n_blocks) {
+            __threadfence();  // this warp's overflow entries before its count
+            atomicAdd(role.done, 1u);
+        }
+        run_warp_role(jp, order, spill, role, 0, W, false, 0);
+    }
+}
+
+template <int L, int C2>
+static cudaError_t abs_impl(int grid, const Job *jp, const uint32_t *order, const uint32_t *n,
+                            uint32_t *ctr, Spill sp, cudaStream_t s)
 {
     (void)cudaGetLastError();
-    kernel<<<grid, kPackedThreads, 0, s>>>(jp, order, n, ctr, sp, 1u);
+    lockstep16_abs_kernel<L, C2><<<grid, kPackedThreads, 0, s>>>(jp, order, n, ctr, sp, 1u);
     return cudaGetLastError();
 }
 
 template <int L, int C2>
 static cudaError_t packed_impl(int grid, const Job *jp, const uint32_t *order, const uint32_t *n,
-                               uint32_t *ctr, Spill sp, cudaStream_t s)
+                               uint32_t *ctr, Spill sp, Spill brief, WarpRole role,
+                               cudaStream_t s)
 {
-    return launch_impl(lockstep16_kernel<L, C2>, grid, jp, order, n, ctr, sp, s);
+    (void)cudaGetLastError();
+    lockstep16_kernel<L, C2><<<grid, kPackedThreads, 0, s>>>(jp, order, n, ctr, sp, brief, 1u, role);
+    return cudaGetLastError();
 }
 
 template <class K>
@@ -39,27 +178,25 @@ static int packed_occupancy_impl()
 }
 
 cudaError_t launch_persistent_packed(Tile t, int grid, const Job *jp, const uint32_t *order,
-                                     const uint32_t *n, uint32_t *ctr, Spill sp,
-                                     cudaStream_t s, bool *handled)
+                                     const uint32_t *n, uint32_t *ctr, Spill sp, Spill brief,
+                                     WarpRole role, cudaStream_t s, bool *handled)
 {
     *handled = true;
     if (t.packed) {
         if (t.absolute && t.c == 32) {
-            if (t.lanes == 2)
-                return launch_impl(lockstep16_abs_kernel<2, 16>, grid, jp, order, n, ctr, sp, s);
-            if (t.lanes == 4)
-                return launch_impl(lockstep16_abs_kernel<4, 16>, grid, jp, order, n, ctr, sp, s);
+            if (t.lanes == 2) return abs_impl<2, 16>(grid, jp, order, n, ctr, sp, s);
+            if (t.lanes == 4) return abs_impl<4, 16>(grid, jp, order, n, ctr, sp, s);
         }
-        if (t.lanes == 4 && t.c == 8) return packed_impl<4, 4>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 2 && t.c == 16) return packed_impl<2, 8>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 4 && t.c == 16) return packed_impl<4, 8>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 8 && t.c == 8) return packed_impl<8, 4>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 8 && t.c == 16) return packed_impl<8, 8>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 16 && t.c == 8) return packed_impl<16, 4>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 2 && t.c == 32) return packed_impl<2, 16>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 4 && t.c == 32) return packed_impl<4, 16>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 1 && t.c == 32) return packed_impl<1, 16>(grid, jp, order, n, ctr, sp, s);
-        if (t.lanes == 2 && t.c == 64) return packed_impl<2, 32>(grid, jp, order, n, ctr, sp, s);
+        if (t.lanes == 4 && t.c == 8) return packed_impl<4, 4>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 2 && t.c == 16) return packed_impl<2, 8>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 4 && t.c == 16) return packed_impl<4, 8>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 8 && t.c == 8) return packed_impl<8, 4>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 8 && t.c == 16) return packed_impl<8, 8>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 16 && t.c == 8) return packed_impl<16, 4>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 2 && t.c == 32) return packed_impl<2, 16>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 4 && t.c == 32) return packed_impl<4, 16>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 1 && t.c == 32) return packed_impl<1, 16>(grid, jp, order, n, ctr, sp, brief, role, s);
+        if (t.lanes == 2 && t.c == 64) return packed_impl<2, 32>(grid, jp, order, n, ctr, sp, brief, role, s);
     }
     *handled = false;
     return cudaSuccess;
@@ -112,6 +249,17 @@ Tile usable_tile(Tile t, const Scoring &sc)
     if (t.width() < 64) return Tile{4, 16, false};  // no 32-bit tile this narrow
     if (t.c >= 32) return Tile{h.lanes, 16, false};
     return Tile{t.lanes, t.c, false};
+}
+
+bool has_warp_role(Tile t) { return t.packed && !t.absolute; }
+
+// What the price of a cut between single warps and groups (bin_scan_kernel)
+// takes from the tile: diagonals per ns of a full first tier (about 5,000
+// window slots per ns) and the ns per diagonal of one of its extensions.
+void tile_rates(Tile t, float *rate, float *group_ns)
+{
+    *rate = 5000.f / (float)t.width();
+    *group_ns = 40.f + 9.f * (float)t.c;
 }
 
 int persistent_block_threads(Tile t) { return t.packed ? kPackedThreads : 256; }

@@ -13,7 +13,7 @@ namespace xd {
 // pairs are validated as validate_kernel does.
 __global__ void __launch_bounds__(kWarpThreads)
 warp_kernel(const Job *jp, const uint32_t *list, const uint32_t *n_ptr, uint32_t *counter,
-            bool skip128, uint32_t *n_bad, Spill over, Spill out)
+            int from, uint32_t *n_bad, Spill over, Spill out)
 {
     const Job J = *jp;
     const int lane = threadIdx.x & 31;
@@ -28,20 +28,20 @@ warp_kernel(const Job *jp, const uint32_t *list, const uint32_t *n_ptr, uint32_t
         if (n_bad && e.side == 0 && lane == 0) write_status(J, e.pair, e.ok, n_bad);
         if (!e.ok) continue;
         int32_t sc, bi, bj;
-        const int st = extend_warp(e, J.sc, skip128, lane, sc, bi, bj);
+        const int st = extend_warp(e, J.sc, from, lane, sc, bi, bj);
         if (lane == 0) {
             if (!list && st) over.list[atomicAdd(over.count, 1u)] = task;
-            if (st == 2) out.list[atomicAdd(out.count, 1u)] = task;
+            if (st < 0) out.list[atomicAdd(out.count, 1u)] = task;
             else write_result(J, e, sc, bi, bj);
         }
         __syncwarp();
     }
 }
 
-bool warp_packed(const Scoring &sc) { return warp16_ok(sc); }
+bool warp_packed(const Scoring &sc) { return warp16_ok<2>(sc); }
 
 cudaError_t launch_warp(uint64_t n_tasks, int sm_count, const Job *jp, const uint32_t *list,
-                        const uint32_t *n_ptr, uint32_t *counter, bool skip128, uint32_t *n_bad,
+                        const uint32_t *n_ptr, uint32_t *counter, int from, uint32_t *n_bad,
                         Spill over, Spill out, cudaStream_t s)
 {
     // a warp per task, in blocks of one warp while there are few (every
@@ -51,7 +51,7 @@ cudaError_t launch_warp(uint64_t n_tasks, int sm_count, const Job *jp, const uin
     const uint64_t blocks = std::min<uint64_t>((n_tasks + warps - 1) / warps, cap);
     if (!blocks) return cudaSuccess;
     (void)cudaGetLastError();
-    warp_kernel<<<(unsigned)blocks, threads, 0, s>>>(jp, list, n_ptr, counter, skip128, n_bad, over,
+    warp_kernel<<<(unsigned)blocks, threads, 0, s>>>(jp, list, n_ptr, counter, from, n_bad, over,
                                                      out);
     return cudaGetLastError();
 }

@@ -43,15 +43,19 @@ cudaError_t launch_validate(const Job *jp, uint64_t n_pairs, uint32_t *n_bad, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_binning(const Job *jp, uint64_t n_pairs, int grid, uint32_t *hist,
-                           uint32_t *offs, uint32_t *n_valid, uint32_t *order, cudaStream_t s)
+cudaError_t launch_binning(const Job *jp, int grid, uint32_t *hist, uint32_t *offs,
+                           uint32_t *n_valid, uint32_t *counter, uint32_t *order, Tile t,
+                           int first_grid, WarpRole role, bool longest, cudaStream_t s)
 {
-    (void)n_pairs;
+    float rate = 1.f, group_ns = 1.f;
+    tile_rates(t, &rate, &group_ns);
     (void)cudaGetLastError();
     bin_count_kernel<<<grid, BIN_THREADS, 0, s>>>(jp, hist);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    bin_scan_kernel<<<1, 32, 0, s>>>(hist, offs, n_valid);
+    bin_scan_kernel<<<1, NBINS, 0, s>>>(hist, offs, n_valid, counter, role, longest,
+                                        (uint32_t)first_grid,
+                                        (uint32_t)persistent_block_threads(t) / 32, rate, group_ns);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     bin_scatter_kernel<<<grid, BIN_THREADS, 0, s>>>(jp, offs, order);
@@ -128,7 +132,7 @@ cudaError_t launch_persistent_mid(Tile, int, const Job *, const uint32_t *, cons
 int occupancy_narrow(Tile);
 int occupancy_mid(Tile);
 cudaError_t launch_persistent_packed(Tile, int, const Job *, const uint32_t *, const uint32_t *,
-                                     uint32_t *, Spill, cudaStream_t, bool *);
+                                     uint32_t *, Spill, Spill, WarpRole, cudaStream_t, bool *);
 int occupancy_packed(Tile);
 cudaError_t launch_serve_packed(Tile, int, const ServeArgs &, const uint32_t *, int64_t,
                                 cudaStream_t, bool *);
@@ -181,13 +185,13 @@ cudaError_t launch_window(Tile t, bool count, const Job *jp, uint32_t task_base,
 }
 
 cudaError_t launch_persistent(Tile t, int grid, const Job *jp, const uint32_t *order,
-                              const uint32_t *n_tasks, uint32_t *counter, Spill spill,
-                              cudaStream_t s)
+                              const uint32_t *n_tasks, uint32_t *counter, Spill spill, Spill brief,
+                              WarpRole role, cudaStream_t s)
 {
     bool handled = false;
     if (t.packed) {
-        cudaError_t e = launch_persistent_packed(t, grid, jp, order, n_tasks, counter, spill, s,
-                                                 &handled);
+        cudaError_t e = launch_persistent_packed(t, grid, jp, order, n_tasks, counter, spill, brief,
+                                                 role, s, &handled);
         return handled ? e : cudaErrorInvalidValue;
     }
     cudaError_t e = launch_persistent_narrow(t, grid, jp, order, n_tasks, counter, spill, s,

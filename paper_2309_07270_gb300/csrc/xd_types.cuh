@@ -47,11 +47,46 @@ struct Job {
     uint32_t tag;
 };
 
+// Length bins: four an octave of min(m, n), the last one for 2^28 and more.
+constexpr int NBINS = 128;
+
+__host__ __device__ inline int length_bin(uint32_t w)
+{
+    if (w < 4) return (int)w;
+    int lg = 0;
+    for (uint32_t v = w; v > 1; v >>= 1) ++lg;
+    return 4 * lg + (int)((w >> (lg - 2)) & 3u);
+}
+
+// Diagonals of the longest extension of a bin (about).
+__host__ __device__ inline double bin_diagonals(int b)
+{
+    if (b < 8) return 2.0 * (b < 4 ? b : 3);
+    return 2.0 * (double)((uint64_t)(5 + b % 4) << (b / 4 - 2));
+}
+
 // Overflow hand-off between tiers.
 struct Spill {
     uint32_t *list;   // task ids
     uint32_t *count;  // number of ids in list
 };
+
+// Device words of a batched launch whose first blocks give a warp to single
+// extensions (xd_tiles_packed.cu): the longest tasks of the order, then the
+// first tier's overflow while the first tier still runs.
+struct WarpRole {
+    uint32_t *n_long;    // tasks at the head of the order for single warps
+    uint32_t *n_blocks;  // blocks that start with them
+    uint32_t *long_ctr;  // next of those tasks
+    uint32_t *taken;     // overflow entries taken
+    uint32_t *done;      // first-tier warps that found no more tasks
+    uint32_t *grown;     // longest tasks that outgrew a warp's first window
+    uint32_t *err;       // set when an overflow entry never appeared
+    Spill wide;          // tasks for the unbounded tier
+    uint32_t few;        // up to this many tasks all go to single warps
+};
+constexpr int32_t kBriefDiagonals = 2048;  // overflow up to this long goes to a second group tier
+constexpr uint32_t kNoTask = 0xFFFFFFFFu;  // overflow entry not written yet
 
 // One base stream c_k (k >= 1): c_k is base s0 + dir*(k-1) of the packed
 // buffer.
