@@ -230,6 +230,14 @@ Spill spill_of(xdrop_ctx *c, int k)
     return Spill{(uint32_t *)c->spill[k].p, c->d_ctrs + C_SPILL0 + k};
 }
 
+// The scoring that decides the tiles of a job: the kernels run every scoring
+// as its effective() one, which fits 16 bits more often (a mismatch below
+// two gaps).  A forced tile is judged by the scoring as given.
+Scoring tile_scoring(const xdrop_ctx *c, const Scoring &sc)
+{
+    return c->forced.lanes ? sc : effective(sc);
+}
+
 // The tiers after a first tier of width w: a warp per extension (the wider
 // ones of windows of 128, 256 and 512 slots), then the unbounded tier.
 int enqueue_wider(xdrop_ctx *c, int w, uint64_t n_tasks)
@@ -322,6 +330,7 @@ int pick_tile(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *out);
 int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
 {
     cudaStream_t s = c->stream;
+    const Scoring sc = tile_scoring(c, job.sc);
     // Scorings that fit 16 bits choose among the packed tiles only (each is
     // faster than the 32-bit tile of its shape), on a third of the job so
     // the end of the sample, where few extensions are left, does not decide
@@ -334,7 +343,7 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     // (48 bytes per sampled pair, at most 16 of the 28 bytes per pair there),
     // so tuning needs no memory beyond the submit's; the buffer is zeroed
     // afterwards, before validation writes the status words.
-    const bool packed = packed_scoring_ok(job.sc);
+    const bool packed = packed_scoring_ok(sc);
     const uint32_t stride = job.n_pairs <= 3 * 4096 ? 1u : (packed ? 3u : 8u);
     const uint64_t m = (job.n_pairs + stride - 1) / stride;
     Job js = job;
@@ -356,22 +365,22 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     // a live band spans at most about x / |gap| slots.  A window under 3/4 of
     // that overflows too often to win, one over 3 times it computes mostly
     // dead slots.
-    const int64_t span = job.sc.x / -(int64_t)job.sc.gap;
+    const int64_t span = sc.x / -(int64_t)sc.gap;
     const int64_t min_w = std::min<int64_t>(128, span * 3 / 4);
     const int64_t max_w = std::max<int64_t>(64, span * 3);
     // Lanes of 32 slots beat 4x8, 8x8 and 4x16 wherever they hold the scoring
     // (29x, first tier: x = 15 4x8 42.1, 1x32 23.0 ms; x = 50 8x8 83.4, 4x16
     // 51.6, 2x32 45.0), and 8x16 beats 16x8 (1M uneven pairs 18.6, 25.3 ms).
-    const bool long_lanes = packed && has_warp_role(in_frame(Tile{2, 32, true}, job.sc)) &&
-                            packed_tile_ok(Tile{2, 32, true}, job.sc);
+    const bool long_lanes = packed && has_warp_role(in_frame(Tile{2, 32, true}, sc)) &&
+                            packed_tile_ok(Tile{2, 32, true}, sc);
     float best_ms = 1e30f;
     *best = Tile{0, 0};
     std::vector<Tile> cands;
     if (packed) cands.assign(std::begin(kPackedTiles), std::end(kPackedTiles));
     else cands.assign(std::begin(kTuneTiles), std::end(kTuneTiles));
     for (const Tile &cand : cands) {
-        if (cand.packed && !packed_tile_ok(cand, job.sc)) continue;
-        const Tile t = in_frame(cand, job.sc);
+        if (cand.packed && !packed_tile_ok(cand, sc)) continue;
+        const Tile t = in_frame(cand, sc);
         if (t.width() < min_w || t.width() > max_w) continue;
         if (long_lanes && (t.c < 16 || (t.c == 16 && t.lanes == 4))) continue;
         const int bps = persistent_blocks_per_sm(t);
@@ -380,7 +389,7 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
         for (int rep = 0; rep < 2; ++rep) {
             if (rep && tmin > 1.25f * best_ms) break;  // far behind after one run
             CK(cudaEventRecord(e0, s));
-            int rc = enqueue_batched(c, t, bps, job.sc, false, nullptr);
+            int rc = enqueue_batched(c, t, bps, sc, false, nullptr);
             if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
             CK(cudaEventRecord(e1, s));
             CK(cudaEventSynchronize(e1));
@@ -426,14 +435,15 @@ int length_bucket(xdrop_ctx *c, Ticket *tk, int *bucket)
 
 int pick_tile(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *out)
 {
+    const Scoring sc = tile_scoring(c, job.sc);
     Tile t = c->forced;
     if (t.lanes) {
-        *out = usable_tile(t, job.sc);
+        *out = usable_tile(t, sc);
         return XDROP_OK;
     }
     int bucket = 0;
     if (int rc = length_bucket(c, tk, &bucket)) return rc;
-    auto key = std::make_tuple(job.sc.match, job.sc.mismatch, job.sc.gap, job.sc.x, bucket);
+    auto key = std::make_tuple(sc.match, sc.mismatch, sc.gap, sc.x, bucket);
     auto it = c->tuned.find(key);
     if (it != c->tuned.end()) {
         *out = it->second;
@@ -491,7 +501,8 @@ int run_plain(xdrop_ctx *c, Ticket *tk, const Job &job)
     cudaStream_t s = c->stream;
     const uint64_t n_pairs = job.n_pairs;
     CK(cudaMemsetAsync(c->d_ctrs, 0, C_NBAD * 4, s));
-    const Tile t0 = usable_tile(c->forced.lanes ? c->forced : Tile{4, 16, true}, job.sc);
+    const Tile t0 = usable_tile(c->forced.lanes ? c->forced : Tile{4, 16, true},
+                                tile_scoring(c, job.sc));
     c->tile0 = t0;
     const int bps = persistent_blocks_per_sm(t0);
     if (bps <= 0) return fail(XDROP_ECUDA, "tile %dx%d not available", t0.lanes, t0.c);
@@ -525,7 +536,7 @@ bool is_small(const xdrop_ctx *c, uint64_t n_pairs)
 int run_small(xdrop_ctx *c, Ticket *tk, const Job &job)
 {
     cudaStream_t s = c->stream;
-    c->tile0 = Tile{32, 4, warp_packed(job.sc)};
+    c->tile0 = Tile{32, 4, warp_packed(effective(job.sc))};
     CK(cudaMemsetAsync(c->d_ctrs, 0, C_MAXLEN * 4, s));
     CK(launch_warp(2 * job.n_pairs, c->sm_count, c->d_job, nullptr, nullptr, c->d_ctrs + C_WARP, 0,
                    tk->device_submit ? c->d_ctrs + C_NBAD : nullptr, spill_of(c, 0),
@@ -572,7 +583,7 @@ int launch_ticket(xdrop_ctx *c, Ticket *tk, const Job &job, uint32_t maxlen)
     if (job.n_pairs) {
         if (small) rc = run_small(c, tk, job);
         else if (c->mode == XDROP_MODE_PLAIN) rc = run_plain(c, tk, job);
-        else rc = run_batched(c, tk, job.sc);
+        else rc = run_batched(c, tk, tile_scoring(c, job.sc));
         if (rc) return rc;
     }
     CK(cudaEventRecord(tk->ev_end, s));
@@ -611,7 +622,7 @@ int launch_ticket_chunked(xdrop_ctx *c, Ticket *tk, const xdrop_pair *h_pairs, s
         if (k == 0) {  // first tile: as for an unchunked submit
             if ((rc = pick_tile(c, tk, job, &c->tile0))) return rc;
         }
-        if ((rc = run_batched(c, tk, job.sc))) return rc;
+        if ((rc = run_batched(c, tk, tile_scoring(c, job.sc)))) return rc;
         CK(cudaMemcpyAsync(tk->h_out + p0, d_out, np * sizeof(xdrop_result), cudaMemcpyDeviceToHost, s));
     }
     CK(cudaEventRecord(tk->ev_end, s));

@@ -557,7 +557,7 @@ struct BatchSrc {
     __device__ __forceinline__ bool aborted() const { return false; }
     __device__ __forceinline__ Ext open(const Job *gj, uint32_t task, Scoring &sc)
     {
-        sc = gj->sc;
+        sc = effective(gj->sc);
         return decode(*gj, task);
     }
     // called by the group leader only

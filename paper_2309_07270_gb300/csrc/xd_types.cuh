@@ -121,6 +121,19 @@ __host__ __device__ inline int32_t max_abs_score(const Scoring &s)
     return m > c ? m : c;
 }
 
+// The scoring with a mismatch worth no less than two gaps: the same scores,
+// positions and live cells.  If H(i-1,j-1) + 2 gap reaches the threshold of
+// diagonal d, then H(i-1,j-1) + gap, larger, reaches the one of d-1, which is
+// no larger: cell (i-1,j), inside the rectangle like (i,j), is live with at
+// least that value and offers (i,j) at least H(i-1,j-1) + 2 gap.  So a
+// mismatch below two gaps never decides a live cell, and raising it to two
+// gaps offers nothing that is not offered already.
+__host__ __device__ inline Scoring effective(Scoring s)
+{
+    if (s.mismatch < 2 * s.gap) s.mismatch = 2 * s.gap;
+    return s;
+}
+
 // n_words: words of the reads themselves (without reverse complements);
 // rc_ok: whether a pair may ask for the reverse strand of b.
 __host__ __device__ inline bool pair_ok(const Pair &p, uint32_t n_reads,

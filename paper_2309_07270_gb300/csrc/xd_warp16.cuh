@@ -283,9 +283,10 @@ __device__ __forceinline__ int extend_warp16(const Ext &e, const Scoring sc, int
 // scoring fits, else 32-bit), 256 (packed scorings only) and 512 slots
 // (32-bit), from the first that is wider than `from` slots.  Returns how many
 // of them the band outgrew, or -1 for all.
-__device__ __forceinline__ int extend_warp(const Ext &e, const Scoring &sc, int from, int lane,
+__device__ __forceinline__ int extend_warp(const Ext &e, const Scoring &s, int from, int lane,
                                            int32_t &best, int32_t &bi, int32_t &bj)
 {
+    const Scoring sc = effective(s);
     int64_t cells;
     int grown = 0;
     if (from < 128) {
