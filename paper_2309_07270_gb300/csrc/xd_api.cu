@@ -995,9 +995,9 @@ int xdrop_load_reads(xdrop_ctx *c, const uint32_t *packed, const uint64_t *read_
         rr.read_len = (const uint32_t *)c->r_len.p;
         rr.n_reads = n_reads;
         std::string err;
-        // Packed 4x16 unless a tile was forced; requests whose scoring does
-        // not fit 16 bits run on the serving kernel's 32-bit second tier.
-        const Tile t = c->forced.lanes ? c->forced : Tile{4, 16, true};
+        // Packed 2x32 unless a tile was forced; requests whose scoring does
+        // not fit it run on the serving kernel's 32-bit second tier.
+        const Tile t = c->forced.lanes ? c->forced : Tile{2, 32, true};
         c->srv = xd::server_create(c->device, c->sm_count, c->budget, t, rr, c->h_len.data(),
                                    (int32_t *)c->wide.p, c->wide_per_cta, c->wide_grid,
                                    c->serve_idle_ns, err);

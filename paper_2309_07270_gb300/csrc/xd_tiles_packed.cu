@@ -281,6 +281,15 @@ static int serve16_occupancy_impl()
     return b;
 }
 
+// The ring warps' tile: 2x32 as it is (75 requests of 1,000 to 20,000 pairs of
+// 29x reads, x = 50: 163 ms, and 172 ms with 4x16), other lanes of 32 and
+// more slots as the 16-slot tile of their width.
+static Tile serve_tile(Tile t)
+{
+    if (t.c <= 16 || (t.lanes == 2 && t.c == 32)) return t;
+    return Tile{t.width() / 16, 16, true};
+}
+
 // Second tier as for the 32-bit tiles: 16x8 after a 64-slot first tier,
 // 32x16 after a 128-slot one.
 cudaError_t launch_serve_packed(Tile t, int grid, const ServeArgs &a, const uint32_t *pk,
@@ -288,8 +297,8 @@ cudaError_t launch_serve_packed(Tile t, int grid, const ServeArgs &a, const uint
 {
     *handled = true;
     if (t.packed) {
-        // lanes of 32 slots serve as the 16-slot tile of the same width
-        if (t.c == 32) t = Tile{2 * t.lanes, 16, true};
+        t = serve_tile(t);
+        if (t.lanes == 2 && t.c == 32) return serve16_impl<2, 16, 16, 8>(grid, a, pk, nw, s);
         if (t.lanes == 4 && t.c == 16) return serve16_impl<4, 8, 16, 8>(grid, a, pk, nw, s);
         if (t.lanes == 8 && t.c == 8) return serve16_impl<8, 4, 16, 8>(grid, a, pk, nw, s);
         if (t.lanes == 8 && t.c == 16) return serve16_impl<8, 8, 32, 16>(grid, a, pk, nw, s);
@@ -302,7 +311,8 @@ cudaError_t launch_serve_packed(Tile t, int grid, const ServeArgs &a, const uint
 int serve_occupancy_packed(Tile t)
 {
     if (!t.packed) return -1;
-    if (t.c == 32) t = Tile{2 * t.lanes, 16, true};
+    t = serve_tile(t);
+    if (t.lanes == 2 && t.c == 32) return serve16_occupancy_impl<2, 16, 16, 8>();
     if (t.lanes == 4 && t.c == 16) return serve16_occupancy_impl<4, 8, 16, 8>();
     if (t.lanes == 8 && t.c == 8) return serve16_occupancy_impl<8, 4, 16, 8>();
     if (t.lanes == 8 && t.c == 16) return serve16_occupancy_impl<8, 8, 32, 16>();
