@@ -220,7 +220,7 @@ int xdrop_get_serve_stats(xdrop_ctx *c, xdrop_serve_stats *st);
  * no work waits at most idle_ns nanoseconds (default 5 s; 0 restores it),
  * then its warp leaves and counts itself in idle_exits; the kernel ends
  * when every warp has left, and the next request launches it again.  The
- * host normally stops an idle kernel after about 50 ms, so the bound only
+ * host normally stops an idle kernel after about 10 ms, so the bound only
  * matters if that stop never arrives.  Takes effect at the next launch of
  * the serving kernel.  Returns XDROP_OK, or XDROP_EINVAL for a NULL c. */
 int xdrop_set_serve_idle(xdrop_ctx *c, uint64_t idle_ns);

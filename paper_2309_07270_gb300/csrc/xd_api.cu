@@ -98,6 +98,7 @@ struct Ticket {
     void *d_mem = nullptr;        // inputs + results (host submit)
     size_t d_bytes = 0;
     void *h_pinned = nullptr;     // results staging + counters + job
+    size_t pin_bytes = 0;
     cudaEvent_t ev_begin = nullptr, ev_end = nullptr, ev_done = nullptr;
     uint32_t launches = 0, graph_replays = 0;
     uint32_t *h_ctrs = nullptr;   // copy of the counter block at the end
@@ -115,6 +116,7 @@ struct xdrop_ctx {
     cudaStream_t stream = nullptr;
     std::mutex mu;
     std::unordered_map<uint64_t, Ticket *> tickets;
+    std::vector<Ticket *> idle;  // done tickets whose buffers the next ones take
     uint64_t next_id = 1;
     size_t used = 0;  // device bytes held (scratch + tickets)
 
@@ -156,6 +158,7 @@ struct xdrop_ctx {
     xd::Server *srv = nullptr;
     uint64_t serve_idle_ns = 0;  // xdrop_set_serve_idle (0: the default)
 
+    cudaMemPool_t pool = nullptr;  // seed discovery's tables (seed_pool)
     // the last seed discovery result (xdrop_find_candidates)
     std::vector<Pair> cand_pairs;
     std::vector<uint32_t> cand_shared;
@@ -242,7 +245,7 @@ Scoring tile_scoring(const xdrop_ctx *c, const Scoring &sc)
 // ones of windows of 128, 256 and 512 slots), then the unbounded tier.
 int enqueue_wider(xdrop_ctx *c, int w, uint64_t n_tasks)
 {
-    CK(launch_warp(n_tasks, c->sm_count, c->d_job, spill_of(c, 0).list, spill_of(c, 0).count,
+    CK(launch_warp(n_tasks, c->sm_count, c->d_job, nullptr, spill_of(c, 0).list, spill_of(c, 0).count,
                    c->d_ctrs + C_WARP, w, nullptr, Spill{}, spill_of(c, 1), c->stream));
     CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
                    c->wide_per_cta, c->stream));
@@ -332,10 +335,10 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     cudaStream_t s = c->stream;
     const Scoring sc = tile_scoring(c, job.sc);
     // Scorings that fit 16 bits choose among the packed tiles only (each is
-    // faster than the 32-bit tile of its shape), on a third of the job so
-    // the end of the sample, where few extensions are left, does not decide
-    // between tiles of different concurrency; other scorings time the
-    // 32-bit tiles on an eighth.  The sample is stratified and random (one
+    // faster than the 32-bit tile of its shape), on the whole job, or a third
+    // of a large one, so that the end of the sample, where few extensions are
+    // left, does not decide between tiles of different concurrency; other
+    // scorings time the 32-bit tiles on an eighth.  The sample is stratified and random (one
     // pair out of every block of 3 or 8, seeded), so it has the job's
     // length mix even when the input is sorted or clustered.
     //
@@ -344,7 +347,8 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     // so tuning needs no memory beyond the submit's; the buffer is zeroed
     // afterwards, before validation writes the status words.
     const bool packed = packed_scoring_ok(sc);
-    const uint32_t stride = job.n_pairs <= 3 * 4096 ? 1u : (packed ? 3u : 8u);
+    const uint64_t whole = packed ? 150000 : 3 * 4096;  // jobs timed as they are
+    const uint32_t stride = job.n_pairs <= whole ? 1u : (packed ? 3u : 8u);
     const uint64_t m = (job.n_pairs + stride - 1) / stride;
     Job js = job;
     if (stride > 1) {
@@ -538,7 +542,7 @@ int run_small(xdrop_ctx *c, Ticket *tk, const Job &job)
     cudaStream_t s = c->stream;
     c->tile0 = Tile{32, 4, warp_packed(effective(job.sc))};
     CK(cudaMemsetAsync(c->d_ctrs, 0, C_MAXLEN * 4, s));
-    CK(launch_warp(2 * job.n_pairs, c->sm_count, c->d_job, nullptr, nullptr, c->d_ctrs + C_WARP, 0,
+    CK(launch_warp(2 * job.n_pairs, c->sm_count, c->d_job, &job, nullptr, nullptr, c->d_ctrs + C_WARP, 0,
                    tk->device_submit ? c->d_ctrs + C_NBAD : nullptr, spill_of(c, 0),
                    spill_of(c, 1), s));
     CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
@@ -547,7 +551,28 @@ int run_small(xdrop_ctx *c, Ticket *tk, const Job &job)
     return XDROP_OK;
 }
 
-void free_ticket(xdrop_ctx *c, Ticket *tk)
+// The pool seed discovery allocates from: it keeps up to kPoolKeep bytes of
+// its pages between calls (the device's default pool gives them back at
+// every synchronisation; a 1 Mb genome at 29x, waited for, 7.2 ms a call so
+// and 4.8 with kept pages), none with a memory budget.  Made at the first
+// call, destroyed with the context.
+constexpr uint64_t kPoolKeep = (uint64_t)4 << 30;
+
+int seed_pool(xdrop_ctx *c)
+{
+    if (c->pool) return XDROP_OK;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = c->device;
+    CK(cudaMemPoolCreate(&c->pool, &props));
+    uint64_t keep = c->budget ? 0 : kPoolKeep;
+    CK(cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    return XDROP_OK;
+}
+
+void destroy_ticket(xdrop_ctx *c, Ticket *tk)
 {
     if (tk->ev_begin) cudaEventDestroy(tk->ev_begin);
     if (tk->ev_end) cudaEventDestroy(tk->ev_end);
@@ -560,16 +585,59 @@ void free_ticket(xdrop_ctx *c, Ticket *tk)
     delete tk;
 }
 
+// A ticket's events and buffers outlive it: allocating them is a good part of
+// a small call (64 short pairs: 100 us a call with new ones, 90 with kept
+// ones, 55 with the polling wait of xdrop_sync and the job as an argument).
+// At most kIdleTickets are kept, none larger than the limits, and no device
+// memory by a context with a memory budget; xdrop_free gives them back.
+// All of it happens under the context's mutex, on tickets whose work is done.
+constexpr size_t kIdleTickets = 4, kIdlePinned = (size_t)64 << 20, kIdleDevice = (size_t)512 << 20;
+
+void free_ticket(xdrop_ctx *c, Ticket *tk)
+{
+    if (tk->d_mem && (c->budget || tk->d_bytes > kIdleDevice)) {
+        cudaFree(tk->d_mem);
+        c->used -= tk->d_bytes;
+        tk->d_mem = nullptr;
+        tk->d_bytes = 0;
+    }
+    if (!tk->ev_done || tk->pin_bytes > kIdlePinned || c->idle.size() >= kIdleTickets) {
+        destroy_ticket(c, tk);
+        return;
+    }
+    c->idle.push_back(tk);
+}
+
+// Device memory of a ticket (inputs and results): what it has from an
+// earlier one if that is enough.
+cudaError_t ticket_mem(xdrop_ctx *c, Ticket *tk, size_t bytes)
+{
+    if (tk->d_mem && tk->d_bytes >= bytes) return cudaSuccess;
+    if (tk->d_mem) {
+        cudaFree(tk->d_mem);
+        c->used -= tk->d_bytes;
+        tk->d_mem = nullptr;
+        tk->d_bytes = 0;
+    }
+    const cudaError_t e = cudaMalloc(&tk->d_mem, bytes);
+    if (e != cudaSuccess) return e;
+    tk->d_bytes = bytes;
+    c->used += bytes;
+    return cudaSuccess;
+}
+
 // Common tail of both submit flavours: descriptor, launches, copies back.
 int launch_ticket(xdrop_ctx *c, Ticket *tk, const Job &job, uint32_t maxlen)
 {
     cudaStream_t s = c->stream;
     int rc;
     if ((rc = ensure_scratch(c, 2 * job.n_pairs, maxlen))) return rc;
-    *tk->h_job = job;
-    CK(cudaMemcpyAsync(c->d_job, tk->h_job, sizeof(Job), cudaMemcpyHostToDevice, s));
-    CK(cudaEventRecord(tk->ev_begin, s));
     const bool small = job.n_pairs && is_small(c, job.n_pairs);
+    if (!small) {  // the small batch's kernel takes the descriptor as an argument
+        *tk->h_job = job;
+        CK(cudaMemcpyAsync(c->d_job, tk->h_job, sizeof(Job), cudaMemcpyHostToDevice, s));
+    }
+    CK(cudaEventRecord(tk->ev_begin, s));
     // the tile first: autotuning uses the result buffer as scratch, and
     // validation then writes every status word
     if (job.n_pairs && c->mode != XDROP_MODE_PLAIN && !small) {
@@ -633,17 +701,44 @@ int launch_ticket_chunked(xdrop_ctx *c, Ticket *tk, const xdrop_pair *h_pairs, s
 
 int new_ticket(xdrop_ctx *c, size_t n_pairs, bool device_submit, Ticket **out, size_t n_jobs = 1)
 {
-    Ticket *tk = new Ticket();
+    const size_t pin = align_up(sizeof(Job) * std::max<size_t>(n_jobs, 1)) + align_up(C_WORDS * 4) +
+                       (device_submit ? 0 : align_up(n_pairs * sizeof(xdrop_result)));
+    // the idle ticket with the largest buffers, or a new one
+    Ticket *tk = nullptr;
+    if (!c->idle.empty()) {
+        auto it = std::max_element(c->idle.begin(), c->idle.end(), [](Ticket *x, Ticket *y) {
+            return x->pin_bytes + x->d_bytes < y->pin_bytes + y->d_bytes;
+        });
+        Ticket kept;
+        std::swap(kept, **it);
+        tk = *it;
+        c->idle.erase(it);
+        tk->h_pinned = kept.h_pinned;
+        tk->pin_bytes = kept.pin_bytes;
+        tk->d_mem = kept.d_mem;
+        tk->d_bytes = kept.d_bytes;
+        tk->ev_begin = kept.ev_begin;
+        tk->ev_end = kept.ev_end;
+        tk->ev_done = kept.ev_done;
+    } else {
+        tk = new Ticket();
+    }
     tk->device_submit = device_submit;
     tk->n_pairs = n_pairs;
-    size_t pin = align_up(sizeof(Job) * std::max<size_t>(n_jobs, 1)) + align_up(C_WORDS * 4) +
-                 (device_submit ? 0 : align_up(n_pairs * sizeof(xdrop_result)));
-    cudaError_t e = cudaHostAlloc(&tk->h_pinned, pin, cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaEventCreate(&tk->ev_begin);
-    if (e == cudaSuccess) e = cudaEventCreate(&tk->ev_end);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&tk->ev_done, cudaEventBlockingSync);
+    cudaError_t e = cudaSuccess;
+    if (tk->pin_bytes < pin) {
+        if (tk->h_pinned) cudaFreeHost(tk->h_pinned);
+        tk->h_pinned = nullptr;
+        tk->pin_bytes = 0;
+        e = cudaHostAlloc(&tk->h_pinned, pin, cudaHostAllocDefault);
+        if (e == cudaSuccess) tk->pin_bytes = pin;
+    }
+    if (e == cudaSuccess && !tk->ev_begin) e = cudaEventCreate(&tk->ev_begin);
+    if (e == cudaSuccess && !tk->ev_end) e = cudaEventCreate(&tk->ev_end);
+    if (e == cudaSuccess && !tk->ev_done)
+        e = cudaEventCreateWithFlags(&tk->ev_done, cudaEventBlockingSync);
     if (e != cudaSuccess) {
-        free_ticket(c, tk);
+        destroy_ticket(c, tk);
         return fail(XDROP_ECUDA, "ticket setup: %s", cudaGetErrorString(e));
     }
     char *p = (char *)tk->h_pinned;
@@ -736,13 +831,11 @@ int xdrop_submit(xdrop_ctx *c, const uint32_t *packed, const uint64_t *read_off,
         return fail(c->tickets.empty() ? XDROP_ENOMEM : XDROP_EBUSY,
                     "device memory budget exceeded (%zu bytes needed)", bytes);
     }
-    cudaError_t e = cudaMalloc(&tk->d_mem, bytes);
+    cudaError_t e = ticket_mem(c, tk, bytes);
     if (e != cudaSuccess) {
-        free_ticket(c, tk);
+        destroy_ticket(c, tk);
         return fail(XDROP_ECUDA, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
     }
-    tk->d_bytes = bytes;
-    c->used += bytes;
     char *d = (char *)tk->d_mem;
     cudaStream_t st = c->stream;
     e = cudaSuccess;
@@ -858,7 +951,14 @@ int xdrop_sync(xdrop_ctx *c, xdrop_ticket t, int64_t timeout_ns)
     }
     CK(cudaSetDevice(c->device));
     if (timeout_ns < 0) {
-        CK(cudaEventSynchronize(tk->ev_done));
+        // A blocking wait wakes 30 to 40 us late: poll first, for
+        // about as long as a small batch takes.
+        const auto until = std::chrono::steady_clock::now() + std::chrono::milliseconds(2);
+        cudaError_t q = cudaErrorNotReady;
+        while (q == cudaErrorNotReady && std::chrono::steady_clock::now() < until)
+            q = cudaEventQuery(tk->ev_done);
+        if (q == cudaErrorNotReady) q = cudaEventSynchronize(tk->ev_done);
+        if (q != cudaSuccess) return fail(XDROP_ECUDA, "sync: %s", cudaGetErrorString(q));
     } else {
         auto t0 = std::chrono::steady_clock::now();
         for (;;) {
@@ -910,8 +1010,10 @@ void xdrop_free(xdrop_ctx *c)
     cudaFree(c->r_off.p);
     cudaFree(c->r_len.p);
     if (c->stream) cudaStreamSynchronize(c->stream);
-    for (auto &kv : c->tickets) free_ticket(c, kv.second);
+    for (auto &kv : c->tickets) destroy_ticket(c, kv.second);
     c->tickets.clear();
+    for (Ticket *tk : c->idle) destroy_ticket(c, tk);
+    c->idle.clear();
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     if (c->ev_main0) cudaEventDestroy(c->ev_main0);
     if (c->ev_main1) cudaEventDestroy(c->ev_main1);
@@ -922,6 +1024,7 @@ void xdrop_free(xdrop_ctx *c)
     cudaFree(c->d_job);
     cudaFree(c->d_ctrs);
     if (c->stream) cudaStreamDestroy(c->stream);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     delete c;
 }
 
@@ -1076,13 +1179,11 @@ int xdrop_submit_pairs(xdrop_ctx *c, const xdrop_pair *pairs, size_t n_pairs,
         return fail(c->tickets.empty() ? XDROP_ENOMEM : XDROP_EBUSY,
                     "device memory budget exceeded (%zu bytes needed)", bytes);
     }
-    cudaError_t e = cudaMalloc(&tk->d_mem, bytes);
+    cudaError_t e = ticket_mem(c, tk, bytes);
     if (e != cudaSuccess) {
-        free_ticket(c, tk);
+        destroy_ticket(c, tk);
         return fail(XDROP_ECUDA, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
     }
-    tk->d_bytes = bytes;
-    c->used += bytes;
     char *d = (char *)tk->d_mem;
     if (n_chunks > 1) {
         Job base{};
@@ -1186,7 +1287,8 @@ int xdrop_find_candidates(xdrop_ctx *c, const xdrop_kmer_params *p, xdrop_pair *
         c->cand_gen = 0;
         const size_t left = c->budget ? (c->budget > c->used ? c->budget - c->used : 1) : 0;
         std::string err;
-        const int rc = find_candidates(c->stream, c->sm_count, left, (const uint32_t *)c->r_packed.p,
+        if (int rc = seed_pool(c)) return rc;
+        const int rc = find_candidates(c->stream, c->pool, c->sm_count, left, (const uint32_t *)c->r_packed.p,
                                        (const uint64_t *)c->r_off.p, (const uint32_t *)c->r_len.p,
                                        c->r_n, c->h_len.data(), p->k, p->stride, p->lo, p->hi,
                                        p->flags, c->cand_pairs, c->cand_shared, c->seed_stats,

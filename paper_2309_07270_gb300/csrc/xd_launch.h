@@ -47,8 +47,9 @@ cudaError_t launch_spill_512(int grid, const Job *jp, Spill in, Spill out, cudaS
 // number *n_ptr) or, without one, all tasks of the job; windows of 128, 256 and
 // 512 slots, from the first wider than `from`, overflow to `out`.  Without a list: tasks that
 // outgrew 128 slots are also noted in `over`, and n_bad asks for the pairs'
-// status.
-cudaError_t launch_warp(uint64_t n_tasks, int sm_count, const Job *jp, const uint32_t *list,
+// status.  value (host): the job, which the kernel stores at jp; else it is
+// read there.
+cudaError_t launch_warp(uint64_t n_tasks, int sm_count, Job *jp, const Job *value, const uint32_t *list,
                         const uint32_t *n_ptr, uint32_t *counter, int from, uint32_t *n_bad,
                         Spill over, Spill out, cudaStream_t s);
 // Blocks per SM of a persistent tile at 256 threads per block.
@@ -109,7 +110,7 @@ struct SeedStats {
     uint32_t product = 0;       // XDROP_SEEDS_ROWWISE or XDROP_SEEDS_SORT: the one that ran
     uint64_t nonzeros = 0;      // A's nonzeros, counted by the row-wise product
 };
-int find_candidates(cudaStream_t s, int sm_count, size_t budget, const uint32_t *packed,
+int find_candidates(cudaStream_t s, cudaMemPool_t pool, int sm_count, size_t budget, const uint32_t *packed,
                     const uint64_t *read_off, const uint32_t *read_len, uint32_t n_reads,
                     const uint32_t *h_len, uint32_t k, uint32_t stride, uint32_t lo, uint32_t hi,
                     uint32_t flags, std::vector<Pair> &out_pairs,

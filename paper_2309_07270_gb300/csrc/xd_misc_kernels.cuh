@@ -59,7 +59,7 @@ bin_count_kernel(const Job *jp, uint32_t *hist)
 // to warps) for a few block counts by the longer of the two parts, each the
 // larger of its total work and its longest task; the cheapest wins.  Without
 // `longest` only overflow goes to warps.
-constexpr float kWarpNs = 75.f;  // measured: 57 ns alone on its scheduler
+constexpr float kWarpNs = 90.f;  // 57 ns alone on its scheduler, more beside others
 
 __global__ void __launch_bounds__(NBINS)
 bin_scan_kernel(const uint32_t *hist, uint32_t *offs, uint32_t *n_valid, uint32_t *counter,

@@ -407,11 +407,12 @@ int grid_for(uint64_t n, int sm_count)
 // Stream-ordered device allocations of one call, released together.
 struct Arena {
     cudaStream_t s;
+    cudaMemPool_t pool;
     size_t budget, used = 0;
     std::vector<void *> held;
     int rc = XDROP_OK;
     std::string err;
-    Arena(cudaStream_t st, size_t b) : s(st), budget(b) {}
+    Arena(cudaStream_t st, cudaMemPool_t p, size_t b) : s(st), pool(p), budget(b) {}
     ~Arena()
     {
         for (void *p : held) cudaFreeAsync(p, s);
@@ -426,9 +427,9 @@ struct Arena {
             return false;
         }
         void *q = nullptr;
-        const cudaError_t e = cudaMallocAsync(&q, bytes, s);
+        const cudaError_t e = cudaMallocFromPoolAsync(&q, bytes, pool, s);
         if (e != cudaSuccess) {
-            err = std::string("cudaMallocAsync: ") + cudaGetErrorString(e);
+            err = std::string("cudaMallocFromPoolAsync: ") + cudaGetErrorString(e);
             rc = e == cudaErrorMemoryAllocation ? XDROP_ENOMEM : XDROP_ECUDA;
             return false;
         }
@@ -705,7 +706,7 @@ int row_product(Arena &ar, const Front &f, std::vector<Pair> &out_pairs,
 
 }  // namespace
 
-int find_candidates(cudaStream_t st, int sm_count, size_t budget, const uint32_t *packed,
+int find_candidates(cudaStream_t st, cudaMemPool_t pool, int sm_count, size_t budget, const uint32_t *packed,
                     const uint64_t *read_off, const uint32_t *read_len, uint32_t n_reads,
                     const uint32_t *h_len, uint32_t k, uint32_t stride, uint32_t lo, uint32_t hi,
                     uint32_t flags, std::vector<Pair> &out_pairs,
@@ -732,7 +733,7 @@ int find_candidates(cudaStream_t st, int sm_count, size_t budget, const uint32_t
     }
     int rc = XDROP_OK;
     {
-        Arena ar(st, budget);
+        Arena ar(st, pool, budget);
         Front f;
         f.packed = packed;
         f.read_len = read_len;

@@ -258,7 +258,7 @@ bool has_warp_role(Tile t) { return t.packed && !t.absolute; }
 // window slots per ns) and the ns per diagonal of one of its extensions.
 void tile_rates(Tile t, float *rate, float *group_ns)
 {
-    *rate = 5000.f / (float)t.width();
+    *rate = 3500.f / (float)t.width();
     *group_ns = 40.f + 9.f * (float)t.c;
 }
 

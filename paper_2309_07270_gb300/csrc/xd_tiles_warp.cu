@@ -12,10 +12,11 @@ namespace xd {
 // list: tasks that outgrew 128 slots are noted in over, and with n_bad the
 // pairs are validated as validate_kernel does.
 __global__ void __launch_bounds__(kWarpThreads)
-warp_kernel(const Job *jp, const uint32_t *list, const uint32_t *n_ptr, uint32_t *counter,
+warp_kernel(Job *jp, const Job value, bool by_value, const uint32_t *list, const uint32_t *n_ptr, uint32_t *counter,
             int from, uint32_t *n_bad, Spill over, Spill out)
 {
-    const Job J = *jp;
+    const Job J = by_value ? value : *jp;
+    if (by_value && blockIdx.x == 0 && threadIdx.x == 0) *jp = value;  // for the next launch
     const int lane = threadIdx.x & 31;
     const uint32_t n = list ? *n_ptr : (uint32_t)(2 * J.n_pairs);
     for (;;) {
@@ -40,7 +41,7 @@ warp_kernel(const Job *jp, const uint32_t *list, const uint32_t *n_ptr, uint32_t
 
 bool warp_packed(const Scoring &sc) { return warp16_ok<2>(sc); }
 
-cudaError_t launch_warp(uint64_t n_tasks, int sm_count, const Job *jp, const uint32_t *list,
+cudaError_t launch_warp(uint64_t n_tasks, int sm_count, Job *jp, const Job *value, const uint32_t *list,
                         const uint32_t *n_ptr, uint32_t *counter, int from, uint32_t *n_bad,
                         Spill over, Spill out, cudaStream_t s)
 {
@@ -51,8 +52,8 @@ cudaError_t launch_warp(uint64_t n_tasks, int sm_count, const Job *jp, const uin
     const uint64_t blocks = std::min<uint64_t>((n_tasks + warps - 1) / warps, cap);
     if (!blocks) return cudaSuccess;
     (void)cudaGetLastError();
-    warp_kernel<<<(unsigned)blocks, threads, 0, s>>>(jp, list, n_ptr, counter, from, n_bad, over,
-                                                     out);
+    warp_kernel<<<(unsigned)blocks, threads, 0, s>>>(jp, value ? *value : Job{}, value != nullptr,
+                                                     list, n_ptr, counter, from, n_bad, over, out);
     return cudaGetLastError();
 }
 
