@@ -258,9 +258,9 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st);
  * keys the first tile by the scoring and the job's length bucket (the
  * octave of an extension's min(m, n) that holds the median of the job's work,
  * read from a device histogram at every batched submit).  The first submit with a new key times the first-tier tiles on
- * a stratified random sample of its pairs (one pair of every 3 with the
- * packed tiles when the scoring fits them, else one of every 8 with the
- * 32-bit tiles; widths far from x / |gap| are left out) and keeps the
+ * its pairs, or on a stratified random sample of a large job (one pair of
+ * every 3 above 150,000 with the packed tiles when the scoring fits them,
+ * else one of every 8 above 12,288 with the 32-bit tiles; widths far from x / |gap| are left out) and keeps the
  * fastest for that key.  Tiles: 4x16, 8x8, 16x4,
  * 8x16, 16x8, 32x4, and packed (cells | XDROP_TILE_PACKED16) 4x8, 2x16,
  * 4x16, 8x8, 2x32, 8x16, 16x8, 4x32, 1x32, 2x64.  Returns XDROP_EINVAL for

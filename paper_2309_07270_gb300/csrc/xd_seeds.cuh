@@ -182,7 +182,8 @@ struct CandMerge {
 };
 
 // Distinct reads of a run (the nonzeros of its column of A), 0 for a run
-// outside [lo, hi].
+// outside [lo, hi].  (This and run_members state a column in plain loops;
+// column_kernel writes the same with a warp.)
 XS_HD uint32_t run_reads(const uint32_t *occ, const uint32_t *occ_rd, uint64_t s, uint32_t cnt,
                          uint32_t lo, uint32_t hi)
 {

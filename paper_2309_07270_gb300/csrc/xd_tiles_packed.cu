@@ -254,8 +254,8 @@ Tile usable_tile(Tile t, const Scoring &sc)
 bool has_warp_role(Tile t) { return t.packed && !t.absolute; }
 
 // What the price of a cut between single warps and groups (bin_scan_kernel)
-// takes from the tile: diagonals per ns of a full first tier (about 5,000
-// window slots per ns) and the ns per diagonal of one of its extensions.
+// takes from the tile: diagonals per ns of a full first tier (3,500 window
+// slots per ns; 5,000 at its best) and the ns per diagonal of one of its extensions.
 void tile_rates(Tile t, float *rate, float *group_ns)
 {
     *rate = 3500.f / (float)t.width();
