@@ -137,7 +137,7 @@ struct xdrop_ctx {
     Tile forced = {0, 0};         // xdrop_set_tile
     // tuned first tile per (scoring, length bucket of the job)
     std::map<std::tuple<int, int, int, int, int>, Tile> tuned;
-    uint64_t scratch_version = 0; // bumped whenever a scratch buffer moves
+    uint64_t scratch_version = 0; // bumped whenever a scratch buffer moves or its slices change
     cudaGraphExec_t gexec = nullptr;
     cudaEvent_t ev_main0 = nullptr, ev_main1 = nullptr;  // recorded inside the graph
     Tile graph_tile = {0, 0};
@@ -211,6 +211,7 @@ int ensure_scratch(xdrop_ctx *c, size_t n_tasks, uint32_t maxlen)
     if (per > c->wide_per_cta) {
         if ((rc = dev_alloc(c, c->wide, (size_t)per * 4 * c->wide_grid))) return rc;
         c->wide_per_cta = per;
+        c->scratch_version += 1;  // a captured launch holds the slice too
     }
     return XDROP_OK;
 }
