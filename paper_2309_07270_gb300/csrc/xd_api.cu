@@ -79,7 +79,9 @@ enum : int {
     C_COUNTER2,               // its work counter
     C_SPILL2,                 // its overflow
     C_ROLE2,                  // the words of its WarpRole
-    C_NBAD = C_ROLE2 + 6,    // kept by the launch sequence's memset, as the next two
+    C_WIDE_M = C_ROLE2 + 6,   // largest m of the extensions for the unbounded tier
+    C_NBAD,                   // from here on kept by the launch sequence's memset
+    C_UNFIT,                  // extensions too long for that tier's whole scratch
     C_MAXLEN,
     C_ROLE_ERR,               // sticky: a lost overflow entry
     C_WORDS
@@ -103,6 +105,7 @@ struct Ticket {
     uint32_t launches = 0, graph_replays = 0;
     uint32_t *h_ctrs = nullptr;   // copy of the counter block at the end
     Job *h_job = nullptr;
+    Job job = {};                 // device submit: as submitted
     xdrop_result *h_out = nullptr;
 };
 
@@ -128,7 +131,8 @@ struct xdrop_ctx {
     int64_t wide_per_cta = 0;
     int wide_grid = 0;
 
-    // cached max read length of the last device submit
+    // longest read of the last device submit that measured it, and the array:
+    // a guess at the reads of its next submit
     const uint32_t *maxlen_ptr = nullptr;
     uint32_t maxlen_n = 0, maxlen_val = 0;
 
@@ -231,7 +235,8 @@ int validate_scoring(const xdrop_scoring *s)
 
 Spill spill_of(xdrop_ctx *c, int k)
 {
-    return Spill{(uint32_t *)c->spill[k].p, c->d_ctrs + C_SPILL0 + k};
+    return Spill{(uint32_t *)c->spill[k].p, c->d_ctrs + C_SPILL0 + k,
+                 k == 1 ? c->d_ctrs + C_WIDE_M : nullptr};
 }
 
 // The scoring that decides the tiles of a job: the kernels run every scoring
@@ -249,7 +254,7 @@ int enqueue_wider(xdrop_ctx *c, int w, uint64_t n_tasks)
     CK(launch_warp(n_tasks, c->sm_count, c->d_job, nullptr, spill_of(c, 0).list, spill_of(c, 0).count,
                    c->d_ctrs + C_WARP, w, nullptr, Spill{}, spill_of(c, 1), c->stream));
     CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
-                   c->wide_per_cta, c->stream));
+                   c->wide_per_cta, c->d_ctrs + C_UNFIT, c->stream));
     return XDROP_OK;
 }
 
@@ -314,7 +319,7 @@ int enqueue_batched(xdrop_ctx *c, Tile t0, int bps, const Scoring &sc, bool main
     }
     if (!role.n_long) return enqueue_wider(c, t0.width(), c->cap_tasks);
     CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
-                   c->wide_per_cta, s));
+                   c->wide_per_cta, c->d_ctrs + C_UNFIT, s));
     return XDROP_OK;
 }
 
@@ -547,7 +552,7 @@ int run_small(xdrop_ctx *c, Ticket *tk, const Job &job)
                    tk->device_submit ? c->d_ctrs + C_NBAD : nullptr, spill_of(c, 0),
                    spill_of(c, 1), s));
     CK(launch_wide(false, c->wide_grid, c->d_job, spill_of(c, 1), (int32_t *)c->wide.p,
-                   c->wide_per_cta, s));
+                   c->wide_per_cta, c->d_ctrs + C_UNFIT, s));
     tk->launches += 2;
     return XDROP_OK;
 }
@@ -644,8 +649,8 @@ int launch_ticket(xdrop_ctx *c, Ticket *tk, const Job &job, uint32_t maxlen)
     if (job.n_pairs && c->mode != XDROP_MODE_PLAIN && !small) {
         if ((rc = pick_tile(c, tk, job, &c->tile0))) return rc;
     }
+    if (!small) CK(cudaMemsetAsync(c->d_ctrs + C_NBAD, 0, (C_MAXLEN - C_NBAD) * 4, s));
     if (tk->device_submit && !small) {
-        CK(cudaMemsetAsync(c->d_ctrs + C_NBAD, 0, 4, s));
         CK(launch_validate(c->d_job, job.n_pairs, c->d_ctrs + C_NBAD, s));
         tk->launches += 1;
     }
@@ -661,6 +666,16 @@ int launch_ticket(xdrop_ctx *c, Ticket *tk, const Job &job, uint32_t maxlen)
         CK(cudaMemcpyAsync(tk->h_out, job.out, tk->n_pairs * sizeof(xdrop_result),
                            cudaMemcpyDeviceToHost, s));
     CK(cudaEventRecord(tk->ev_done, s));
+    return XDROP_OK;
+}
+
+// The longest of n_reads device lengths.  Synchronous.
+int longest_read(xdrop_ctx *c, const uint32_t *read_len, uint32_t n_reads, uint32_t *maxlen)
+{
+    CK(cudaMemsetAsync(c->d_ctrs + C_MAXLEN, 0, 4, c->stream));
+    CK(launch_max_len(read_len, n_reads, c->d_ctrs + C_MAXLEN, c->stream));
+    CK(cudaMemcpyAsync(maxlen, c->d_ctrs + C_MAXLEN, 4, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
     return XDROP_OK;
 }
 
@@ -899,13 +914,14 @@ int xdrop_submit_device(xdrop_ctx *c, const uint32_t *packed, uint64_t n_words,
     if (n_words * 16 >= ((uint64_t)1 << 32)) return fail(XDROP_EINVAL, "packed buffer too large");
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
-    // Largest read (sizes the unbounded tier); cached per read_len array.
+    // The longest read sizes the unbounded tier's slices.  It is measured for a
+    // new array; the same one may hold longer reads by now, for which that tier
+    // then takes fewer, larger slices, and if the whole scratch is too small for
+    // one the sync runs the ticket again (measuring every time would cost
+    // every small batch a round trip).
     uint32_t maxlen = c->maxlen_val;
     if (n_pairs && (read_len != c->maxlen_ptr || n_reads != c->maxlen_n)) {
-        CK(cudaMemsetAsync(c->d_ctrs + C_MAXLEN, 0, 4, c->stream));
-        CK(launch_max_len(read_len, n_reads, c->d_ctrs + C_MAXLEN, c->stream));
-        CK(cudaMemcpyAsync(&maxlen, c->d_ctrs + C_MAXLEN, 4, cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
+        if ((rc = longest_read(c, read_len, n_reads, &maxlen))) return rc;
         c->maxlen_ptr = read_len;
         c->maxlen_n = n_reads;
         c->maxlen_val = maxlen;
@@ -923,6 +939,7 @@ int xdrop_submit_device(xdrop_ctx *c, const uint32_t *packed, uint64_t n_words,
     job.sc = Scoring{s->match, s->mismatch, s->gap, s->x};
     job.out = (int32_t *)out;
     job.cells = nullptr;
+    tk->job = job;
     if ((rc = launch_ticket(c, tk, job, maxlen))) {
         cudaStreamSynchronize(c->stream);
         free_ticket(c, tk);
@@ -976,6 +993,18 @@ int xdrop_sync(xdrop_ctx *c, xdrop_ticket t, int64_t timeout_ns)
     auto it = c->tickets.find(t);
     if (it == c->tickets.end()) return fail(XDROP_EINVAL, "ticket %llu already synced", (unsigned long long)t);
     c->tickets.erase(it);
+    if (tk->h_ctrs[C_WIDE_M] > c->maxlen_val) c->maxlen_ptr = nullptr;  // measure again
+    if (tk->device_submit && tk->h_ctrs[C_UNFIT]) {
+        uint32_t maxlen = 0;
+        tk->launches = tk->graph_replays = 0;
+        int rc = longest_read(c, tk->job.read_len, tk->job.n_reads, &maxlen);
+        if (!rc) rc = launch_ticket(c, tk, tk->job, maxlen);
+        const cudaError_t e = cudaStreamSynchronize(c->stream);
+        if (rc || e != cudaSuccess) {
+            free_ticket(c, tk);
+            return rc ? rc : fail(XDROP_ECUDA, "sync: %s", cudaGetErrorString(e));
+        }
+    }
     if (!tk->device_submit && tk->n_pairs)
         memcpy(tk->out, tk->h_out, tk->n_pairs * sizeof(xdrop_result));
     float ms = 0.f, ms_main = 0.f;
@@ -1413,11 +1442,8 @@ int xdrop_count_cells_device(xdrop_ctx *c, const uint32_t *packed, uint64_t n_wo
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
     cudaStream_t st = c->stream;
-    CK(cudaMemsetAsync(c->d_ctrs + C_MAXLEN, 0, 4, st));
-    CK(launch_max_len(read_len, n_reads, c->d_ctrs + C_MAXLEN, st));
     uint32_t maxlen = 0;
-    CK(cudaMemcpyAsync(&maxlen, c->d_ctrs + C_MAXLEN, 4, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    if ((rc = longest_read(c, read_len, n_reads, &maxlen))) return rc;
     if ((rc = ensure_scratch(c, 2 * n_pairs, maxlen))) return rc;
     Job job{};
     job.packed = packed;
@@ -1438,7 +1464,7 @@ int xdrop_count_cells_device(xdrop_ctx *c, const uint32_t *packed, uint64_t n_wo
         CK(launch_window(Tile{32, 16}, true, c->d_job, (uint32_t)t0, nt, spill_of(c, 0), st));
     }
     CK(launch_wide(true, c->wide_grid, c->d_job, spill_of(c, 0), (int32_t *)c->wide.p,
-                   c->wide_per_cta, st));
+                   c->wide_per_cta, c->d_ctrs + C_UNFIT, st));
     CK(cudaStreamSynchronize(st));
     return XDROP_OK;
 }

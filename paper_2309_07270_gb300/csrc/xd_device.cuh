@@ -899,18 +899,35 @@ __device__ void extend_wide(const Ext &e, const Scoring sc, int32_t *diag,
     cells_out = cells;
 }
 
+// Each CTA runs its tasks on a slice of the scratch: scratch_per_cta words,
+// or, where the reads may have grown since the host sized it (in.longest),
+// what the longest extension of the list needs, on as many CTAs as then have
+// room.  One too long for the whole scratch is counted in unfit.
 template <bool COUNT>
 __global__ void __launch_bounds__(WIDE_THREADS)
-wide_kernel(const Job *jp, Spill in, int32_t *scratch, int64_t scratch_per_cta)
+wide_kernel(const Job *jp, Spill in, int32_t *scratch, int64_t scratch_per_cta, uint32_t *unfit)
 {
-    const Job J = *jp;
     const uint32_t n = *in.count;
-    int32_t *diag = scratch + (int64_t)blockIdx.x * scratch_per_cta;
-    for (uint32_t q = blockIdx.x; q < n; q += gridDim.x) {
+    if (n == 0) return;
+    int64_t per = scratch_per_cta;
+    uint32_t ctas = gridDim.x;
+    if (in.longest) {
+        const int64_t need = 3 * ((int64_t)*in.longest + 1), all = per * gridDim.x;
+        if (need > per) {
+            per = need < all ? need : all;
+            ctas = (uint32_t)(all / per);
+        }
+    }
+    const Job J = *jp;
+    int32_t *diag = scratch + (int64_t)blockIdx.x * per;
+    for (uint32_t q = blockIdx.x; q < n && blockIdx.x < ctas; q += ctas) {
         const uint32_t task = in.list[q];
         Ext e = decode(J, task);
         if (!e.ok) continue;
-        if ((int64_t)3 * (e.m + 1) > scratch_per_cta) continue;  // sized by the host
+        if ((int64_t)3 * (e.m + 1) > per) {
+            if (unfit && threadIdx.x == 0) atomicAdd(unfit, 1u);
+            continue;
+        }
         int32_t sc, bi, bj;
         int64_t cells;
         extend_wide<COUNT>(e, J.sc, diag, sc, bi, bj, cells);

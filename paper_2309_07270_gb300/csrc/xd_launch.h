@@ -70,7 +70,7 @@ bool warp_packed(const Scoring &sc);
 Tile in_frame(Tile t, const Scoring &sc);
 
 cudaError_t launch_wide(bool count, int grid, const Job *jp, Spill in, int32_t *scratch,
-                        int64_t scratch_per_cta, cudaStream_t s);
+                        int64_t scratch_per_cta, uint32_t *unfit, cudaStream_t s);
 cudaError_t launch_validate(const Job *jp, uint64_t n_pairs, uint32_t *n_bad, cudaStream_t s);
 // The longest-first order of a job's tasks (hist zeroed before), their number
 // and, with a role, the first tasks (none unless `longest`) and blocks that go

@@ -380,7 +380,8 @@ void Server::handle_spills(std::vector<Req *> &sp)
         if (e == cudaSuccess)
             e = launch_spill_512(2 * sm_count, d_jobs + r->slot, in, out, s_side);
         if (e == cudaSuccess)
-            e = launch_wide(false, wide_grid, d_jobs + r->slot, out, wide_scratch, wide_per_cta, s_side);
+            e = launch_wide(false, wide_grid, d_jobs + r->slot, out, wide_scratch, wide_per_cta, nullptr,
+                            s_side);
         if (e == cudaSuccess) {
             char *h = h_pool + r->host_off;
             e = cudaMemcpyAsync(h + r->h_out, d + r->d_out, r->n * sizeof(xdrop_result),

@@ -97,7 +97,7 @@ static __device__ __noinline__ void run_warp_role(const Job *jp, const uint32_t 
         const int st = extend_warp(e, J.sc, whole ? 0 : width, lane, sc, bi, bj);
         if (lane == 0) {
             if (whole && st) atomicAdd(role.grown, 1u);
-            if (st < 0) role.wide.list[atomicAdd(role.wide.count, 1u)] = task;
+            if (st < 0) hand_on_wide(role.wide, task, e.m);
             else write_result(J, e, sc, bi, bj);
         }
         __syncwarp();

@@ -32,7 +32,7 @@ warp_kernel(Job *jp, const Job value, bool by_value, const uint32_t *list, const
         const int st = extend_warp(e, J.sc, from, lane, sc, bi, bj);
         if (lane == 0) {
             if (!list && st) over.list[atomicAdd(over.count, 1u)] = task;
-            if (st < 0) out.list[atomicAdd(out.count, 1u)] = task;
+            if (st < 0) hand_on_wide(out, task, e.m);
             else write_result(J, e, sc, bi, bj);
         }
         __syncwarp();

@@ -25,11 +25,13 @@ cudaError_t launch_window_count(const Job *jp, uint32_t task_base, uint32_t n_ta
 }
 
 cudaError_t launch_wide(bool count, int grid, const Job *jp, Spill in, int32_t *scratch,
-                        int64_t scratch_per_cta, cudaStream_t s)
+                        int64_t scratch_per_cta, uint32_t *unfit, cudaStream_t s)
 {
     (void)cudaGetLastError();
-    if (count) wide_kernel<true><<<grid, WIDE_THREADS, 0, s>>>(jp, in, scratch, scratch_per_cta);
-    else wide_kernel<false><<<grid, WIDE_THREADS, 0, s>>>(jp, in, scratch, scratch_per_cta);
+    if (count)
+        wide_kernel<true><<<grid, WIDE_THREADS, 0, s>>>(jp, in, scratch, scratch_per_cta, unfit);
+    else
+        wide_kernel<false><<<grid, WIDE_THREADS, 0, s>>>(jp, in, scratch, scratch_per_cta, unfit);
     return cudaGetLastError();
 }
 

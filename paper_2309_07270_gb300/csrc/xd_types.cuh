@@ -69,6 +69,7 @@ __host__ __device__ inline double bin_diagonals(int b)
 struct Spill {
     uint32_t *list;   // task ids
     uint32_t *count;  // number of ids in list
+    uint32_t *longest = nullptr;  // unbounded tier: the largest m of them
 };
 
 // Device words of a batched launch whose first blocks give a warp to single
@@ -212,6 +213,13 @@ __device__ __forceinline__ void write_result(const Job &J, const Ext &e,
         o[1] = (int32_t)e.sa - bi;
         o[2] = (int32_t)e.sb - bj;
     }
+}
+
+// Hands a task on to the unbounded tier (one thread).
+__device__ __forceinline__ void hand_on_wide(const Spill &wide, uint32_t task, int32_t m)
+{
+    if (wide.longest) atomicMax(wide.longest, (uint32_t)m);
+    wide.list[atomicAdd(wide.count, 1u)] = task;
 }
 
 // Status of a pair of a device submit: zero scores for a pair that fails

@@ -39,3 +39,26 @@ def test_growing_reads(X, orc, n):
             got = al.align(w.packed, w.read_off, w.read_len, w.pairs, sc).view(np.int32)
             assert al.stats()["wide_tasks"] > 0
             assert np.array_equal(got, _want(orc, w)), length
+
+
+@pytest.mark.parametrize("n,short,long", [(3, 600, 1500), (700, 600, 1500), (3, 40, 15000)],
+                         ids=["small", "graph", "longer_than_the_scratch"])
+@pytest.mark.parametrize("tile", [None, (2, 32 | 0x100)], ids=["tuned", "forced"])
+def test_read_lengths_rewritten_in_place(X, orc, n, short, long, tile):
+    """The arrays of a device submit may hold longer reads once its ticket is
+    synced: first the reads' heads, then the whole reads, at the same addresses."""
+    w = _reads(n, long, long)
+    sc = X.scoring(1, -1, -1, X_DROP)
+    dev = X.DeviceInputs.from_workload(w)
+    whole = dev.read_len.clone()
+    with X.Aligner() as al:
+        if tile:
+            al.set_tile(*tile)
+        dev.read_len.fill_(short)
+        al.align_device(dev, sc)
+        dev.read_len.copy_(whole)
+        dev.out.fill_(-1)
+        for _ in range(2):  # the first finds the slices too short
+            al.align_device(dev, sc)
+            assert al.stats()["wide_tasks"] > 0
+            assert np.array_equal(dev.results().view(np.int32), _want(orc, w))
