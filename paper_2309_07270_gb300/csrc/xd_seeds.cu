@@ -269,7 +269,9 @@ row_kernel(const uint64_t *__restrict__ occ_off, const uint32_t *__restrict__ ro
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const uint32_t half = lane >> 4, hl = lane & 15;
     for (uint64_t b0 = q0 + 32 * warp; b0 < q1; b0 += 32 * n_warps) {
-        if (*(volatile uint32_t *)&ovf) break;
+        // a vote: other warps set the flag at any time, and the collectives
+        // below need all lanes of this one
+        if (__any_sync(0xFFFFFFFFu, *(volatile uint32_t *)&ovf)) break;
         const uint64_t q = b0 + lane;
         uint32_t own = q < q1 ? row_of[q] : kNone;
         uint64_t word = 0;
