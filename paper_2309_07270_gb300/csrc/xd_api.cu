@@ -74,12 +74,12 @@ enum : int {
     C_SPILL1,                 // extensions for the unbounded tier
     C_WARP,                   // work counter of the warp kernel
     C_ROLE,                   // the words of a WarpRole, but for err
-    C_GROWN = C_ROLE + 5,     // longest tasks that outgrew a warp's first window
+    C_GROWN = C_ROLE + 6,     // longest tasks that outgrew a warp's first window
     C_BRIEF,                  // short overflow, the second group tier's tasks
     C_COUNTER2,               // its work counter
     C_SPILL2,                 // its overflow
     C_ROLE2,                  // the words of its WarpRole
-    C_WIDE_M = C_ROLE2 + 6,   // largest m of the extensions for the unbounded tier
+    C_WIDE_M = C_ROLE2 + 7,   // largest m of the extensions for the unbounded tier
     C_NBAD,                   // from here on kept by the launch sequence's memset
     C_UNFIT,                  // extensions too long for that tier's whole scratch
     C_MAXLEN,
@@ -263,7 +263,7 @@ WarpRole role_of(xdrop_ctx *c, Tile t)
 {
     if (!has_warp_role(t)) return WarpRole{};
     uint32_t *w = c->d_ctrs + C_ROLE;
-    return WarpRole{w, w + 1, w + 2, w + 3, w + 4, c->d_ctrs + C_GROWN, c->d_ctrs + C_ROLE_ERR,
+    return WarpRole{w, w + 1, w + 2, w + 3, w + 4, w + 5, c->d_ctrs + C_GROWN, c->d_ctrs + C_ROLE_ERR,
                     spill_of(c, 1), 0};
 }
 
@@ -285,7 +285,7 @@ int enqueue_brief(xdrop_ctx *c)
     uint32_t *ctr = c->d_ctrs, *w = ctr + C_ROLE2, *list = (uint32_t *)c->order.p;
     const int grid = c->sm_count * bps;
     const uint32_t few = (uint32_t)(grid * persistent_block_threads(t) / 32);
-    const WarpRole role{w, w + 1, w + 2, w + 3, w + 4, w + 5, ctr + C_ROLE_ERR, spill_of(c, 1), few};
+    const WarpRole role{w, w + 1, w + 2, w + 3, w + 4, w + 5, w + 6, ctr + C_ROLE_ERR, spill_of(c, 1), few};
     CK(cudaMemsetAsync(list, 0xFF, c->cap_tasks * 4, c->stream));
     CK(launch_persistent(t, grid, c->d_job, (uint32_t *)c->spill[2].p, ctr + C_BRIEF,
                          ctr + C_COUNTER2, Spill{list, ctr + C_SPILL2}, Spill{}, role, c->stream));

@@ -37,6 +37,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "xd_claim.cuh"
 #include "xd_types.cuh"
 
 namespace xd {
@@ -526,6 +527,12 @@ __device__ __forceinline__ void store_result_cg(const Job &J, uint32_t task, int
     }
 }
 
+struct DeviceMem {  // for xd_claim.cuh
+    __device__ __forceinline__ uint32_t load(const uint32_t *p) { return *(const volatile uint32_t *)p; }
+    __device__ __forceinline__ uint32_t add(uint32_t *p, uint32_t v) { return atomicAdd(p, v); }
+    __device__ __forceinline__ void fence() { __threadfence(); }
+};
+
 // Task source of the batched form: positions of a longest-first order
 // array pulled from a global counter; overflowing tasks go to a spill list.
 struct BatchSrc {
@@ -536,6 +543,7 @@ struct BatchSrc {
     uint32_t *counter;
     Spill spill;
     Spill brief = {};  // with a list: overflow of short extensions goes there
+    uint32_t *ready = nullptr;  // with a WarpRole: the written entries of spill
 
     // Warp-level fetch, executed by every lane: the leaders of the groups
     // that need a task are the set bits of needm.  Returns, for this lane's
@@ -572,6 +580,10 @@ struct BatchSrc {
             }
             const uint32_t q = atomicAdd(to.count, 1u);
             *(volatile uint32_t *)&to.list[q] = task;
+            if (ready && to.list == spill.list) {
+                DeviceMem mem;
+                entry_written(mem, ClaimWords{to.count, ready, nullptr});
+            }
         } else {
             store_result(*gj, task, T, bi, bj);
         }

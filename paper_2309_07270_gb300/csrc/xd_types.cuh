@@ -79,6 +79,7 @@ struct WarpRole {
     uint32_t *n_long;    // tasks at the head of the order for single warps
     uint32_t *n_blocks;  // blocks that start with them
     uint32_t *long_ctr;  // next of those tasks
+    uint32_t *ready;     // overflow entries written and not claimed (xd_claim.cuh)
     uint32_t *taken;     // overflow entries taken
     uint32_t *done;      // first-tier warps that found no more tasks
     uint32_t *grown;     // longest tasks that outgrew a warp's first window
