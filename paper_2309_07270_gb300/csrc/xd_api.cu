@@ -82,8 +82,8 @@ enum : int {
     C_WIDE_M = C_ROLE2 + 7,   // largest m of the extensions for the unbounded tier
     C_NBAD,                   // from here on kept by the launch sequence's memset
     C_UNFIT,                  // extensions too long for that tier's whole scratch
-    C_MAXLEN,
-    C_ROLE_ERR,               // sticky: a lost overflow entry
+    C_ROLE_ERR,               // a lost overflow entry
+    C_MAXLEN,                 // kept by every ticket, which clears the words before it
     C_WORDS
 };
 
@@ -705,6 +705,7 @@ int launch_ticket_chunked(xdrop_ctx *c, Ticket *tk, const xdrop_pair *h_pairs, s
         CK(cudaMemcpyAsync(c->d_job, &tk->h_job[k], sizeof(Job), cudaMemcpyHostToDevice, s));
         if (k == 0) {  // first tile: as for an unchunked submit
             if ((rc = pick_tile(c, tk, job, &c->tile0))) return rc;
+            CK(cudaMemsetAsync(c->d_ctrs + C_NBAD, 0, (C_MAXLEN - C_NBAD) * 4, s));
         }
         if ((rc = run_batched(c, tk, tile_scoring(c, job.sc)))) return rc;
         CK(cudaMemcpyAsync(tk->h_out + p0, d_out, np * sizeof(xdrop_result), cudaMemcpyDeviceToHost, s));

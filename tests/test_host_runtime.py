@@ -1,0 +1,67 @@
+"""The library's host code over a CUDA runtime of host memory
+(tests/fake_cuda.cpp): what a context does when a kernel reports an error, an
+allocation fails or a result is late.  No kernel runs, so results are zeros."""
+import ctypes
+import importlib.util
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+PKG = os.path.join(os.path.dirname(HERE), "paper_2309_07270_gb300")
+
+
+@pytest.fixture(scope="module")
+def built(tmp_path_factory):
+    gxx = shutil.which("g++")
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    if gxx is None or not os.path.exists(os.path.join(include, "cuda_runtime.h")):
+        pytest.skip("no g++ or no CUDA headers")
+    so = tmp_path_factory.mktemp("fake") / "libfake.so"
+    subprocess.run([gxx, "-x", "c++", "-std=c++17", "-O1", "-w", "-shared", "-fPIC", "-pthread",
+                    "-I", os.path.join(os.path.dirname(HERE), "include"), "-I", include, "-o",
+                    str(so), os.path.join(HERE, "fake_cuda.cpp")], check=True)
+    return str(so)
+
+
+@pytest.fixture
+def X(built, tmp_path):
+    """The binding over a fresh copy of the fake library (4 SMs: 16 pairs and
+    fewer are a small batch)."""
+    so = shutil.copy(built, tmp_path / "libfake.so")
+    spec = importlib.util.spec_from_file_location("xdrop_fake", os.path.join(PKG, "xdrop.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.LIB_PATH = str(so)
+    lib = mod.load()
+    for name in ("fake_device_size", "fake_pool_reserved"):
+        getattr(lib, name).argtypes = [ctypes.c_size_t]
+        getattr(lib, name).restype = None
+    lib.fake_device_used.restype = ctypes.c_size_t
+    mod.fake = lib
+    return mod
+
+
+def _job(X, n, words=64):
+    """n pairs of two 64-base reads in a buffer of `words` words."""
+    pairs = np.zeros(n, X.PAIR_DTYPE)
+    pairs["b"] = 1
+    pairs["seed_len"] = 8
+    off = np.array([0, 16 * words - 64], np.uint64)
+    return np.zeros(words, np.uint32), off, np.array([64, 64], np.uint32), pairs
+
+
+def test_a_lost_entry_is_reported_to_its_own_call(X):
+    sc = X.scoring()
+    with X.Aligner() as al:
+        al.align(*_job(X, 40), sc)  # tuned
+        X.fake.fake_lose_entries(1)
+        with pytest.raises(X.XdropError) as ei:
+            al.align(*_job(X, 40), sc)
+        assert ei.value.code == X.XDROP_ECUDA and "never appeared" in str(ei.value)
+        al.align(*_job(X, 40), sc)
+        al.align(*_job(X, 4), sc)
