@@ -213,6 +213,7 @@ int ensure_scratch(xdrop_ctx *c, size_t n_tasks, uint32_t maxlen)
     int64_t per = (int64_t)3 * ((int64_t)maxlen + 1);
     per = (per + 63) / 64 * 64;
     if (per > c->wide_per_cta) {
+        c->wide_per_cta = 0;  // a failed growth leaves no buffer
         if ((rc = dev_alloc(c, c->wide, (size_t)per * 4 * c->wide_grid))) return rc;
         c->wide_per_cta = per;
         c->scratch_version += 1;  // a captured launch holds the slice too
@@ -1100,9 +1101,16 @@ int xdrop_load_reads(xdrop_ctx *c, const uint32_t *packed, const uint64_t *read_
     int rc;
     const uint64_t nw = std::max<uint64_t>(n_words, 1);
     // the reads, then their reverse complements (reverse-strand pairs)
-    if ((rc = dev_alloc(c, c->r_packed, 2 * nw * 4))) return rc;
-    if ((rc = dev_alloc(c, c->r_off, std::max<size_t>(n_reads, 1) * 8))) return rc;
-    if ((rc = dev_alloc(c, c->r_len, std::max<size_t>(n_reads, 1) * 4))) return rc;
+    auto room = [c](DevBuf &b, size_t bytes) {
+        const bool moves = b.cap < bytes;
+        const int e = dev_alloc(c, b, bytes);
+        if (moves && !(e && b.p)) c->have_reads = false;  // the old set went with its buffer
+        return e;
+    };
+    if ((rc = room(c->r_packed, 2 * nw * 4))) return rc;
+    if ((rc = room(c->r_off, std::max<size_t>(n_reads, 1) * 8))) return rc;
+    if ((rc = room(c->r_len, std::max<size_t>(n_reads, 1) * 4))) return rc;
+    c->have_reads = false;
     if (n_words) CK(cudaMemcpy(c->r_packed.p, packed, n_words * 4, cudaMemcpyHostToDevice));
     if (n_reads) {
         CK(cudaMemcpy(c->r_off.p, read_off, (size_t)n_reads * 8, cudaMemcpyHostToDevice));

@@ -20,7 +20,7 @@ struct Event { std::chrono::steady_clock::time_point at; };
 struct Graph { std::vector<std::function<void()>> run; };
 std::map<void *, size_t> device_mem;
 size_t device_used = 0, device_size = (size_t)-1, pool_reserved = 0;
-int graphs = 0, longest_cuts = 0, last_longest = -1;
+int graphs = 0, last_longest = -1, bad_scratch = 0;
 int lose_entries = 0;                        // the next first tiers lose an entry
 std::atomic<int> late_us{0}, polling{0}, polling_max{0};
 Graph *capture = nullptr;
@@ -44,6 +44,7 @@ void fake_pool_reserved(size_t bytes) { fake::pool_reserved = bytes; }
 void fake_lose_entries(int n) { fake::lose_entries = n; }
 void fake_late_us(int us) { fake::late_us = us; }
 int fake_polling_max(void) { return fake::polling_max.exchange(0); }
+int fake_bad_scratch(void) { return fake::bad_scratch; }
 int fake_graphs(void) { return fake::graphs; }
 int fake_last_longest(void) { return fake::last_longest; }
 
@@ -170,7 +171,13 @@ cudaError_t launch_warp(uint64_t, int, Job *jp, const Job *value, const uint32_t
     if (value) *jp = *value;
     return cudaSuccess;
 }
-cudaError_t launch_wide(bool, int, const Job *, Spill, int32_t *, int64_t, uint32_t *, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_wide(bool, int grid, const Job *, Spill, int32_t *scratch, int64_t per, uint32_t *, cudaStream_t)
+{
+    return fake::launched([=] {  // a scratch that is not there, or too small for the slices
+        auto it = fake::device_mem.find(scratch);
+        fake::bad_scratch += it == fake::device_mem.end() || it->second < (size_t)per * 4 * grid;
+    });
+}
 cudaError_t launch_window(Tile, bool, const Job *, uint32_t, uint32_t, Spill, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_validate(const Job *, uint64_t, uint32_t *, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_binning(const Job *, int, uint32_t *, uint32_t *, uint32_t *, uint32_t *, uint32_t *,

@@ -65,3 +65,44 @@ def test_a_lost_entry_is_reported_to_its_own_call(X):
         assert ei.value.code == X.XDROP_ECUDA and "never appeared" in str(ei.value)
         al.align(*_job(X, 40), sc)
         al.align(*_job(X, 4), sc)
+
+
+def _long(X, length):
+    """One pair of reads of `length` bases."""
+    packed, off, lens, pairs = _job(X, 1, words=2 * (length // 16 + 1))
+    off[1] = 16 * (length // 16 + 1)
+    lens[:] = length
+    return packed, off, lens, pairs
+
+
+def test_a_failed_growth_leaves_no_stale_scratch(X):
+    """The unbounded tier's buffer is freed before the larger one is asked for:
+    when that fails, a later call must not run on the freed one."""
+    sc = X.scoring()
+    with X.Aligner() as al:
+        al.align(*_long(X, 1000), sc)
+        X.fake.fake_device_size(X.fake.fake_device_used() + 100_000)
+        with pytest.raises(X.XdropError):
+            al.align(*_long(X, 100_000), sc)
+        al.align(*_long(X, 900), sc)
+        assert X.fake.fake_bad_scratch() == 0
+
+
+@pytest.mark.parametrize("budget", [0, 1 << 20], ids=["out_of_memory", "over_budget"])
+def test_a_failed_load_leaves_no_half_read_set(X, budget):
+    """Out of memory the old reads have gone with their buffer; a budget refuses
+    before anything is freed, and they stay."""
+    sc = X.scoring()
+    packed, off, lens, pairs = _job(X, 3)
+    out = np.zeros(3, X.RESULT_DTYPE)
+    with X.Aligner(budget=budget) as al:
+        X.xdrop_load_reads(al.ctx, packed, off, lens)
+        X.fake.fake_device_size(X.fake.fake_device_used() + 100_000)
+        with pytest.raises(X.XdropError):
+            X.xdrop_load_reads(al.ctx, *_job(X, 3, words=1 << 20)[:3])
+        if budget:
+            X.xdrop_sync(al.ctx, X.xdrop_submit_pairs(al.ctx, pairs, sc, out))
+        else:
+            with pytest.raises(X.XdropError) as ei:
+                X.xdrop_submit_pairs(al.ctx, pairs, sc, out)
+            assert ei.value.code == X.XDROP_EINVAL
