@@ -175,6 +175,42 @@ constexpr uint64_t kServeTicket = 1ull << 63;
 
 namespace {
 
+void destroy_ticket(xdrop_ctx *c, Ticket *tk)
+{
+    if (tk->ev_begin) cudaEventDestroy(tk->ev_begin);
+    if (tk->ev_end) cudaEventDestroy(tk->ev_end);
+    if (tk->ev_done) cudaEventDestroy(tk->ev_done);
+    if (tk->d_mem) {
+        cudaFree(tk->d_mem);
+        c->used -= tk->d_bytes;
+    }
+    if (tk->h_pinned) cudaFreeHost(tk->h_pinned);
+    delete tk;
+}
+
+// Gives back what is only kept for later calls: the idle tickets' buffers and
+// the seed pool's pages.  For a call that runs out of memory.
+void release_kept(xdrop_ctx *c)
+{
+    (void)cudaGetLastError();  // of the failed allocation
+    for (Ticket *tk : c->idle) destroy_ticket(c, tk);
+    c->idle.clear();
+    if (c->pool) {
+        cudaStreamSynchronize(c->stream);
+        cudaMemPoolTrimTo(c->pool, 0);
+    }
+}
+
+cudaError_t device_malloc(xdrop_ctx *c, void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        release_kept(c);
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 int dev_alloc(xdrop_ctx *c, DevBuf &b, size_t bytes)
 {
     if (b.cap >= bytes) return XDROP_OK;
@@ -193,7 +229,7 @@ int dev_alloc(xdrop_ctx *c, DevBuf &b, size_t bytes)
         b.p = nullptr;
         b.cap = 0;
     }
-    CK(cudaMalloc(&b.p, nb));
+    CK(device_malloc(c, &b.p, nb));
     b.cap = nb;
     c->used += nb;
     c->scratch_version += 1;
@@ -579,24 +615,12 @@ int seed_pool(xdrop_ctx *c)
     return XDROP_OK;
 }
 
-void destroy_ticket(xdrop_ctx *c, Ticket *tk)
-{
-    if (tk->ev_begin) cudaEventDestroy(tk->ev_begin);
-    if (tk->ev_end) cudaEventDestroy(tk->ev_end);
-    if (tk->ev_done) cudaEventDestroy(tk->ev_done);
-    if (tk->d_mem) {
-        cudaFree(tk->d_mem);
-        c->used -= tk->d_bytes;
-    }
-    if (tk->h_pinned) cudaFreeHost(tk->h_pinned);
-    delete tk;
-}
-
 // A ticket's events and buffers outlive it: allocating them is a good part of
 // a small call (64 short pairs: 100 us a call with new ones, 90 with kept
 // ones, 55 with the polling wait of xdrop_sync and the job as an argument).
 // At most kIdleTickets are kept, none larger than the limits, and no device
-// memory by a context with a memory budget; xdrop_free gives them back.
+// memory by a context with a memory budget; xdrop_free gives them back, and
+// so does a call that would run out of memory (release_kept).
 // All of it happens under the context's mutex, on tickets whose work is done.
 constexpr size_t kIdleTickets = 4, kIdlePinned = (size_t)64 << 20, kIdleDevice = (size_t)512 << 20;
 
@@ -626,7 +650,7 @@ cudaError_t ticket_mem(xdrop_ctx *c, Ticket *tk, size_t bytes)
         tk->d_mem = nullptr;
         tk->d_bytes = 0;
     }
-    const cudaError_t e = cudaMalloc(&tk->d_mem, bytes);
+    const cudaError_t e = device_malloc(c, &tk->d_mem, bytes);
     if (e != cudaSuccess) return e;
     tk->d_bytes = bytes;
     c->used += bytes;
@@ -717,20 +741,29 @@ int launch_ticket_chunked(xdrop_ctx *c, Ticket *tk, const xdrop_pair *h_pairs, s
     return XDROP_OK;
 }
 
-int new_ticket(xdrop_ctx *c, size_t n_pairs, bool device_submit, Ticket **out, size_t n_jobs = 1)
+// dev_bytes: of device memory that ticket_mem will be asked for.
+int new_ticket(xdrop_ctx *c, size_t n_pairs, size_t dev_bytes, Ticket **out, size_t n_jobs = 1)
 {
+    const bool device_submit = dev_bytes == 0;
     const size_t pin = align_up(sizeof(Job) * std::max<size_t>(n_jobs, 1)) + align_up(C_WORDS * 4) +
                        (device_submit ? 0 : align_up(n_pairs * sizeof(xdrop_result)));
-    // the idle ticket with the largest buffers, or a new one
+    // the smallest idle ticket whose buffers are large enough, else the
+    // largest, else a new one; a device submit leaves those with device memory
+    auto worth = [&](const Ticket *x) {
+        const int64_t size = (int64_t)(x->pin_bytes + x->d_bytes);
+        return x->pin_bytes >= pin && x->d_bytes >= dev_bytes ? INT64_MAX - size : size;
+    };
+    int pick = -1;
+    for (size_t k = 0; k < c->idle.size(); ++k) {
+        if (device_submit && c->idle[k]->d_mem) continue;
+        if (pick < 0 || worth(c->idle[k]) > worth(c->idle[pick])) pick = (int)k;
+    }
     Ticket *tk = nullptr;
-    if (!c->idle.empty()) {
-        auto it = std::max_element(c->idle.begin(), c->idle.end(), [](Ticket *x, Ticket *y) {
-            return x->pin_bytes + x->d_bytes < y->pin_bytes + y->d_bytes;
-        });
+    if (pick >= 0) {
         Ticket kept;
-        std::swap(kept, **it);
-        tk = *it;
-        c->idle.erase(it);
+        tk = c->idle[pick];
+        std::swap(kept, *tk);
+        c->idle.erase(c->idle.begin() + pick);
         tk->h_pinned = kept.h_pinned;
         tk->pin_bytes = kept.pin_bytes;
         tk->d_mem = kept.d_mem;
@@ -749,6 +782,10 @@ int new_ticket(xdrop_ctx *c, size_t n_pairs, bool device_submit, Ticket **out, s
         tk->h_pinned = nullptr;
         tk->pin_bytes = 0;
         e = cudaHostAlloc(&tk->h_pinned, pin, cudaHostAllocDefault);
+        if (e == cudaErrorMemoryAllocation) {
+            release_kept(c);
+            e = cudaHostAlloc(&tk->h_pinned, pin, cudaHostAllocDefault);
+        }
         if (e == cudaSuccess) tk->pin_bytes = pin;
     }
     if (e == cudaSuccess && !tk->ev_begin) e = cudaEventCreate(&tk->ev_begin);
@@ -835,15 +872,15 @@ int xdrop_submit(xdrop_ctx *c, const uint32_t *packed, const uint64_t *read_off,
     const uint64_t pk_words = any_rc ? 2 * n_words : n_words;
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
-    Ticket *tk = nullptr;
-    if ((rc = new_ticket(c, n_pairs, false, &tk))) return rc;
-    tk->out = out;
     // One device allocation for the inputs and results of this ticket.
     size_t o_packed = 0, o_off = align_up(std::max<uint64_t>(pk_words, 1) * 4);
     size_t o_len = o_off + align_up((size_t)std::max(n_reads, 1u) * 8);
     size_t o_pairs = o_len + align_up((size_t)std::max(n_reads, 1u) * 4);
     size_t o_out = o_pairs + align_up(std::max<size_t>(n_pairs, 1) * sizeof(xdrop_pair));
     size_t bytes = o_out + align_up(std::max<size_t>(n_pairs, 1) * sizeof(xdrop_result));
+    Ticket *tk = nullptr;
+    if ((rc = new_ticket(c, n_pairs, bytes, &tk))) return rc;
+    tk->out = out;
     if (c->budget && c->used + bytes > c->budget) {
         free_ticket(c, tk);
         return fail(c->tickets.empty() ? XDROP_ENOMEM : XDROP_EBUSY,
@@ -929,7 +966,7 @@ int xdrop_submit_device(xdrop_ctx *c, const uint32_t *packed, uint64_t n_words,
         c->maxlen_val = maxlen;
     }
     Ticket *tk = nullptr;
-    if ((rc = new_ticket(c, n_pairs, true, &tk))) return rc;
+    if ((rc = new_ticket(c, n_pairs, 0, &tk))) return rc;
     Job job{};
     job.packed = packed;
     job.n_words = (int64_t)n_words;
@@ -1140,9 +1177,12 @@ int xdrop_load_reads(xdrop_ctx *c, const uint32_t *packed, const uint64_t *read_
         // Packed 2x32 unless a tile was forced; requests whose scoring does
         // not fit it run on the serving kernel's 32-bit second tier.
         const Tile t = c->forced.lanes ? c->forced : Tile{2, 32, true};
-        c->srv = xd::server_create(c->device, c->sm_count, c->budget, t, rr, c->h_len.data(),
-                                   (int32_t *)c->wide.p, c->wide_per_cta, c->wide_grid,
-                                   c->serve_idle_ns, err);
+        for (int tries = 0; tries < 2 && !c->srv; ++tries) {
+            if (tries) release_kept(c);
+            c->srv = xd::server_create(c->device, c->sm_count, c->budget, t, rr, c->h_len.data(),
+                                       (int32_t *)c->wide.p, c->wide_per_cta, c->wide_grid,
+                                       c->serve_idle_ns, err);
+        }
         if (!c->srv) return fail(XDROP_ECUDA, "%s", err.c_str());
     }
     return XDROP_OK;
@@ -1208,11 +1248,11 @@ int xdrop_submit_pairs(xdrop_ctx *c, const xdrop_pair *pairs, size_t n_pairs,
         }
     }
     const size_t n_chunks = (std::max<size_t>(n_pairs, 1) + chunk - 1) / chunk;
-    Ticket *tk = nullptr;
-    if ((rc = new_ticket(c, n_pairs, false, &tk, n_chunks))) return rc;
-    tk->out = out;
     const size_t o_out = align_up(chunk * sizeof(xdrop_pair));
     const size_t bytes = o_out + align_up(chunk * sizeof(xdrop_result));
+    Ticket *tk = nullptr;
+    if ((rc = new_ticket(c, n_pairs, bytes, &tk, n_chunks))) return rc;
+    tk->out = out;
     if (c->budget && c->mode == XDROP_MODE_PLAIN && c->used + bytes > c->budget) {
         free_ticket(c, tk);
         return fail(c->tickets.empty() ? XDROP_ENOMEM : XDROP_EBUSY,
@@ -1327,11 +1367,18 @@ int xdrop_find_candidates(xdrop_ctx *c, const xdrop_kmer_params *p, xdrop_pair *
         const size_t left = c->budget ? (c->budget > c->used ? c->budget - c->used : 1) : 0;
         std::string err;
         if (int rc = seed_pool(c)) return rc;
-        const int rc = find_candidates(c->stream, c->pool, c->sm_count, left, (const uint32_t *)c->r_packed.p,
-                                       (const uint64_t *)c->r_off.p, (const uint32_t *)c->r_len.p,
-                                       c->r_n, c->h_len.data(), p->k, p->stride, p->lo, p->hi,
-                                       p->flags, c->cand_pairs, c->cand_shared, c->seed_stats,
-                                       err);
+        auto find = [&] {
+            return find_candidates(c->stream, c->pool, c->sm_count, left,
+                                   (const uint32_t *)c->r_packed.p, (const uint64_t *)c->r_off.p,
+                                   (const uint32_t *)c->r_len.p, c->r_n, c->h_len.data(), p->k,
+                                   p->stride, p->lo, p->hi, p->flags, c->cand_pairs,
+                                   c->cand_shared, c->seed_stats, err);
+        };
+        int rc = find();
+        if (rc == XDROP_ENOMEM && !c->budget && !c->idle.empty()) {
+            release_kept(c);
+            rc = find();
+        }
         if (rc) return fail(rc, "%s", err.c_str());
         c->cand_params = key;
         c->cand_gen = c->reads_gen;

@@ -19,7 +19,7 @@ namespace fake {
 struct Event { std::chrono::steady_clock::time_point at; };
 struct Graph { std::vector<std::function<void()>> run; };
 std::map<void *, size_t> device_mem;
-size_t device_used = 0, device_size = (size_t)-1, pool_reserved = 0;
+size_t device_used = 0, device_size = (size_t)-1, pool_reserved = 0, seed_tables = 0;
 int graphs = 0, last_longest = -1, bad_scratch = 0;
 int lose_entries = 0;                        // the next first tiers lose an entry
 std::atomic<int> late_us{0}, polling{0}, polling_max{0};
@@ -41,6 +41,7 @@ const char *xdrop_static_last_error(void) { return ""; }
 void fake_device_size(size_t bytes) { fake::device_size = bytes; }
 size_t fake_device_used(void) { return fake::device_used + fake::pool_reserved; }
 void fake_pool_reserved(size_t bytes) { fake::pool_reserved = bytes; }
+void fake_seed_tables(size_t bytes) { fake::seed_tables = bytes; }
 void fake_lose_entries(int n) { fake::lose_entries = n; }
 void fake_late_us(int us) { fake::late_us = us; }
 int fake_polling_max(void) { return fake::polling_max.exchange(0); }
@@ -200,8 +201,13 @@ cudaError_t launch_max_len(const uint32_t *len, uint32_t n, uint32_t *out, cudaS
 int find_candidates(cudaStream_t, cudaMemPool_t, int, size_t, const uint32_t *, const uint64_t *,
                     const uint32_t *, uint32_t, const uint32_t *, uint32_t, uint32_t, uint32_t,
                     uint32_t, uint32_t, std::vector<Pair> &, std::vector<uint32_t> &, SeedStats &,
-                    std::string &)
+                    std::string &err)
 {
+    if (fake::device_used + std::max(fake::seed_tables, fake::pool_reserved) > fake::device_size) {
+        err = "out of memory";
+        return XDROP_ENOMEM;
+    }
+    fake::pool_reserved = std::max(fake::seed_tables, fake::pool_reserved);
     return XDROP_OK;
 }
 Server *server_create(int, int, size_t, Tile, const ResidentReads &, const uint32_t *, int32_t *,

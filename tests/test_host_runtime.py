@@ -38,7 +38,7 @@ def X(built, tmp_path):
     spec.loader.exec_module(mod)
     mod.LIB_PATH = str(so)
     lib = mod.load()
-    for name in ("fake_device_size", "fake_pool_reserved"):
+    for name in ("fake_device_size", "fake_pool_reserved", "fake_seed_tables"):
         getattr(lib, name).argtypes = [ctypes.c_size_t]
         getattr(lib, name).restype = None
     lib.fake_device_used.restype = ctypes.c_size_t
@@ -106,3 +106,54 @@ def test_a_failed_load_leaves_no_half_read_set(X, budget):
             with pytest.raises(X.XdropError) as ei:
                 X.xdrop_submit_pairs(al.ctx, pairs, sc, out)
             assert ei.value.code == X.XDROP_EINVAL
+
+
+def _device_submit(X, al, job, sc):
+    packed, off, lens, pairs = job
+    out = np.zeros(len(pairs), X.RESULT_DTYPE)
+    p = [a.ctypes.data for a in (packed, off, lens, pairs, out)]
+    t = X.xdrop_submit_device(al.ctx, p[0], len(packed), p[1], p[2], len(lens), p[3], len(pairs),
+                              sc, p[4])
+    return t, (job, out)
+
+
+@pytest.mark.parametrize("call", ["submit", "load_reads", "scratch", "seeds"])
+def test_kept_memory_makes_room_for_a_call(X, call):
+    """Idle tickets keep their buffers and seed discovery its pages; a call that
+    runs out of memory gets them, as it did when nothing was kept."""
+    sc, mb = X.scoring(), 1 << 20
+    with X.Aligner() as al:
+        X.xdrop_load_reads(al.ctx, *_job(X, 3)[:3])
+        al.align(*_job(X, 4, words=16 * mb // 4), sc)  # a ticket with 16 MB stays
+        X.xdrop_find_candidates(al.ctx, k=9)           # makes the pool
+        X.fake.fake_pool_reserved(16 * mb)
+        X.fake.fake_device_size(X.fake.fake_device_used() + 2 * mb)
+        if call == "submit":
+            al.align(*_job(X, 4, words=24 * mb // 4), sc)
+        elif call == "load_reads":
+            X.xdrop_load_reads(al.ctx, *_job(X, 3, words=12 * mb // 4)[:3])
+        elif call == "scratch":
+            t, _keep = _device_submit(X, al, _long(X, 300_000), sc)
+            X.xdrop_sync(al.ctx, t)
+        else:
+            X.fake.fake_seed_tables(24 * mb)
+            X.xdrop_find_candidates(al.ctx, k=11)
+        assert X.fake.fake_device_used() <= 35 * mb
+
+
+def test_a_device_submit_leaves_the_large_buffers_idle(X):
+    """It needs none; the next host submit finds its buffer kept."""
+    sc = X.scoring()
+    with X.Aligner() as al:
+        big = _job(X, 4, words=1 << 20)
+        packed, off, lens, pairs = big
+        out = [np.zeros(4, X.RESULT_DTYPE) for _ in range(2)]
+        small = _job(X, 4)
+        t = [X.xdrop_submit(al.ctx, *job, sc, o) for job, o in zip((big, small), out)]
+        for k in t:
+            X.xdrop_sync(al.ctx, k)
+        used = X.fake.fake_device_used()
+        t, _keep = _device_submit(X, al, _job(X, 4), sc)
+        al.align(*big, sc)
+        assert X.fake.fake_device_used() == used
+        X.xdrop_sync(al.ctx, t)
