@@ -145,7 +145,7 @@ struct xdrop_ctx {
     cudaGraphExec_t gexec = nullptr;
     cudaEvent_t ev_main0 = nullptr, ev_main1 = nullptr;  // recorded inside the graph
     Tile graph_tile = {0, 0};
-    bool graph_brief = false;
+    bool graph_brief = false, graph_longest = false;
     uint32_t graph_launches = 0;
     uint64_t graph_version = ~0ull;
 
@@ -506,7 +506,8 @@ int pick_tile(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *out)
 int run_batched(xdrop_ctx *c, Ticket *tk, const Scoring &sc)
 {
     if (!c->gexec || c->graph_version != c->scratch_version ||
-        !c->graph_tile.same(c->tile0) || c->graph_brief != has_brief(c->tile0, sc)) {
+        !c->graph_tile.same(c->tile0) || c->graph_brief != has_brief(c->tile0, sc) ||
+        c->graph_longest != !c->forced.lanes) {
         c->tile0_bps = persistent_blocks_per_sm(c->tile0);
         if (c->gexec) {
             cudaGraphExecDestroy(c->gexec);
@@ -528,6 +529,7 @@ int run_batched(xdrop_ctx *c, Ticket *tk, const Scoring &sc)
         c->graph_version = c->scratch_version;
         c->graph_tile = c->tile0;
         c->graph_brief = has_brief(c->tile0, sc);
+        c->graph_longest = !c->forced.lanes;
         c->graph_launches = launches;
     }
     CK(cudaGraphLaunch(c->gexec, c->stream));

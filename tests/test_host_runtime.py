@@ -157,3 +157,17 @@ def test_a_device_submit_leaves_the_large_buffers_idle(X):
         al.align(*big, sc)
         assert X.fake.fake_device_used() == used
         X.xdrop_sync(al.ctx, t)
+
+
+@pytest.mark.parametrize("order", [(1, 0, 1), (0, 1, 0)], ids=["tuned_first", "forced_first"])
+def test_a_forced_tile_runs_without_the_longest_cut(X, order):
+    """The longest tasks skip the first tile only when it was tuned: the captured
+    launch of the one must not be replayed for the other."""
+    sc = X.scoring()
+    with X.Aligner() as al:
+        al.align(*_job(X, 40), sc)
+        lanes, cells = al.tile()
+        for tuned in order:
+            al.set_tile(*((0, 0) if tuned else (lanes, cells)))
+            al.align(*_job(X, 40), sc)
+            assert X.fake.fake_last_longest() == tuned
