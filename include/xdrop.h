@@ -120,7 +120,8 @@ typedef struct {
     uint32_t tile_lanes;     /* first band tier: lanes per extension      */
     uint32_t tile_cells;     /* first band tier: cells per lane, with
                                 XDROP_TILE_PACKED16 set for a packed tile */
-    uint64_t device_bytes;   /* device memory the context holds now       */
+    uint64_t device_bytes;   /* device memory the context holds now, kept
+                                buffers and seed-discovery pages included */
 } xdrop_stats;
 
 typedef struct {

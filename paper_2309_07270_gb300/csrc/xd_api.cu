@@ -1112,7 +1112,10 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st)
     if (!c || !st) return fail(XDROP_EINVAL, "NULL argument");
     std::lock_guard<std::mutex> lk(c->mu);
     *st = c->last;
-    st->device_bytes = c->used;
+    uint64_t pages = 0;  // of seed discovery, between its calls
+    if (c->pool && cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &pages) != cudaSuccess)
+        pages = 0;
+    st->device_bytes = c->used + pages;
     return XDROP_OK;
 }
 

@@ -171,3 +171,13 @@ def test_a_forced_tile_runs_without_the_longest_cut(X, order):
             al.set_tile(*((0, 0) if tuned else (lanes, cells)))
             al.align(*_job(X, 40), sc)
             assert X.fake.fake_last_longest() == tuned
+
+
+def test_device_bytes_holds_the_seed_pool(X):
+    """device_bytes is what the context holds now, pages kept between calls too."""
+    with X.Aligner() as al:
+        X.xdrop_load_reads(al.ctx, *_job(X, 3)[:3])
+        before = al.stats()["device_bytes"]
+        X.xdrop_find_candidates(al.ctx, k=9)
+        X.fake.fake_pool_reserved(1 << 20)
+        assert al.stats()["device_bytes"] == before + (1 << 20)
