@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -150,6 +151,7 @@ struct xdrop_ctx {
     uint64_t graph_version = ~0ull;
 
     xdrop_stats last = {};
+    std::atomic<bool> polling{false};  // a thread polls in xdrop_sync
 
     // resident reads (xdrop_load_reads) and the serving loop
     DevBuf r_packed, r_off, r_len;
@@ -1011,11 +1013,14 @@ int xdrop_sync(xdrop_ctx *c, xdrop_ticket t, int64_t timeout_ns)
     CK(cudaSetDevice(c->device));
     if (timeout_ns < 0) {
         // A blocking wait wakes 30 to 40 us late: poll first, for
-        // about as long as a small batch takes.
-        const auto until = std::chrono::steady_clock::now() + std::chrono::milliseconds(2);
+        // about as long as a small batch takes, on one thread at a time.
         cudaError_t q = cudaErrorNotReady;
-        while (q == cudaErrorNotReady && std::chrono::steady_clock::now() < until)
-            q = cudaEventQuery(tk->ev_done);
+        if (!c->polling.exchange(true)) {
+            const auto until = std::chrono::steady_clock::now() + std::chrono::milliseconds(2);
+            while (q == cudaErrorNotReady && std::chrono::steady_clock::now() < until)
+                q = cudaEventQuery(tk->ev_done);
+            c->polling = false;
+        }
         if (q == cudaErrorNotReady) q = cudaEventSynchronize(tk->ev_done);
         if (q != cudaSuccess) return fail(XDROP_ECUDA, "sync: %s", cudaGetErrorString(q));
     } else {

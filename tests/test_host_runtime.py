@@ -181,3 +181,21 @@ def test_device_bytes_holds_the_seed_pool(X):
         X.xdrop_find_candidates(al.ctx, k=9)
         X.fake.fake_pool_reserved(1 << 20)
         assert al.stats()["device_bytes"] == before + (1 << 20)
+
+
+def test_one_thread_polls(X):
+    """Waiting threads beside the first sleep until their result is there."""
+    import threading
+    sc = X.scoring()
+    X.fake.fake_late_us(1500)
+    with X.Aligner() as al:
+        job = _job(X, 4)
+        out = [np.zeros(4, X.RESULT_DTYPE) for _ in range(6)]
+        tickets = [X.xdrop_submit(al.ctx, *job, sc, o) for o in out]
+        X.fake.fake_polling_max()
+        th = [threading.Thread(target=X.xdrop_sync, args=(al.ctx, t)) for t in tickets]
+        for t in th:
+            t.start()
+        for t in th:
+            t.join()
+        assert X.fake.fake_polling_max() == 1
