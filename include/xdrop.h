@@ -380,7 +380,8 @@ int xdrop_accept_device(xdrop_ctx *c, const xdrop_pair *pairs, const xdrop_resul
 
 /* Task ids (2*pair + 1 for a right extension, 2*pair for a left one)
  * that the first band tier handed to a wider tier during the most recently
- * synced ticket.  Copies up to cap ids to dst (host memory) and the total
+ * synced ticket, or that outgrew their first window where a warp ran them
+ * beside it (the overflow_tasks of xdrop_stats).  Copies up to cap ids to dst (host memory) and the total
  * number to *n.  For diagnostics and for separating the first tier's work
  * in rate measurements. */
 int xdrop_last_spills(xdrop_ctx *c, uint32_t *dst, size_t cap, size_t *n);

@@ -302,8 +302,10 @@ WarpRole role_of(xdrop_ctx *c, Tile t)
 {
     if (!has_warp_role(t)) return WarpRole{};
     uint32_t *w = c->d_ctrs + C_ROLE;
-    return WarpRole{w, w + 1, w + 2, w + 3, w + 4, w + 5, c->d_ctrs + C_GROWN, c->d_ctrs + C_ROLE_ERR,
-                    spill_of(c, 1), 0};
+    // the longest tasks never enter the overflow list, so there is room at its
+    // end for those that outgrow their window
+    return WarpRole{w, w + 1, w + 2, w + 3, w + 4, w + 5, c->d_ctrs + C_GROWN,
+                    spill_of(c, 0).list + c->cap_tasks, c->d_ctrs + C_ROLE_ERR, spill_of(c, 1), 0};
 }
 
 bool has_brief(Tile t0, const Scoring &sc)
@@ -324,7 +326,8 @@ int enqueue_brief(xdrop_ctx *c)
     uint32_t *ctr = c->d_ctrs, *w = ctr + C_ROLE2, *list = (uint32_t *)c->order.p;
     const int grid = c->sm_count * bps;
     const uint32_t few = (uint32_t)(grid * persistent_block_threads(t) / 32);
-    const WarpRole role{w, w + 1, w + 2, w + 3, w + 4, w + 5, w + 6, ctr + C_ROLE_ERR, spill_of(c, 1), few};
+    const WarpRole role{w, w + 1, w + 2, w + 3, w + 4, w + 5, w + 6, nullptr, ctr + C_ROLE_ERR,
+                        spill_of(c, 1), few};
     CK(cudaMemsetAsync(list, 0xFF, c->cap_tasks * 4, c->stream));
     CK(launch_persistent(t, grid, c->d_job, (uint32_t *)c->spill[2].p, ctr + C_BRIEF,
                          ctr + C_COUNTER2, Spill{list, ctr + C_SPILL2}, Spill{}, role, c->stream));
@@ -1479,15 +1482,16 @@ int xdrop_last_spills(xdrop_ctx *c, uint32_t *dst, size_t cap, size_t *n)
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
     CK(cudaStreamSynchronize(c->stream));
-    // the long overflow of the first tier, then the short
-    const int word[2] = {C_SPILL0, C_BRIEF}, list[2] = {0, 2};
+    // the long overflow of the first tier, the short, the longest tasks that
+    // outgrew a warp's first window (role_of)
+    const int word[3] = {C_SPILL0, C_BRIEF, C_GROWN}, list[3] = {0, 2, 0};
     size_t total = 0;
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < 3; ++k) {
         uint32_t cnt = 0;
         CK(cudaMemcpy(&cnt, c->d_ctrs + word[k], 4, cudaMemcpyDeviceToHost));
         const size_t take = total < cap ? std::min<size_t>(cap - total, cnt) : 0;
-        if (take)
-            CK(cudaMemcpy(dst + total, c->spill[list[k]].p, take * 4, cudaMemcpyDeviceToHost));
+        const uint32_t *from = (const uint32_t *)c->spill[list[k]].p + (k == 2 ? c->cap_tasks - cnt : 0);
+        if (take) CK(cudaMemcpy(dst + total, from, take * 4, cudaMemcpyDeviceToHost));
         total += cnt;
     }
     *n = total;

@@ -91,7 +91,10 @@ static __device__ __noinline__ void run_warp_role(const Job *jp, const uint32_t 
         int32_t sc, bi, bj;
         const int st = extend_warp(e, J.sc, whole ? 0 : width, lane, sc, bi, bj);
         if (lane == 0) {
-            if (whole && st) atomicAdd(role.grown, 1u);
+            if (whole && st) {
+                const uint32_t k = atomicAdd(role.grown, 1u);
+                if (role.grown_end) *(role.grown_end - 1 - k) = task;
+            }
             if (st < 0) hand_on_wide(role.wide, task, e.m);
             else write_result(J, e, sc, bi, bj);
         }

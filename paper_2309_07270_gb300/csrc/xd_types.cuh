@@ -83,6 +83,7 @@ struct WarpRole {
     uint32_t *taken;     // overflow entries taken
     uint32_t *done;      // first-tier warps that found no more tasks
     uint32_t *grown;     // longest tasks that outgrew a warp's first window
+    uint32_t *grown_end; // their ids, stored downwards from here (null: not noted)
     uint32_t *err;       // set when an overflow entry never appeared
     Spill wide;          // tasks for the unbounded tier
     uint32_t few;        // up to this many tasks all go to single warps
