@@ -645,13 +645,20 @@ int row_product(Arena &ar, const Front &f, std::vector<Pair> &out_pairs,
     uint64_t *cand_cnt, *cand_end;
     uint32_t *flags, *big;  // flags[0]: table overflow, flags[1]: reads listed in big
     Stage stage;
-    XS_GET(cand_cnt, n_reads);
-    XS_GET(cand_end, n_reads);
-    XS_GET(flags, 2);
-    XS_GET(big, n_reads);
-    XS_GET(stage.key, (uint64_t)n_reads * kStage);
-    XS_GET(stage.best, (uint64_t)n_reads * kStage);
-    XS_GET(stage.cnt, (uint64_t)n_reads * kStage);
+    const uint64_t n_stage = (uint64_t)n_reads * kStage;
+    if (!(ar.get(cand_cnt, n_reads) && ar.get(cand_end, n_reads) && ar.get(flags, 2) &&
+          ar.get(big, n_reads) && ar.get(stage.key, n_stage) && ar.get(stage.best, n_stage) &&
+          ar.get(stage.cnt, n_stage))) {
+        // without a reliable k-mer there is nothing to accumulate (asked only
+        // here: the answer costs a round trip)
+        const int rc = ar.rc;
+        if (rc != XDROP_ENOMEM) return rc;
+        if (read_back(ar, &h_counts, counts)) return ar.rc;
+        if (h_counts.nonzeros) return rc;
+        ar.rc = XDROP_OK;
+        *done = true;
+        return XDROP_OK;
+    }
     XS_CK(cudaMemsetAsync(flags, 0, 8, ar.s));
     row_kernel<false><<<n_reads, kRowThreads, 0, ar.s>>>(
         f.occ_off, row_of, members, f.read_len, f.k, f.stride, f.nb, f.n_occ, cand_cnt, nullptr, flags,
