@@ -267,9 +267,10 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st);
  * 4x16, 8x8, 2x32, 8x16, 16x8, 4x32, 1x32, 2x64.  Returns XDROP_EINVAL for
  * another shape.  Serving mode (set the tile before the first xdrop_submit_pairs)
  * runs packed 2x32 by default (other packed tiles of 32 or 64 cells per lane
- * serve as the 16-cell tile of their width); with a packed first tier,
- * requests whose scoring does not fit it (16 bits; for 2x32 also x + 2 match
- * + 2|gap| <= 1023) run on the serving kernel's 32-bit second tier. */
+ * serve as the 16-cell tile of their width), and 4x16 from the first request
+ * on whose scoring fits 16 bits but not 2x32 (x + 2 match + 2|gap| <= 1023);
+ * with a packed first tier, requests whose scoring does not fit 16 bits run
+ * on the serving kernel's 32-bit second tier. */
 int xdrop_set_tile(xdrop_ctx *c, int lanes, int cells);
 
 /* Several seeds per read pair, keeping the best extension.  Consecutive

@@ -165,6 +165,7 @@ public:
     std::thread worker;
 
     void run();
+    bool tile_holds(const Req *r);
     bool admit(Req *r);
     void complete_kernel_part(Req *r);
     void finish_copy(Req *r);
@@ -183,6 +184,9 @@ cudaError_t set_flag(Server *s, unsigned int *field, int value, cudaStream_t st)
 }
 
 }  // namespace
+
+// Blocks of the serving kernel: room is left for the side-stream pass.
+int serve_grid(Tile t, int sm_count) { return std::max(1, serve_blocks_per_sm(t) * sm_count - 2); }
 
 bool Server::wait_kernel_exit(double secs)
 {
@@ -229,6 +233,28 @@ cudaError_t Server::ensure_kernel()
         stats.relaunches += 1;
     }
     return e;
+}
+
+// Whether the kernel's tile is right for a request.  Lanes of 32 slots hold
+// fewer scorings than lanes of 16, and a request whose scoring the tile does
+// not hold runs on the second tier alone (24 requests, 203,406 pairs, x =
+// 950 at 16/-16/-32: 5.8 s, on 4x16 0.08).  So from the first request that
+// needs 16 slots on the kernel runs 4x16: what is in flight ends first, then
+// the kernel is stopped for good.
+bool Server::tile_holds(const Req *r)
+{
+    const Tile t = tile;
+    if (!(t.packed && t.lanes == 2 && t.c == 32) || !packed_scoring_ok(r->sc)) return true;
+    if (packed_tile_ok(t, r->sc) && !in_frame(t, r->sc).absolute) return true;
+    for (auto *q : slots)
+        if (q) return false;
+    if (kernel_running) {  // the worker's loop waits for its exit
+        if (!stop_sent && set_flag(this, &d_ctl->stop, 1, s_copy) == cudaSuccess) stop_sent = true;
+        return false;
+    }
+    tile = Tile{4, 16, true};
+    grid = serve_grid(tile, sm_count);
+    return true;
 }
 
 bool Server::admit(Req *r)
@@ -459,7 +485,7 @@ void Server::run()
         // admission, in arrival order
         bool published_any = false;
         while (!queue.empty() && fatal.empty()) {
-            if (!admit(queue.front())) break;
+            if (!tile_holds(queue.front()) || !admit(queue.front())) break;
             queue.pop_front();
             published_any = true;
             progress = true;
@@ -514,13 +540,12 @@ Server *server_create(int device, int sm_count, size_t device_budget, Tile tile,
     (void)wide_scratch;
     s->wide_per_cta = wide_per_cta;
     s->wide_grid = wide_grid;
-    const int bps = serve_blocks_per_sm(tile);
-    if (bps <= 0) {
+    if (serve_blocks_per_sm(tile) <= 0) {
         err = "serving tile not available";
         delete s;
         return nullptr;
     }
-    s->grid = std::max(1, bps * sm_count - 2);  // room for the side-stream pass
+    s->grid = serve_grid(tile, sm_count);
     const size_t arena = device_budget ? device_budget : ((size_t)1 << 30);
     s->dev_arena = Arena(arena);
     s->host_arena = Arena(kHostPool);
