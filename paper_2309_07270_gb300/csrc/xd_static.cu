@@ -43,6 +43,9 @@ constexpr int32_t kWideLeft = 1 << 8;
 // XDROP_STATUS_TOO_LONG and zeros in its side's three fields; a band wider
 // than 512 slots is left to static_wide_kernel (64 pairs of 2-4 kb reads:
 // 5.9 ms with a CTA per task on the scratch alone, 0.4 ms this way).
+// Without WINDOWS every extension is left to it: the launch decides that by
+// the length of the buffer (a test per task took 64 pairs from 413 to 420 us).
+template <bool WINDOWS>
 __global__ void __launch_bounds__(kWarpThreads)
 static_warp_kernel(Job J, int64_t per_cta)
 {
@@ -67,7 +70,7 @@ static_warp_kernel(Job J, int64_t per_cta)
             continue;
         }
         int32_t sc, bi, bj;
-        const int st = extend_warp(e, J.sc, 0, lane, sc, bi, bj);
+        const int st = WINDOWS ? extend_warp(e, J.sc, 0, lane, sc, bi, bj) : -1;
         if (lane == 0) {
             if (st < 0) atomicOr(&o[6], kWideLeft << e.side);
             else write_result(J, e, sc, bi, bj);
@@ -179,7 +182,8 @@ extern "C" int xdrop_align_static(const uint32_t *packed, uint64_t n_words,
     const uint64_t cb = (n_pairs + 255) / 256;
     static_clear_status<<<(unsigned)std::min<uint64_t>(cb, 1024), 256, 0, st>>>(J);
     const uint64_t wb = (2 * n_pairs + kWarpThreads / 32 - 1) / (kWarpThreads / 32);
-    static_warp_kernel<<<(unsigned)std::min<uint64_t>(wb, 4096), kWarpThreads, 0, st>>>(J, per_cta);
+    const auto warps = J.n_words <= kWarp16Words ? static_warp_kernel<true> : static_warp_kernel<false>;
+    warps<<<(unsigned)std::min<uint64_t>(wb, 4096), kWarpThreads, 0, st>>>(J, per_cta);
     static_wide_kernel<<<grid, WIDE_THREADS, 0, st>>>(J, scratch, per_cta);
     e = cudaGetLastError();
     if (e != cudaSuccess) return static_fail(XDROP_ECUDA, "kernel launch", e);

@@ -279,30 +279,29 @@ __device__ __forceinline__ int extend_warp16(const Ext &e, const Scoring sc, int
     return 0;
 }
 
-// Words of a buffer whose bases extend_warp16 can name: it counts words in 32
-// bits, and an extension's last loads lie up to 2^21 words and a window
+// Words of the longest buffer for extend_warp: extend_warp16 counts words in
+// 32 bits, and an extension's last loads lie up to 2^21 words and a window
 // behind its first base.
 constexpr int64_t kWarp16Words = INT32_MAX - (1 << 22);
 
 // Extends one task with the whole warp on windows of 128 slots (packed if the
-// scoring and the buffer fit, else 32-bit), 256 (packed only) and 512 slots
+// scoring fits, else 32-bit), 256 (packed scorings only) and 512 slots
 // (32-bit), from the first that is wider than `from` slots.  Returns how many
 // of them the band outgrew, or -1 for all.
 __device__ __forceinline__ int extend_warp(const Ext &e, const Scoring &s, int from, int lane,
                                            int32_t &best, int32_t &bi, int32_t &bj)
 {
     const Scoring sc = effective(s);
-    const bool fits = e.A.nw <= kWarp16Words;
     int64_t cells;
     int grown = 0;
     if (from < 128) {
-        const int st = fits && warp16_ok<2>(sc)
+        const int st = warp16_ok<2>(sc)
                            ? extend_warp16<2>(e, sc, lane, best, bi, bj)
                            : extend_window<32, 4, false>(e, sc, lane, 0, best, bi, bj, cells);
         if (!st) return 0;
         ++grown;
     }
-    if (fits && warp16_ok<4>(sc)) {
+    if (warp16_ok<4>(sc)) {
         if (!extend_warp16<4>(e, sc, lane, best, bi, bj)) return grown;
         ++grown;
     }

@@ -1,5 +1,6 @@
-"""xdrop_align_static on a packed buffer of more than 2^31 words: only it takes
-one, as its extensions name bases in 64 bits wherever 32 are not enough."""
+"""xdrop_align_static on a packed buffer of more than 2^31 words (no other call
+takes one): its extensions then run on the scratch, which names bases in 64
+bits, and those of a buffer just short of the limit on the windows."""
 import numpy as np
 import pytest
 
