@@ -257,13 +257,14 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st);
  * and `cells` cells per lane (lanes*cells slots per anti-diagonal parity),
  * or pass lanes = 0 to go back to autotuning.  Autotuning (the default)
  * keys the first tile by the scoring and the job's length bucket (the
- * octave of an extension's min(m, n) that holds the median of the job's work,
- * read from a device histogram at every batched submit).  The first submit with a new key times the first-tier tiles on
- * its pairs, or on a stratified random sample of a large job (one pair of
- * every 3 above 150,000 with the packed tiles when the scoring fits them,
- * else one of every 8 above 12,288 with the 32-bit tiles; widths far from x / |gap| are left out) and keeps the
- * fastest for that key.  Tiles: 4x16, 8x8, 16x4,
- * 8x16, 16x8, 32x4, and packed (cells | XDROP_TILE_PACKED16) 4x8, 2x16,
+ * octave of an extension's min(m, n) that holds the median of the job's
+ * work, read from a device histogram at every batched submit).  The first
+ * submit with a new key times the first-tier tiles on its pairs, or on a
+ * stratified random sample of a large job (one pair of every 3 above 150,000
+ * with the packed tiles when the scoring fits them, else one of every 8 above
+ * 12,288 with the 32-bit tiles; widths far from x / |gap| are left out) and
+ * keeps the fastest for that key; a tuned job's longest extensions may start
+ * on single warps beside the tile.  Tiles: 4x16, 8x8, 16x4, 8x16, 16x8, 32x4, and packed (cells | XDROP_TILE_PACKED16) 4x8, 2x16,
  * 4x16, 8x8, 2x32, 8x16, 16x8, 4x32, 1x32, 2x64.  Returns XDROP_EINVAL for
  * another shape.  Serving mode (set the tile before the first xdrop_submit_pairs)
  * runs packed 2x32 by default (other packed tiles of 32 or 64 cells per lane
@@ -315,7 +316,9 @@ int xdrop_best_seeds_device(xdrop_ctx *c, const xdrop_pair *pairs, const xdrop_r
  * submits too) wait until it returns.  Limits: 1 <= k <= 32, stride >= 1,
  * 1 <= lo <= hi <= 1024 (XDROP_EINVAL; also without resident reads);
  * fewer than 2^31 occurrences and 2^31 (pair, shared k-mer) entries, and
- * the context's memory budget (XDROP_ENOMEM).
+ * the context's memory budget (XDROP_ENOMEM).  Without a budget the context
+ * keeps up to 4 GB of the tables' pages for the next call (xdrop_stats counts
+ * them); it gives them back when one of its calls runs out of memory.
  *
  * Two products compute the same candidates.  XDROP_SEEDS_ROWWISE (default)
  * builds A's rows and columns and accumulates each read's partners in a
@@ -382,8 +385,8 @@ int xdrop_accept_device(xdrop_ctx *c, const xdrop_pair *pairs, const xdrop_resul
 /* Task ids (2*pair + 1 for a right extension, 2*pair for a left one)
  * that the first band tier handed to a wider tier during the most recently
  * synced ticket, or that outgrew their first window where a warp ran them
- * beside it (the overflow_tasks of xdrop_stats).  Copies up to cap ids to dst (host memory) and the total
- * number to *n.  For diagnostics and for separating the first tier's work
+ * beside it (the overflow_tasks of xdrop_stats).  Copies up to cap ids to
+ * dst (host memory) and the total number to *n.  For diagnostics and for separating the first tier's work
  * in rate measurements. */
 int xdrop_last_spills(xdrop_ctx *c, uint32_t *dst, size_t cap, size_t *n);
 
@@ -417,9 +420,10 @@ int xdrop_count_cells_device(xdrop_ctx *c, const uint32_t *packed,
  * first call before any stream capture that should contain later calls.
  * All calls on a device share the array: calls whose work may overlap on
  * the GPU race and must be ordered (same stream, or events).  Every
- * extension has a warp of its own (windows of 128, then 512 slots); wider
- * bands run on the unbounded tier (one CTA per extension).  While the call's
- * work runs, a pair's status may hold further bits; they are clear once it
+ * extension has a warp of its own (windows of 128, 256, then 512 slots; the
+ * packed buffer may be longer than the 2^32 bases of the layout above, but
+ * from about 2^31 words on all of them run as the following do); wider bands
+ * run on the unbounded tier (one CTA per extension).  While the call's work runs, a pair's status may hold further bits; they are clear once it
  * is done.
  *
  * max_read_len must bound every read length; it sizes the per-CTA scratch

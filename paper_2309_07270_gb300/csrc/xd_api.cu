@@ -5,11 +5,12 @@
 // in batched mode, one instantiated CUDA graph of the whole launch
 // sequence.  Kernels read their job descriptor from device memory, so the
 // graph is replayed unchanged for every submit (and every chunk of a
-// large submit); it is re-captured only when scratch has to grow.
+// large submit); it is re-captured when scratch has to grow or the job's
+// tiles change.
 //
 // Plain mode is the paper's baseline scheme (Section "Baseline": the work
 // is split into batches of 10,000 and each is fed to the GPU in turn): one
-// launch of the 32-lane tile per 10,000-pair sub-batch, in submit order.
+// launch of the first band tile per 10,000-pair sub-batch, in submit order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -386,9 +387,9 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     // faster than the 32-bit tile of its shape), on the whole job, or a third
     // of a large one, so that the end of the sample, where few extensions are
     // left, does not decide between tiles of different concurrency; other
-    // scorings time the 32-bit tiles on an eighth.  The sample is stratified and random (one
-    // pair out of every block of 3 or 8, seeded), so it has the job's
-    // length mix even when the input is sorted or clustered.
+    // scorings time the 32-bit tiles on an eighth.  The sample is stratified
+    // and random (one pair out of every block of 3 or 8, seeded), so it has
+    // the job's length mix even when the input is sorted or clustered.
     //
     // The sample and its results live in the job's own result buffer
     // (48 bytes per sampled pair, at most 16 of the 28 bytes per pair there),
@@ -1042,7 +1043,7 @@ int xdrop_sync(xdrop_ctx *c, xdrop_ticket t, int64_t timeout_ns)
     auto it = c->tickets.find(t);
     if (it == c->tickets.end()) return fail(XDROP_EINVAL, "ticket %llu already synced", (unsigned long long)t);
     c->tickets.erase(it);
-    if (tk->h_ctrs[C_WIDE_M] > c->maxlen_val) c->maxlen_ptr = nullptr;  // measure again
+    if (tk->device_submit && tk->h_ctrs[C_WIDE_M] > c->maxlen_val) c->maxlen_ptr = nullptr;  // measure again
     if (tk->device_submit && tk->h_ctrs[C_UNFIT]) {
         uint32_t maxlen = 0;
         tk->launches = tk->graph_replays = 0;

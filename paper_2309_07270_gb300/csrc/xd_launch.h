@@ -12,7 +12,7 @@
 namespace xd {
 
 struct Tile {
-    int lanes;            // lanes per extension (4, 8, 16 or 32)
+    int lanes;            // lanes per extension (4, 8, 16 or 32; packed also 1 and 2)
     int c;                // cells per lane per diagonal
     bool packed = false;  // 16-bit cells, two per register (xd_lockstep16.cuh)
     bool absolute = false;  // packed: cells in the absolute frame (in_frame)

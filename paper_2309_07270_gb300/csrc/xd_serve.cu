@@ -46,9 +46,10 @@ constexpr uint64_t kRing = 1ull << kRingBits;
 constexpr size_t kAlign = 256;
 constexpr size_t kHostPool = (size_t)512 << 20;  // pinned staging
 // The host stops the serving kernel once nothing has been queued or in
-// flight for kHostIdleS (until then it holds the GPU, and whoever waits for the
-// device waits for it; a relaunch costs tens of microseconds); kIdleNs only bounds a group's wait if that never
-// happens (hang guard), so groups do not drop out during ordinary lulls.
+// flight for kHostIdleS (until then it holds the GPU, and whoever waits for
+// the device waits for it; a relaunch costs tens of microseconds); kIdleNs
+// only bounds a group's wait if that never happens (hang guard), so groups do
+// not drop out during ordinary lulls.
 constexpr unsigned long long kIdleNs = 5ull * 1000 * 1000 * 1000;
 constexpr double kHostIdleS = 0.01;
 constexpr double kShutdownWaitS = 60.0;       // bound on draining at context free

@@ -26,7 +26,7 @@
 // prune (dp16r), two diagonals' chains overlap.
 //
 // Measured, one extension per warp scheduler: a diagonal takes 57 ns (200 pairs
-// of 2-4 kb reads: 0.44 ms of kernels, 0.50 ms a call) against 81 ns for the
+// of 2-4 kb reads: 0.41 ms of kernels, 0.44 ms a call) against 81 ns for the
 // same window in lockstep16_loop's order and about 200 ns before (1.59 ms a
 // call on the 16x8 tile).  As the tier behind a 2x32 first tier (29x, x = 50,
 // 3,582 extensions) it takes 2.5 ms where the 32-bit window of 128 slots took 8.2.

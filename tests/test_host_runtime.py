@@ -23,6 +23,7 @@ def built(tmp_path_factory):
         pytest.skip("no g++ or no CUDA headers")
     so = tmp_path_factory.mktemp("fake") / "libfake.so"
     subprocess.run([gxx, "-x", "c++", "-std=c++17", "-O1", "-w", "-shared", "-fPIC", "-pthread",
+                    "-Wl,-Bsymbolic",  # not the CUDA runtime that torch has loaded
                     "-I", os.path.join(os.path.dirname(HERE), "include"), "-I", include, "-o",
                     str(so), os.path.join(HERE, "fake_cuda.cpp")], check=True)
     return str(so)
