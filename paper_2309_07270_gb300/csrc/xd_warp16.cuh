@@ -284,6 +284,52 @@ __device__ __forceinline__ int extend_warp16(const Ext &e, const Scoring sc, int
 // behind its first base.
 constexpr int64_t kWarp16Words = INT32_MAX - (1 << 22);
 
+// Task source of lockstep16_loop for one extension and the whole warp.
+struct OneSrc {
+    static constexpr bool kCanAbort = false;
+    const Ext &e;
+    const Scoring &s;
+    bool fresh = true;
+    int32_t status = 1, best = 0, bi = 0, bj = 0;  // lane 0
+    __device__ __forceinline__ int fetch_warp(unsigned, int, int, unsigned, bool, uint32_t &,
+                                              const Job *&)
+    {
+        const bool first = fresh;
+        fresh = false;
+        return first ? 1 : -1;
+    }
+    __device__ __forceinline__ void idle() {}
+    __device__ __forceinline__ bool aborted() const { return false; }
+    __device__ __forceinline__ Ext open(const Job *, uint32_t, Scoring &sc)
+    {
+        sc = s;
+        return e;
+    }
+    __device__ __forceinline__ void retire(const Job *, uint32_t, bool overflow, int32_t T, int32_t i,
+                                           int32_t j)
+    {
+        status = overflow;
+        best = T;
+        bi = i;
+        bj = j;
+    }
+};
+
+// extend_warp16<2>'s window for the packed scorings beyond warp16_ok: the group
+// loop on 32 lanes of 4 slots, whose keys take 16 units where a window's take
+// 128 (81 ns a diagonal; the 32-bit window about 200).  Out of line and on
+// copies, so that it costs the callers' registers nothing.
+struct WarpResult { int32_t status, best, bi, bj; };
+static __device__ __noinline__ WarpResult extend_lockstep16(const Ext &e, const Scoring &sc)
+{
+    OneSrc src{e, sc};
+    uint32_t one;
+    asm volatile("mov.u32 %0, 1;" : "=r"(one));
+    lockstep16_loop<32, 2>(src, e.A.pk, e.A.nw, one);
+    return WarpResult{__shfl_sync(FULL, src.status, 0), __shfl_sync(FULL, src.best, 0),
+                      __shfl_sync(FULL, src.bi, 0), __shfl_sync(FULL, src.bj, 0)};
+}
+
 // Extends one task with the whole warp on windows of 128 slots (packed if the
 // scoring fits, else 32-bit), 256 (packed scorings only) and 512 slots
 // (32-bit), from the first that is wider than `from` slots.  Returns how many
@@ -295,9 +341,20 @@ __device__ __forceinline__ int extend_warp(const Ext &e, const Scoring &s, int f
     int64_t cells;
     int grown = 0;
     if (from < 128) {
-        const int st = warp16_ok<2>(sc)
-                           ? extend_warp16<2>(e, sc, lane, best, bi, bj)
-                           : extend_window<32, 4, false>(e, sc, lane, 0, best, bi, bj, cells);
+        int st;
+        if (warp16_ok<2>(sc)) {
+            st = extend_warp16<2>(e, sc, lane, best, bi, bj);
+        } else if (packed16_ok(sc)) {
+            const Ext ec = e;
+            const Scoring scc = sc;
+            const WarpResult r = extend_lockstep16(ec, scc);
+            st = r.status;
+            best = r.best;
+            bi = r.bi;
+            bj = r.bj;
+        } else {
+            st = extend_window<32, 4, false>(e, sc, lane, 0, best, bi, bj, cells);
+        }
         if (!st) return 0;
         ++grown;
     }
