@@ -262,10 +262,12 @@ int xdrop_get_stats(xdrop_ctx *c, xdrop_stats *st);
  * submit with a new key times the first-tier tiles on its pairs, or on a
  * stratified random sample of a large job (one pair of every 3 above 150,000
  * with the packed tiles when the scoring fits them, else one of every 8 above
- * 12,288 with the 32-bit tiles; widths far from x / |gap| are left out) and
- * keeps the fastest for that key; a tuned job's longest extensions may start
- * on single warps beside the tile.  Tiles: 4x16, 8x8, 16x4, 8x16, 16x8, 32x4, and packed (cells | XDROP_TILE_PACKED16) 4x8, 2x16,
- * 4x16, 8x8, 2x32, 8x16, 16x8, 4x32, 1x32, 2x64.  Returns XDROP_EINVAL for
+ * 12,288 with the 32-bit tiles), and keeps the fastest for that key.  Widths
+ * far from x / |gap| are left out, but for 32-bit tiles on a small job.  A
+ * tuned job's longest extensions may start on single warps beside the tile.
+ * Tiles: 4x16, 8x8, 16x4, 8x16, 16x8, 32x4, and packed (cells |
+ * XDROP_TILE_PACKED16) 4x8, 2x16, 4x16, 8x8, 2x32, 8x16, 16x8, 4x32, 1x32,
+ * 2x64.  Returns XDROP_EINVAL for
  * another shape.  Serving mode (set the tile before the first xdrop_submit_pairs)
  * runs packed 2x32 by default (other packed tiles of 32 or 64 cells per lane
  * serve as the 16-cell tile of their width), and 4x16 from the first request

@@ -417,7 +417,10 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     // Widths worth timing: a gap step costs |gap| and moves half a slot, so
     // a live band spans at most about x / |gap| slots.  A window under 3/4 of
     // that overflows too often to win, one over 3 times it computes mostly
-    // dead slots.
+    // dead slots.  A small job on 32-bit tiles times all of them: its longest
+    // extensions end it there, and more lanes make a shorter diagonal (pairs
+    // of 1-3 kb reads at 100/-200/-60, x = 900: 1,500 of them 32x4 2.3 ms, 4x16
+    // 3.6; 30,000 of 0.2-1.5 kb 6.6 and 2.6).
     const int64_t span = sc.x / -(int64_t)sc.gap;
     const int64_t min_w = std::min<int64_t>(128, span * 3 / 4);
     const int64_t max_w = std::max<int64_t>(64, span * 3);
@@ -434,7 +437,7 @@ int autotune(xdrop_ctx *c, Ticket *tk, const Job &job, Tile *best)
     for (const Tile &cand : cands) {
         if (cand.packed && !packed_tile_ok(cand, sc)) continue;
         const Tile t = in_frame(cand, sc);
-        if (t.width() < min_w || t.width() > max_w) continue;
+        if ((packed || stride > 1) && (t.width() < min_w || t.width() > max_w)) continue;
         if (long_lanes && (t.c < 16 || (t.c == 16 && t.lanes == 4))) continue;
         const int bps = persistent_blocks_per_sm(t);
         if (bps <= 0) continue;
