@@ -10,7 +10,10 @@ namespace xd {
 // A warp per task: tasks list[0 .. *n_ptr), or all tasks of the job without
 // a list, by a counter; tasks too wide for 512 slots go to out.  Without a
 // list: tasks that outgrew 128 slots are noted in over, and with n_bad the
-// pairs are validated as validate_kernel does.
+// pairs are validated as validate_kernel does.  ANY as in extend_warp: its code
+// costs the others registers (137 and 165) and 200 pairs of 2-4 kb reads 8 us
+// of 443.
+template <bool ANY>
 __global__ void __launch_bounds__(kWarpThreads)
 warp_kernel(Job *jp, const Job value, bool by_value, const uint32_t *list, const uint32_t *n_ptr, uint32_t *counter,
             int from, uint32_t *n_bad, Spill over, Spill out)
@@ -29,7 +32,7 @@ warp_kernel(Job *jp, const Job value, bool by_value, const uint32_t *list, const
         if (n_bad && e.side == 0 && lane == 0) write_status(J, e.pair, e.ok, n_bad);
         if (!e.ok) continue;
         int32_t sc, bi, bj;
-        const int st = extend_warp(e, J.sc, from, lane, sc, bi, bj);
+        const int st = extend_warp<ANY>(e, J.sc, from, lane, sc, bi, bj);
         if (lane == 0) {
             if (!list && st) over.list[atomicAdd(over.count, 1u)] = task;
             if (st < 0) hand_on_wide(out, task, e.m);
@@ -52,8 +55,12 @@ cudaError_t launch_warp(uint64_t n_tasks, int sm_count, Job *jp, const Job *valu
     const uint64_t blocks = std::min<uint64_t>((n_tasks + warps - 1) / warps, cap);
     if (!blocks) return cudaSuccess;
     (void)cudaGetLastError();
-    warp_kernel<<<(unsigned)blocks, threads, 0, s>>>(jp, value ? *value : Job{}, value != nullptr,
-                                                     list, n_ptr, counter, from, n_bad, over, out);
+    // a list's scoring is in device memory, and a captured launch serves them all
+    const Scoring sc = value ? effective(value->sc) : Scoring{};
+    const bool any = !value || (packed16_ok(sc) && !warp_packed(sc));
+    const auto kernel = any ? warp_kernel<true> : warp_kernel<false>;
+    kernel<<<(unsigned)blocks, threads, 0, s>>>(jp, value ? *value : Job{}, value != nullptr, list,
+                                                n_ptr, counter, from, n_bad, over, out);
     return cudaGetLastError();
 }
 

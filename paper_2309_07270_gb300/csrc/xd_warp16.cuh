@@ -333,7 +333,9 @@ static __device__ __noinline__ WarpResult extend_lockstep16(const Ext &e, const 
 // Extends one task with the whole warp on windows of 128 slots (packed if the
 // scoring fits, else 32-bit), 256 (packed scorings only) and 512 slots
 // (32-bit), from the first that is wider than `from` slots.  Returns how many
-// of them the band outgrew, or -1 for all.
+// of them the band outgrew, or -1 for all.  Without ANY the scoring is known not
+// to lie between warp16_ok<2> and packed16_ok.
+template <bool ANY = true>
 __device__ __forceinline__ int extend_warp(const Ext &e, const Scoring &s, int from, int lane,
                                            int32_t &best, int32_t &bi, int32_t &bj)
 {
@@ -344,7 +346,7 @@ __device__ __forceinline__ int extend_warp(const Ext &e, const Scoring &s, int f
         int st;
         if (warp16_ok<2>(sc)) {
             st = extend_warp16<2>(e, sc, lane, best, bi, bj);
-        } else if (packed16_ok(sc)) {
+        } else if (ANY && packed16_ok(sc)) {
             const Ext ec = e;
             const Scoring scc = sc;
             const WarpResult r = extend_lockstep16(ec, scc);
