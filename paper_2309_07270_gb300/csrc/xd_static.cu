@@ -70,7 +70,7 @@ static_warp_kernel(Job J, int64_t per_cta)
             continue;
         }
         int32_t sc, bi, bj;
-        const int st = WINDOWS ? extend_warp(e, J.sc, 0, lane, sc, bi, bj) : -1;
+        const int st = WINDOWS ? extend_warp<true>(e, J.sc, 0, lane, sc, bi, bj) : -1;
         if (lane == 0) {
             if (st < 0) atomicOr(&o[6], kWideLeft << e.side);
             else write_result(J, e, sc, bi, bj);

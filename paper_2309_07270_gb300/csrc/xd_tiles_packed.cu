@@ -89,7 +89,9 @@ static __device__ __noinline__ void run_warp_role(const Job *jp, const uint32_t 
         const Ext e = decode(J, task);
         if (!e.ok) continue;
         int32_t sc, bi, bj;
-        const int st = extend_warp(e, J.sc, whole ? 0 : width, lane, sc, bi, bj);
+        // (with ANY the group loop of the calling kernel is compiled worse: 29x,
+        // x = 15, 22.4 and 23.9 ms)
+        const int st = extend_warp<false>(e, J.sc, whole ? 0 : width, lane, sc, bi, bj);
         if (lane == 0) {
             if (whole && st) {
                 const uint32_t k = atomicAdd(role.grown, 1u);

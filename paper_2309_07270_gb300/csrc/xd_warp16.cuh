@@ -318,7 +318,7 @@ struct OneSrc {
 // extend_warp16<2>'s window for the packed scorings beyond warp16_ok: the group
 // loop on 32 lanes of 4 slots, whose keys take 16 units where a window's take
 // 128 (81 ns a diagonal; the 32-bit window about 200).  Out of line and on
-// copies, so that it costs the callers' registers nothing.
+// copies, for the callers' registers.
 struct WarpResult { int32_t status, best, bi, bj; };
 static __device__ __noinline__ WarpResult extend_lockstep16(const Ext &e, const Scoring &sc)
 {
@@ -333,9 +333,9 @@ static __device__ __noinline__ WarpResult extend_lockstep16(const Ext &e, const 
 // Extends one task with the whole warp on windows of 128 slots (packed if the
 // scoring fits, else 32-bit), 256 (packed scorings only) and 512 slots
 // (32-bit), from the first that is wider than `from` slots.  Returns how many
-// of them the band outgrew, or -1 for all.  Without ANY the scoring is known not
-// to lie between warp16_ok<2> and packed16_ok.
-template <bool ANY = true>
+// of them the band outgrew, or -1 for all.  With ANY every 16-bit scoring takes
+// packed cells in the first, else only those of warp16_ok.
+template <bool ANY>
 __device__ __forceinline__ int extend_warp(const Ext &e, const Scoring &s, int from, int lane,
                                            int32_t &best, int32_t &bi, int32_t &bj)
 {
