@@ -685,7 +685,8 @@ int launch_ticket(xdrop_ctx *c, Ticket *tk, const Job &job, uint32_t maxlen)
     if (job.n_pairs && c->mode != XDROP_MODE_PLAIN && !small) {
         if ((rc = pick_tile(c, tk, job, &c->tile0))) return rc;
     }
-    if (!small) CK(cudaMemsetAsync(c->d_ctrs + C_NBAD, 0, (C_MAXLEN - C_NBAD) * 4, s));
+    const int from = job.n_pairs ? C_NBAD : 0;  // without pairs no launch sequence clears the rest
+    if (!small) CK(cudaMemsetAsync(c->d_ctrs + from, 0, (C_MAXLEN - from) * 4, s));
     if (tk->device_submit && !small) {
         CK(launch_validate(c->d_job, job.n_pairs, c->d_ctrs + C_NBAD, s));
         tk->launches += 1;
