@@ -224,15 +224,19 @@ struct Stage {
 // stale read of it can only be too large, which costs one atomic).  1 Mb
 // genome at 29x, 182.8 M terms: 1.28 ms, issue and the columns' loads
 // (1.6 GB of DRAM); with a warp per whole column and three atomics a term
-// 4.85.  256, 512 and 1,024 threads: the pipeline took 6.5, 5.5 and 5.3 ms
-// (a block lasts as long as its read).
+// 4.85.  A block lasts as long as its read, so long reads take 1,024 threads
+// (that genome's pipeline at 256, 512 and 1,024: 4.9, 4.5, 4.5 ms; 12 reads of
+// 100-200 kb 4.7, 2.6, 1.6), and fills and empties its table, so short ones take
+// 256 (60,000 of 100-150 bases: 3.0, 3.4, 4.8 ms; 40,000 of 300: 2.7, 2.8, 3.7;
+// 5,000 of 1 kb: 0.98, 0.95, 1.02).
 //
 // WRITE = false (first pass, block a = read a): cand_cnt[a] = number of
 // partners (0 and the overflow flag when the table is full); up to kStage
 // partners go to a's staging area, a read with more is listed in big.
 // WRITE = true (second pass, block i = read big[i]): the partners' records
 // at cand_end[a-1] ..., in table order.
-constexpr int kRowThreads = 1024;  // two blocks per SM: the longest reads end the kernel
+constexpr int kRowThreads = 1024, kShortRowThreads = 256;
+constexpr uint64_t kShortMean = 1024, kShortLongest = 32768;  // positions a read, of short reads
 constexpr int kCols = 2;          // columns in flight per half warp
 template <bool WRITE>
 __global__ void __launch_bounds__(kRowThreads)
@@ -467,7 +471,7 @@ struct Front {
     const uint64_t *read_off;
     uint32_t n_reads, k, stride, lo, hi, nb;
     int sm_count;
-    uint64_t n_occ = 0;
+    uint64_t n_occ = 0, longest = 0;  // positions of all reads, of the longest
     uint64_t *occ_off = nullptr;
     const uint64_t *codes = nullptr;
     const uint32_t *occ = nullptr;
@@ -660,7 +664,9 @@ int row_product(Arena &ar, const Front &f, std::vector<Pair> &out_pairs,
         return XDROP_OK;
     }
     XS_CK(cudaMemsetAsync(flags, 0, 8, ar.s));
-    row_kernel<false><<<n_reads, kRowThreads, 0, ar.s>>>(
+    const int threads = f.n_occ <= kShortMean * f.n_reads && f.longest <= kShortLongest
+                            ? kShortRowThreads : kRowThreads;
+    row_kernel<false><<<n_reads, threads, 0, ar.s>>>(
         f.occ_off, row_of, members, f.read_len, f.k, f.stride, f.nb, f.n_occ, cand_cnt, nullptr, flags,
         stage, big, flags + 1, nullptr, nullptr, nullptr, nullptr);
     XS_CK(cudaGetLastError());
@@ -696,7 +702,7 @@ int row_product(Arena &ar, const Front &f, std::vector<Pair> &out_pairs,
         cand_cnt, cand_end, stage, (uint32_t)n_reads, f.nb, rk0, rbest, rshared, ri0);
     XS_CK(cudaGetLastError());
     if (n_big) {
-        row_kernel<true><<<n_big, kRowThreads, 0, ar.s>>>(
+        row_kernel<true><<<n_big, threads, 0, ar.s>>>(
             f.occ_off, row_of, members, f.read_len, f.k, f.stride, f.nb, f.n_occ, nullptr, cand_end,
             nullptr, stage, big, nullptr, rk0, rbest, rshared, ri0);
         XS_CK(cudaGetLastError());
@@ -761,6 +767,8 @@ int find_candidates(cudaStream_t st, cudaMemPool_t pool, int sm_count, size_t bu
         f.nb = xs::id_bits(n_reads);
         f.sm_count = sm_count;
         f.n_occ = stats.occurrences;
+        for (uint32_t r = 0; r < n_reads; ++r)
+            f.longest = std::max(f.longest, occ_off[r + 1] - occ_off[r]);
         rc = ar.cuda(cudaEventRecord(ev[0], st), "cudaEventRecord");
         if (!rc) rc = front(ar, f, occ_off);
         stats.runs = rc ? 0 : (uint64_t)std::max(f.n_runs, 0);
