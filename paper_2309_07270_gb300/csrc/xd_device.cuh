@@ -537,6 +537,7 @@ struct DeviceMem {  // for xd_claim.cuh
 // array pulled from a global counter; overflowing tasks go to a spill list.
 struct BatchSrc {
     static constexpr bool kCanAbort = false;  // teardown may stop the loop
+    static constexpr int kWaitPairs = 1;      // never waits: out of tasks is out for good
     const Job *jp;
     const uint32_t *order;
     uint32_t n_tasks;

@@ -651,9 +651,11 @@ __device__ __forceinline__ void lockstep16_loop(Src &src, const uint32_t *pk, in
         refresh_budget();
         lift_n = min(lift_n, __reduce_min_sync(FULL, lift));
         la_n = min(la_n, lift_n);
-        // a group that still waits for a task asks again after every pair
+        // a group that still waits for a task asks again after kWaitPairs pairs
         const bool waits = __any_sync(FULL, !active && !exhausted);
-        ctr0 = ctr = waits ? 1 : budget >= 1 ? min(la_n, budget) : la_n;
+        const int32_t most = budget >= 1 ? min(la_n, budget) : la_n;
+        if constexpr (Src::kWaitPairs == 1) ctr0 = ctr = waits ? 1 : most;
+        else ctr0 = ctr = waits ? min(most, Src::kWaitPairs) : most;
         if (budget < 1) {
             for (;;) {
                 if (pair(T1{}, T1{}) && handle(true)) break;

@@ -287,6 +287,7 @@ constexpr int64_t kWarp16Words = INT32_MAX - (1 << 22);
 // Task source of lockstep16_loop for one extension and the whole warp.
 struct OneSrc {
     static constexpr bool kCanAbort = false;
+    static constexpr int kWaitPairs = 1;
     const Ext &e;
     const Scoring &s;
     bool fresh = true;
